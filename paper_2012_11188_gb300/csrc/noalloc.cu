@@ -16,7 +16,7 @@ namespace {
 
 // scratch layout, in int32 words:
 //   [0, NOALLOC_MAX_N)            parents
-//   NOALLOC_MAX_N + 0 .. +5       core count and its prefix sums (3 x int64)
+//   NOALLOC_MAX_N + 0 .. +5       prefix sums of the core count (2 of 3 x int64)
 //   NOALLOC_MAX_N + 6             mu (int32)
 //   NOALLOC_MAX_N + 8 .. +9       eps (double)
 //   NOALLOC_MAX_N + 10            status word

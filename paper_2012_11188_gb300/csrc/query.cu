@@ -1,25 +1,42 @@
 // (mu, eps) queries on the index (Algorithms 3-5, Section 6.2, Section 4.3).
 //
-// For a batch of Q queries every phase is one launch over all of them
-// (blockIdx.y = query), so CO/NO reads are shared in L2 across the batch:
+// Phases, each over all (query, core) items of a batch:
 //  1. GetCores (Algorithm 3): the cores are the prefix of CO[mu] whose
-//     threshold is >= eps; its length comes from one binary search (CO[mu] is
+//     threshold is >= eps; its length comes from one search (CO[mu] is
 //     sorted by non-increasing threshold). The prefix marks parent[v] = v.
 //  2. Cluster (Algorithm 5, union-find of Section 6.2): every core u takes the
-//     eps-prefix of NO[u] (binary search) and unions with each core neighbour
-//     of larger id. The union-find is lock-free: find() halves paths, unite()
-//     CASes the larger root under the smaller one, so every root is the
-//     smallest id of its component and labels are canonical.
+//     eps-prefix of NO[u] and unions with each core neighbour of larger id.
+//     The union-find is lock-free: find() halves paths, unite() CASes the
+//     larger root under the smaller one, so every root is the smallest id of
+//     its component and labels are canonical.
 //  3. AssignNonCores (Algorithm 4) with the deterministic rule of Section
 //     7.3.4: a non-core takes the label of the first core in its own
 //     eps-prefix of NO -- the most similar eps-similar core, smallest id among
 //     equal similarities (NO breaks ties by id). Only the non-cores found in
 //     the cores' eps-prefixes are visited (each claimed once by a CAS on its
-//     label), and a non-core's own eps-prefix is shorter than mu-1, so the
-//     query's work follows the eps-edges of its clusters (Theorem 4.3's O(Z))
-//     plus two memsets of n words; every other label stays -1.
+//     label), so the query's work follows the eps-edges of its clusters
+//     (Theorem 4.3's O(Z)) plus two clears of n words; every other label
+//     stays -1.
 //  4. With SCAN_Q_HUBS (Section 4.3): an unclustered vertex whose neighbours
 //     carry two distinct labels becomes -2.
+//
+// What bounds them is latency, not bytes: dependent loads (a search, a
+// neighbour, its parent), the longest row a single warp walks, and the
+// launches. So searches are 32-way (a warp probes 32 places at once: five
+// steps for 4M entries instead of 22); prefixes longer than PIECE entries go
+// to a queue in pieces that any warp may take (R-MAT s22 has rows of 1.5e5
+// entries: a batch of 64 queries spent 2.2 ms in phase 2 on the warps that
+// walked them, and one thread scanning a border's long prefix alone made
+// phase 3 83% of a parameter sweep); and a single query is one cooperative
+// launch whose phases are separated by grid barriers, instead of eight
+// launches, two clears and three small copies.
+// Measured, before and after: one query with hubs on an SBM graph of 10k
+// vertices 85 -> 50 us, (5, 0.3) on R-MAT s22 73 -> 31 us, a batch of 64 on
+// R-MAT s22 1.78 -> 1.41 ms, 594 pairs of a sweep on R-MAT s20 438 -> 72 ms.
+#include <cooperative_groups.h>
+
+#include <mutex>
+
 #include "scan_internal.cuh"
 
 namespace gscan {
@@ -54,15 +71,30 @@ __device__ __forceinline__ bool uf_unite(int32_t* parent, int32_t a, int32_t b) 
   return false;
 }
 
-// number of leading entries of the non-increasing array x[0..len) that are >= eps
-__device__ __forceinline__ int64_t prefix_ge(const double* x, int64_t len, double eps) {
-  int64_t lo = 0, hi = len;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (x[mid] >= eps) lo = mid + 1; else hi = mid;
+// Warp-wide: number of leading entries of the non-increasing array
+// x[0..len) that are >= eps, 32 probes a step.
+__device__ __forceinline__ int64_t prefix_ge(const double* __restrict__ x, int64_t len, double eps) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = len;  // the answer is in [lo, hi]
+  while (hi - lo > 32) {
+    const int64_t step = (hi - lo + 32) / 33;
+    const int64_t at = lo + step * (lane + 1) - 1;
+    const unsigned m = __ballot_sync(0xffffffffu, at < hi && x[at] >= eps);
+    const int c = __popc(m);  // the first c probes hold
+    const int64_t nlo = lo + step * c;
+    if (c < 32) hi = min(hi, nlo + step - 1);  // probe c does not
+    lo = nlo;
   }
-  return lo;
+  const int64_t at = lo + lane;
+  return lo + __popc(__ballot_sync(0xffffffffu, at < hi && x[at] >= eps));
 }
+
+// A piece of a core's eps-prefix, for any warp to take.
+constexpr int PIECE = 1024;
+struct QPiece {
+  int32_t q, u;
+  int32_t begin, end;  // entries of NO[u]; begin = end: none
+};
 
 struct QArgs {
   const int64_t* off;
@@ -77,13 +109,15 @@ struct QArgs {
   int32_t maxdeg;
   const int* mu;       // Q
   const double* eps;   // Q
-  int64_t* ncores;     // Q
-  int64_t* ncp;        // Q+1: exclusive prefix of ncores (flattened (query, core) items)
+  int64_t* ncp;        // Q+1: exclusive prefix of the core counts (flattened (query, core) items)
   int Q;
   int32_t* parent;     // Q * n (-1 = not a core)
   int32_t* labels;     // Q * n, used when lab_ptrs is null
   int32_t* const* lab_ptrs;  // Q destinations (device), or null
   unsigned* status;
+  QPiece* queue;       // null: every warp walks its whole prefixes
+  unsigned long long* queued;  // pieces asked for; more than queue_cap: the queue was full
+  unsigned queue_cap;
 };
 
 __device__ __forceinline__ int32_t* labels_of(const QArgs& a, int q) {
@@ -107,113 +141,244 @@ __device__ __forceinline__ int item_query(const QArgs& a, int64_t i) {
   return lo;
 }
 
-__global__ void k_core_prefix(QArgs a) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    int64_t acc = 0;
-    for (int q = 0; q < a.Q; ++q) { a.ncp[q] = acc; acc += a.ncores[q]; }
-    a.ncp[a.Q] = acc;
+// Warp-wide: number of cores of (mu, eps).
+__device__ __forceinline__ int64_t count_cores(const QArgs& a, int mu, double eps) {
+  if (mu < 2 || mu > a.maxdeg + 1) return 0;
+  const int64_t b = a.co_off[mu - 2], e = a.co_off[mu - 1];
+  return prefix_ge(a.co_thr + b, e - b, eps);
+}
+
+// Core counts of all queries, a warp each, into ncp[0..Q); then their
+// exclusive prefix sums in place (one CTA).
+__global__ void k_get_cores(QArgs a) {
+  const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (q >= a.Q) return;
+  const int64_t c = count_cores(a, a.mu[q], a.eps[q]);
+  if ((threadIdx.x & 31) == 0) a.ncp[q] = c;
+}
+
+constexpr int PREFIX_T = 256;
+__global__ void __launch_bounds__(PREFIX_T) k_core_prefix(QArgs a) {
+  __shared__ int64_t ws[PREFIX_T / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int64_t carry = 0;
+  for (int q0 = 0; q0 < a.Q; q0 += PREFIX_T) {
+    const int q = q0 + threadIdx.x;
+    const int64_t own = q < a.Q ? a.ncp[q] : 0;
+    int64_t inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) ws[wid] = inc;
+    __syncthreads();
+    int64_t before = carry;
+    for (int w = 0; w < PREFIX_T / 32; ++w) {
+      if (w < wid) before += ws[w];
+      carry += ws[w];
+    }
+    if (q < a.Q) a.ncp[q] = before + inc - own;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) a.ncp[a.Q] = carry;
+}
+
+// One query's arguments, or the batch's by item: what a phase needs of item it.
+struct Item {
+  int q;
+  int32_t u;
+  double eps;
+  int32_t* parent;
+  int32_t* lab;
+};
+template <bool ONE>
+__device__ __forceinline__ Item item_at(const QArgs& a, int64_t it, int mu, double eps) {
+  if (ONE) return {0, a.co_id[a.co_off[mu - 2] + it], eps, a.parent, a.labels};
+  const int q = item_query(a, it);
+  return {q, a.co_id[a.co_off[a.mu[q] - 2] + (it - a.ncp[q])], a.eps[q],
+          a.parent + (int64_t)q * a.n, labels_of(a, q)};
+}
+
+template <bool ONE>
+__device__ __forceinline__ void phase_mark(const QArgs& a, int64_t total, int mu, double eps,
+                                           int64_t t0, int64_t nt) {
+  for (int64_t it = t0; it < total; it += nt) {
+    const Item x = item_at<ONE>(a, it, mu, eps);
+    x.parent[x.u] = x.u;
   }
 }
 
-__global__ void k_get_cores(QArgs a, int Q) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= Q) return;
-  const int mu = a.mu[q];
-  int64_t nc = 0;
-  if (mu >= 2 && mu <= a.maxdeg + 1) {
-    const int64_t b = a.co_off[mu - 2], e = a.co_off[mu - 1];
-    nc = prefix_ge(a.co_thr + b, e - b, a.eps[q]);
-  }
-  a.ncores[q] = nc;
-}
-
-__global__ void k_mark_cores(QArgs a) {
-  const int64_t total = a.ncp[a.Q];
-  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < total;
-       it += (int64_t)gridDim.x * blockDim.x) {
-    const int q = item_query(a, it);
-    const int32_t v = a.co_id[a.co_off[a.mu[q] - 2] + (it - a.ncp[q])];
-    a.parent[(int64_t)q * a.n + v] = v;
-  }
-}
-
-// warp per (query, core) item
-__global__ void k_union(QArgs a) {
+// unions of core u with the cores of larger id in entries [b, e) of NO[u]
+__device__ __forceinline__ bool union_range(const QArgs& a, int32_t* parent, int32_t u, int64_t b,
+                                            int64_t e) {
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = a.ncp[a.Q];
+  const int32_t* ids = a.no_id + a.off[u];
+  bool ok = true;
+  for (int64_t j = b + lane; j < e; j += 32) {
+    const int32_t x = ids[j];
+    if (x > u && ld_volatile(parent + x) >= 0) ok &= uf_unite(parent, u, x);
+  }
+  return ok;
+}
+
+// A warp per (query, core) item; what is past the first PIECE entries of a
+// prefix is queued if there is room for all of it, else walked here.
+template <bool ONE>
+__device__ __forceinline__ void phase_union(const QArgs& a, int64_t total, int mu, double eps,
+                                            int64_t w0, int64_t nw) {
+  const int lane = threadIdx.x & 31;
   bool fail = false;
   for (int64_t it = w0; it < total; it += nw) {
-    const int q = item_query(a, it);
-    const double eps = a.eps[q];
-    int32_t* parent = a.parent + (int64_t)q * a.n;
-    const int32_t u = a.co_id[a.co_off[a.mu[q] - 2] + (it - a.ncp[q])];
-    const int64_t rb = a.off[u];
-    const int64_t pu = prefix_ge(a.no_sim + rb, a.deg[u], eps);
-    for (int64_t j = lane; j < pu; j += 32) {
-      const int32_t x = a.no_id[rb + j];
-      if (x > u && ld_volatile(parent + x) >= 0) fail |= !uf_unite(parent, u, x);
+    const Item x = item_at<ONE>(a, it, mu, eps);
+    int64_t pu = prefix_ge(a.no_sim + a.off[x.u], a.deg[x.u], x.eps);
+    if (pu > PIECE && a.queue) {
+      const unsigned np = (unsigned)((pu - 1) / PIECE);  // pieces past the first
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(a.queued, (unsigned long long)np);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      const bool fits = at + np <= a.queue_cap;
+      for (unsigned i = lane; i < np && at + i < a.queue_cap; i += 32) {
+        const int32_t b = (int32_t)(i + 1) * PIECE;
+        const int32_t e = (int32_t)min(pu, (int64_t)b + PIECE);
+        a.queue[at + i] = QPiece{x.q, x.u, b, fits ? e : b};
+      }
+      if (fits) pu = PIECE;
     }
+    fail |= !union_range(a, x.parent, x.u, 0, pu);
+  }
+  if (__any_sync(0xffffffffu, fail) && lane == 0) atomicOr(a.status, (unsigned)DEV_LIMIT);
+}
+
+__device__ __forceinline__ void phase_union_queue(const QArgs& a, int64_t w0, int64_t nw) {
+  const int lane = threadIdx.x & 31;
+  const int64_t cnt = (int64_t)min(*a.queued, (unsigned long long)a.queue_cap);
+  bool fail = false;
+  for (int64_t i = w0; i < cnt; i += nw) {
+    const QPiece p = a.queue[i];
+    fail |= !union_range(a, a.parent + (int64_t)p.q * a.n, p.u, p.begin, p.end);
   }
   if (__any_sync(0xffffffffu, fail) && lane == 0) atomicOr(a.status, (unsigned)DEV_LIMIT);
 }
 
 // labels of the cores: their union-find root (the smallest id of the cluster)
-__global__ void k_core_labels(QArgs a) {
-  const int64_t total = a.ncp[a.Q];
-  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < total;
-       it += (int64_t)gridDim.x * blockDim.x) {
-    const int q = item_query(a, it);
-    const int32_t u = a.co_id[a.co_off[a.mu[q] - 2] + (it - a.ncp[q])];
-    labels_of(a, q)[u] = uf_find(a.parent + (int64_t)q * a.n, u);
+template <bool ONE>
+__device__ __forceinline__ void phase_core_labels(const QArgs& a, int64_t total, int mu, double eps,
+                                                  int64_t t0, int64_t nt) {
+  for (int64_t it = t0; it < total; it += nt) {
+    const Item x = item_at<ONE>(a, it, mu, eps);
+    x.lab[x.u] = uf_find(x.parent, x.u);
   }
 }
 
 constexpr int32_t CLAIMED = -3;
+constexpr int OWN_SCAN = 8;  // entries of its own prefix a border's lane looks at alone
 
-// warp per core: every non-core x in the core's eps-prefix is a border. The
-// first thread to claim x scans x's own eps-prefix of NO for its first core
-// (most similar, smallest id on ties); sigma is symmetric, so that prefix
-// holds at least this core.
-__global__ void k_borders(QArgs a) {
+// Every non-core x in entries [b, e) of NO[u] is a border. The lane that
+// claims x first looks for the first core in x's own eps-prefix of NO (most
+// similar, smallest id on ties; sigma is symmetric, so that prefix holds at
+// least u): OWN_SCAN entries by itself, all loads in flight, the rest of a
+// longer prefix by the whole warp, 128 entries at a time.
+__device__ __forceinline__ void border_range(const QArgs& a, const Item& c, int64_t b, int64_t e) {
+  constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int64_t total = a.ncp[a.Q];
-  for (int64_t it = w0; it < total; it += nw) {
-    const int q = item_query(a, it);
-    const double eps = a.eps[q];
-    int32_t* parent = a.parent + (int64_t)q * a.n;
-    int32_t* lab = labels_of(a, q);
-    const int32_t u = a.co_id[a.co_off[a.mu[q] - 2] + (it - a.ncp[q])];
-    const int64_t rb = a.off[u];
-    const int64_t pu = prefix_ge(a.no_sim + rb, a.deg[u], eps);
-    for (int64_t j = lane; j < pu; j += 32) {
-      const int32_t x = a.no_id[rb + j];
-      if (ld_volatile(parent + x) >= 0) continue;
-      if (atomicCAS(lab + x, -1, CLAIMED) != -1) continue;
-      int32_t l = -1;
-      const int64_t xb = a.off[x], xe = xb + a.deg[x];
-      for (int64_t t = xb; t < xe; ++t) {
-        if (a.no_sim[t] < eps) break;
-        const int32_t y = a.no_id[t];
-        if (ld_volatile(parent + y) >= 0) { l = uf_find(parent, y); break; }
+  int32_t* parent = c.parent;
+  const int32_t* ids = a.no_id + a.off[c.u];
+  for (int64_t j0 = b; j0 < e; j0 += 32) {
+    const int64_t j = j0 + lane;
+    const int32_t x = j < e ? ids[j] : -1;
+    bool mine = x >= 0 && ld_volatile(parent + x) < 0 &&
+                atomicCAS(c.lab + x, -1, CLAIMED) == -1;
+    int64_t xb = 0;
+    int32_t xd = 0;
+    if (mine) {
+      xb = a.off[x];
+      xd = a.deg[x];
+      double sv[OWN_SCAN];
+      int32_t y[OWN_SCAN], py[OWN_SCAN];
+#pragma unroll
+      for (int t = 0; t < OWN_SCAN; ++t) {
+        sv[t] = t < xd ? a.no_sim[xb + t] : -1.0;
+        y[t] = t < xd ? a.no_id[xb + t] : x;
       }
-      lab[x] = l;
+#pragma unroll
+      for (int t = 0; t < OWN_SCAN; ++t) py[t] = ld_volatile(parent + y[t]);
+      bool over = false;
+#pragma unroll
+      for (int t = 0; t < OWN_SCAN; ++t) {
+        if (over || !mine) continue;
+        if (!(sv[t] >= c.eps)) {  // end of the prefix
+          over = true;
+        } else if (py[t] >= 0) {
+          c.lab[x] = uf_find(parent, y[t]);
+          mine = false;
+        }
+      }
+      if (mine && (over || xd <= OWN_SCAN)) {  // no core (cannot be with symmetric similarities)
+        c.lab[x] = -1;
+        mine = false;
+      }
+    }
+    unsigned todo = __ballot_sync(FULL, mine);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int64_t rb = __shfl_sync(FULL, xb, src);
+      const int32_t rd = __shfl_sync(FULL, xd, src);
+      const int32_t xs = __shfl_sync(FULL, x, src);
+      int32_t first = -1;
+      bool end = false;
+      for (int32_t t0 = OWN_SCAN; t0 < rd && first < 0 && !end; t0 += 128) {
+        double sv[4];
+        int32_t y[4], py[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int32_t t = t0 + 32 * k + lane;
+          sv[k] = t < rd ? a.no_sim[rb + t] : -1.0;
+          y[k] = t < rd ? a.no_id[rb + t] : xs;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) py[k] = ld_volatile(parent + y[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const bool in = sv[k] >= c.eps;
+          const unsigned m = __ballot_sync(FULL, in && py[k] >= 0);
+          if (first < 0 && m) first = __shfl_sync(FULL, y[k], __ffs(m) - 1);
+          end |= !__all_sync(FULL, in);
+        }
+      }
+      if (lane == 0) c.lab[xs] = first >= 0 ? uf_find(parent, first) : -1;
     }
   }
 }
 
+template <bool ONE>
+__device__ __forceinline__ void phase_borders(const QArgs& a, int64_t total, int mu, double eps,
+                                              int64_t w0, int64_t nw) {
+  // the pieces queued for the unions are the ones of this phase too, unless
+  // the queue was full: then every warp walks its whole prefixes
+  const int64_t asked = a.queue ? (int64_t)*a.queued : 0;
+  const bool queued = asked <= (int64_t)a.queue_cap;
+  for (int64_t it = w0; it < total; it += nw) {
+    const Item x = item_at<ONE>(a, it, mu, eps);
+    int64_t pu = prefix_ge(a.no_sim + a.off[x.u], a.deg[x.u], x.eps);
+    if (a.queue && queued) pu = min(pu, (int64_t)PIECE);
+    border_range(a, x, 0, pu);
+  }
+  if (a.queue && queued)
+    for (int64_t i = w0; i < asked; i += nw) {
+      const QPiece p = a.queue[i];
+      const Item x{p.q, p.u, ONE ? eps : a.eps[p.q], a.parent + (int64_t)p.q * a.n,
+                   ONE ? a.labels : labels_of(a, p.q)};
+      border_range(a, x, p.begin, p.end);
+    }
+}
+
 // warp per unclustered vertex
-__global__ void k_hubs(QArgs a) {
-  const int q = blockIdx.y;
-  int32_t* lab = labels_of(a, q);
+__device__ __forceinline__ void phase_hubs(const QArgs& a, int32_t* lab, int64_t w0, int64_t nw) {
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = w0; v < a.n; v += nw) {
-    if (lab[v] != -1) continue;
+    if (ld_volatile(lab + v) != -1) continue;
     const int64_t rb = a.off[v], re = rb + a.deg[v];
     int32_t first = -1;
     bool hub = false;
@@ -232,17 +397,151 @@ __global__ void k_hubs(QArgs a) {
   }
 }
 
+__device__ __forceinline__ int64_t grid_thread() {
+  return (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+}
+__device__ __forceinline__ int64_t grid_threads() { return (int64_t)gridDim.x * blockDim.x; }
+
+// The batch's phases, one launch each.
+__global__ void k_mark_cores(QArgs a) {
+  phase_mark<false>(a, a.ncp[a.Q], 0, 0.0, grid_thread(), grid_threads());
+}
+__global__ void k_union(QArgs a) {
+  phase_union<false>(a, a.ncp[a.Q], 0, 0.0, grid_thread() >> 5, grid_threads() >> 5);
+}
+__global__ void k_union_queue(QArgs a) {
+  phase_union_queue(a, grid_thread() >> 5, grid_threads() >> 5);
+}
+__global__ void k_labels(QArgs a) {  // borders do not read core labels, only parents
+  const int64_t total = a.ncp[a.Q];
+  phase_core_labels<false>(a, total, 0, 0.0, grid_thread(), grid_threads());
+  phase_borders<false>(a, total, 0, 0.0, grid_thread() >> 5, grid_threads() >> 5);
+}
+__global__ void k_hubs(QArgs a) {
+  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  phase_hubs(a, labels_of(a, blockIdx.y), w0, ((int64_t)gridDim.x * blockDim.x) >> 5);
+}
+
+// -1 in p[0..n), as 16-byte stores between the first and last 16-byte boundary
+__device__ __forceinline__ void fill_minus1(int32_t* p, int64_t n, int64_t t0, int64_t nt) {
+  const int64_t head = min(n, (int64_t)(((16 - ((uintptr_t)p & 15)) & 15) / 4));
+  const int64_t vec = (n - head) / 4;
+  int4* p4 = reinterpret_cast<int4*>(p + head);
+  for (int64_t i = t0; i < vec; i += nt) p4[i] = make_int4(-1, -1, -1, -1);
+  for (int64_t i = t0; i < head; i += nt) p[i] = -1;
+  for (int64_t i = head + 4 * vec + t0; i < n; i += nt) p[i] = -1;
+}
+
+// One query as one cooperative launch: the same phases between grid barriers,
+// (mu, eps) as arguments, the status in a word that the host reads directly.
+// Every CTA searches the core count for itself (it is one cached path).
+constexpr int ONE_T = 256;
+__global__ void __launch_bounds__(ONE_T)
+k_query_one(QArgs a, int mu, double eps, int hubs) {
+  cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  __shared__ int64_t s_nc;
+  const int64_t t0 = grid_thread(), nt = grid_threads();
+  if (t0 == 0) *a.queued = 0;
+  fill_minus1(a.parent, a.n, t0, nt);
+  fill_minus1(a.labels, a.n, t0, nt);
+  if (threadIdx.x < 32) {
+    const int64_t c = count_cores(a, mu, eps);
+    if (threadIdx.x == 0) s_nc = c;
+  }
+  __syncthreads();
+  const int64_t nc = s_nc;
+  if (nc == 0 && !hubs) return;  // the same in every CTA
+  grid.sync();
+  phase_mark<true>(a, nc, mu, eps, t0, nt);
+  grid.sync();
+  phase_union<true>(a, nc, mu, eps, t0 >> 5, nt >> 5);
+  grid.sync();
+  if (a.queue && *a.queued) {  // the same in every CTA: nothing adds to it any more
+    phase_union_queue(a, t0 >> 5, nt >> 5);
+    grid.sync();
+  }
+  phase_core_labels<true>(a, nc, mu, eps, t0, nt);
+  phase_borders<true>(a, nc, mu, eps, t0 >> 5, nt >> 5);
+  if (!hubs) return;
+  grid.sync();
+  phase_hubs(a, a.labels, t0 >> 5, nt >> 5);
+}
+
+// Words of pinned host memory that kernels write their status to: one page
+// for the process, words handed out and taken back under a lock.
+constexpr int STATUS_WORDS = 256;
+std::mutex g_word_mu;
+unsigned* g_words = nullptr;
+bool g_word_used[STATUS_WORDS];
+
+struct HostWord {
+  unsigned* p = nullptr;
+  HostWord() {
+    std::lock_guard<std::mutex> lk(g_word_mu);
+    if (!g_words &&
+        cudaHostAlloc((void**)&g_words, STATUS_WORDS * sizeof(unsigned),
+                      cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaGetLastError();
+      g_words = nullptr;
+      return;
+    }
+    for (int i = 0; i < STATUS_WORDS; ++i)
+      if (!g_word_used[i]) {
+        g_word_used[i] = true;
+        p = g_words + i;
+        *p = 0;
+        return;
+      }
+  }
+  ~HostWord() {
+    if (!p) return;
+    std::lock_guard<std::mutex> lk(g_word_mu);
+    g_word_used[p - g_words] = false;
+  }
+};
+
+// Resident CTAs of k_query_one per multiprocessor (0: no cooperative launch).
+int query_one_per_sm() {
+  static std::atomic<int> cached[64];  // 1 + the value, zero until looked up
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int c = cached[dev].load(std::memory_order_relaxed);
+  if (c == 0) {
+    int coop = 0, per = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_query_one, ONE_T, 0) != cudaSuccess) {
+      cudaGetLastError();
+      per = 0;
+    }
+    c = 1 + (per < 4 ? per : 4);
+    cached[dev].store(c, std::memory_order_relaxed);
+  }
+  return c - 1;
+}
+
+unsigned queue_capacity(const IndexData& ix, int Q) {
+  // pieces past the first of a row: none when no row is longer than one
+  if (ix.maxdeg <= PIECE) return 0;
+  const int64_t all = (int64_t)Q * (ix.arcs / PIECE + 1);
+  return (unsigned)std::min<int64_t>(all, QUERY_QUEUE_MAX);
+}
+
 }  // namespace
 
 // Launch sequence of a batch of Q queries; every pointer is device memory.
 int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* eps, int64_t* nc,
                        int32_t* parent, int32_t* labels, int32_t* const* lab_ptrs, int flags,
-                       cudaStream_t s, unsigned* status_dev) {
+                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes) {
   const int64_t n = ix.n;
   GS_CUDA(cudaMemsetAsync(parent, 0xff, sizeof(int32_t) * (size_t)Q * n, s));
-  // nc holds 2Q+1 words: Q core counts, then their Q+1 prefix sums
+  // queue: a 16-byte head with the count, then the pieces
+  const unsigned cap = queue && queue_bytes > 16 && ix.maxdeg > PIECE
+      ? (unsigned)std::min<size_t>((queue_bytes - 16) / sizeof(QPiece), QUERY_QUEUE_MAX) : 0;
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
-          n, ix.maxdeg, mu, eps, nc, nc + Q, Q, parent, labels, lab_ptrs, status_dev};
+          n, ix.maxdeg, mu, eps, nc, Q, parent, labels, lab_ptrs, status_dev,
+          cap ? reinterpret_cast<QPiece*>((char*)queue + 16) : nullptr,
+          reinterpret_cast<unsigned long long*>(queue), cap};
+  if (cap) GS_CUDA(cudaMemsetAsync(queue, 0, 16, s));
   const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, sm_count() * 8 / std::min(Q, 8) + 1));
   const unsigned gw = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, sm_count() * 16 / std::min(Q, 16) + 1));
   if (lab_ptrs) {
@@ -251,23 +550,63 @@ int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* 
   } else {
     GS_CUDA(cudaMemsetAsync(labels, 0xff, sizeof(int32_t) * (size_t)Q * n, s));
   }
-  k_get_cores<<<(Q + 127) / 128, 128, 0, s>>>(a, Q);
+  k_get_cores<<<(Q + 3) / 4, 128, 0, s>>>(a);
   GS_LAUNCH();
-  k_core_prefix<<<1, 32, 0, s>>>(a);
+  k_core_prefix<<<1, PREFIX_T, 0, s>>>(a);
   GS_LAUNCH();
   // the (query, core) items of the whole batch share one grid
   k_mark_cores<<<sm_count() * 8, 256, 0, s>>>(a);
   GS_LAUNCH();
   k_union<<<sm_count() * 16, 256, 0, s>>>(a);
   GS_LAUNCH();
-  k_core_labels<<<sm_count() * 8, 256, 0, s>>>(a);
-  GS_LAUNCH();
-  k_borders<<<sm_count() * 16, 256, 0, s>>>(a);
+  if (cap) {
+    k_union_queue<<<sm_count() * 16, 256, 0, s>>>(a);
+    GS_LAUNCH();
+  }
+  k_labels<<<sm_count() * 16, 256, 0, s>>>(a);
   GS_LAUNCH();
   if (flags & SCAN_Q_HUBS) {
     k_hubs<<<dim3(gw, Q), 256, 0, s>>>(a);
     GS_LAUNCH();
   }
+  return SCAN_OK;
+}
+
+size_t query_queue_bytes(const IndexData& ix, int Q) {
+  const unsigned cap = queue_capacity(ix, Q);
+  return cap ? 16 + (size_t)cap * sizeof(QPiece) : 0;
+}
+
+int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int32_t* host_labels,
+                  int flags, Pool& pool, cudaStream_t s, bool* done) {
+  *done = false;
+  const int64_t n = ix.n;
+  const int per_sm = query_one_per_sm();
+  HostWord status;
+  if (per_sm == 0 || !status.p) return SCAN_OK;
+  const size_t qb = query_queue_bytes(ix, 1);
+  const size_t head = ((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255;
+  char* scratch = pool.get<char>(head + (qb ? qb : 16));
+  if (!scratch) return SCAN_ENOMEM;
+  *done = true;
+  int32_t* parent = reinterpret_cast<int32_t*>(scratch);
+  unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + head);
+  QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
+          n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status.p,
+          qb ? reinterpret_cast<QPiece*>(scratch + head + 16) : nullptr, queued,
+          queue_capacity(ix, 1)};
+  // a warp per core at most, and no more CTAs than are resident at once
+  const int64_t want = std::max<int64_t>(1, (n + ONE_T / 32 - 1) / (ONE_T / 32));
+  const unsigned g = (unsigned)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
+  int hubs = flags & SCAN_Q_HUBS;
+  void* args[] = {&a, &mu, &eps, &hubs};
+  GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_query_one, dim3(g), dim3(ONE_T), args, 0, s));
+  GS_LAUNCH();
+  if (host_labels)
+    GS_CUDA(cudaMemcpyAsync(host_labels, labels, (size_t)n * sizeof(int32_t),
+                            cudaMemcpyDeviceToHost, s));
+  GS_CUDA(cudaStreamSynchronize(s));
+  if (*(volatile unsigned*)status.p & DEV_LIMIT) return SCAN_ETIMEOUT;
   return SCAN_OK;
 }
 
@@ -277,17 +616,21 @@ int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* ep
   const int64_t n = ix.n;
   int* mu = pool.get<int>(Q);
   double* eps = pool.get<double>(Q);
-  int64_t* nc = pool.get<int64_t>(2 * (size_t)Q + 1);
+  int64_t* nc = pool.get<int64_t>((size_t)Q + 1);
   int32_t* parent = pool.get<int32_t>((size_t)Q * (size_t)(n > 0 ? n : 1));
-  if (!mu || !eps || !nc || !parent) return SCAN_ENOMEM;
+  const size_t qb = query_queue_bytes(ix, Q);
+  char* queue = qb ? pool.get<char>(qb) : nullptr;
+  if (!mu || !eps || !nc || !parent || (qb && !queue)) return SCAN_ENOMEM;
   GS_CUDA(cudaMemcpyAsync(mu, mu_host, sizeof(int) * Q, cudaMemcpyHostToDevice, s));
   GS_CUDA(cudaMemcpyAsync(eps, eps_host, sizeof(double) * Q, cudaMemcpyHostToDevice, s));
   if (n == 0) return SCAN_OK;
-  GS_TRY(launch_query_batch(ix, Q, mu, eps, nc, parent, labels_dev, nullptr, flags, s, status_dev));
+  GS_TRY(launch_query_batch(ix, Q, mu, eps, nc, parent, labels_dev, nullptr, flags, s, status_dev,
+                            queue, qb));
   pool.put(mu);
   pool.put(eps);
   pool.put(nc);
   pool.put(parent);
+  if (queue) pool.put(queue);
   return SCAN_OK;
 }
 
@@ -299,7 +642,7 @@ int run_queries_prealloc(const IndexData& ix, int Q, const int* mu_dev, const do
                          cudaStream_t s, unsigned* status_dev) {
   if (Q <= 0 || ix.n == 0) return SCAN_OK;
   return launch_query_batch(ix, Q, mu_dev, eps_dev, nc_dev, parent, labels_dev, nullptr, flags, s,
-                            status_dev);
+                            status_dev, nullptr, 0);
 }
 
 }  // namespace gscan

@@ -728,6 +728,11 @@ int query_impl(scan_index* index, int q, const int* mu, const double* eps, int32
   const bool dev_out = is_device_ptr(labels);
   int32_t* lab = dev_out ? labels : pool.get<int32_t>((size_t)q * ix.n);
   if (!lab) return SCAN_ENOMEM;
+  if (q == 1) {
+    bool done = false;
+    GS_TRY(run_query_one(ix, mu[0], eps[0], lab, dev_out ? nullptr : labels, flags, pool, s, &done));
+    if (done) return SCAN_OK;
+  }
   unsigned* st_dev = pool.get<unsigned>(1);
   if (!st_dev) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(st_dev, 0, sizeof(unsigned), s));

@@ -194,15 +194,26 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
 int run_queries(const IndexData& ix, int q, const int* mu, const double* eps, int32_t* labels_dev,
                 int flags, Pool& pool, cudaStream_t s, unsigned* status_dev);
 
+// One query into device labels (copied to host_labels too unless null) as one
+// cooperative launch; synchronises s. *done = false: such a launch is not to
+// be had, nothing was enqueued.
+int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels_dev,
+                  int32_t* host_labels, int flags, Pool& pool, cudaStream_t s, bool* done);
+
 // Launch sequence of a batch of Q queries on device arrays: mu/eps hold Q
-// entries, nc 2Q+1 (core counts and their prefix sums), parent Q*n; labels either Q*n contiguous (lab_ptrs null) or Q
-// device destinations listed in lab_ptrs.
+// entries, nc Q+1 (prefix sums of the core counts), parent Q*n; labels either
+// Q*n contiguous (lab_ptrs null) or Q device destinations listed in lab_ptrs;
+// queue: query_queue_bytes(ix, Q) of scratch for the pieces of long rows
+// (null: none, a warp walks a long row alone).
+constexpr unsigned QUERY_QUEUE_MAX = 1u << 17;  // pieces
+constexpr size_t QUERY_QUEUE_MAX_BYTES = 16 + (size_t)QUERY_QUEUE_MAX * 16;
+size_t query_queue_bytes(const IndexData& ix, int Q);
 int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* eps, int64_t* nc,
                        int32_t* parent, int32_t* labels, int32_t* const* lab_ptrs, int flags,
-                       cudaStream_t s, unsigned* status_dev);
+                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes);
 
 // run_queries with caller-supplied device scratch: mu_dev/eps_dev hold Q
-// entries, nc_dev 2Q+1, parent Q*n; nothing is allocated.
+// entries, nc_dev Q+1, parent Q*n; nothing is allocated.
 int run_queries_prealloc(const IndexData& ix, int Q, const int* mu_dev, const double* eps_dev,
                          int64_t* nc_dev, int32_t* parent, int32_t* labels_dev, int flags,
                          cudaStream_t s, unsigned* status_dev);

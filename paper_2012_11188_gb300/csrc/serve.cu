@@ -89,7 +89,7 @@ void finish(scan_server* s, Request* r, int status) {
 }
 
 // Scratch of the query worker, kept across batches and grown on demand:
-// parents (cap x n), mu/eps/core counts and the table of label destinations,
+// parents (cap x n), mu/eps/core counts, the queue of row pieces and the table of label destinations,
 // and two sets of what a batch in flight owns until its copies are done:
 // staging rows for host destinations, a device status word, its pinned host
 // copy and the event that marks its kernels done.
@@ -101,6 +101,7 @@ struct QueryScratch {
   int* mu = nullptr;
   double* eps = nullptr;
   int64_t* nc = nullptr;
+  char* queue = nullptr;
   unsigned* status[2] = {nullptr, nullptr};
   unsigned* status_host = nullptr;  // pinned, 2 words
   int32_t* staging[2] = {nullptr, nullptr};
@@ -135,7 +136,8 @@ struct QueryScratch {
     ptrs = get<int32_t*>(c, s);
     mu = get<int>(c, s);
     eps = get<double>(c, s);
-    nc = get<int64_t>(2 * (size_t)c + 1, s);
+    nc = get<int64_t>((size_t)c + 1, s);
+    queue = get<char>(gscan::QUERY_QUEUE_MAX_BYTES, s);
     status[0] = get<unsigned>(1, s);
     status[1] = get<unsigned>(1, s);
     if (cudaHostAlloc((void**)&status_host, 2 * sizeof(unsigned), cudaHostAllocDefault) !=
@@ -144,7 +146,7 @@ struct QueryScratch {
     bool ev_ok = true;
     for (auto& e : kern_done)
       ev_ok &= cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
-    if (!parent || !ptrs || !mu || !eps || !nc || !status[0] || !status[1] || !status_host ||
+    if (!parent || !ptrs || !mu || !eps || !nc || !queue || !status[0] || !status[1] || !status_host ||
         !ev_ok) {
       release(s);
       return SCAN_ENOMEM;
@@ -219,7 +221,8 @@ int launch_batch(scan_server* s, QueryScratch& qs, const std::vector<Request*>& 
   GS_CUDA(cudaMemcpyAsync(qs.ptrs, dst.data(), sizeof(int32_t*) * Q, cudaMemcpyHostToDevice, s->qs));
   GS_CUDA(cudaMemsetAsync(qs.status[set], 0, sizeof(unsigned), s->qs));
   GS_TRY(gscan::launch_query_batch(d, Q, qs.mu, qs.eps, qs.nc, qs.parent, nullptr, qs.ptrs,
-                                   batch[0]->flags, s->qs, qs.status[set]));
+                                   batch[0]->flags, s->qs, qs.status[set], qs.queue,
+                                   gscan::QUERY_QUEUE_MAX_BYTES));
   GS_CUDA(cudaEventRecord(qs.kern_done[set], s->qs));
   GS_CUDA(cudaStreamWaitEvent(s->cs, qs.kern_done[set], 0));
   for (size_t r = 0; r < host_rows.size(); ++r)
