@@ -65,6 +65,20 @@ def test_unaligned_device_labels(graph, shift):
     assert (got[:shift] == 77).all() and (got[shift + g.n:] == 77).all()
 
 
+@pytest.mark.parametrize("count", [1, 7, 8, 31, 32, 33, 70])
+def test_sweep_lengths(graph, count):
+    """One clustering at a time, a full batch, a batch and a remainder; rows
+    longer than one arc piece of the modularity pass (512)."""
+    g, ox = graph
+    pairs = [(m, e) for m in MUS for e in EPSS]
+    pairs = [pairs[(11 * i) % len(pairs)] for i in range(count)]
+    with gs.ScanIndex.build(g) as ix:
+        got = ix.sweep([m for m, _ in pairs], [e for _, e in pairs])
+    want = [oracle.modularity(g, ox.query(m, e)) for m, e in pairs]
+    # whole numbers below 2^53 on both sides up to the last two divisions
+    assert np.abs(got - np.array(want)).max() <= 1e-12
+
+
 def test_threads_and_streams(graph):
     import torch
     g, ox = graph
