@@ -11,7 +11,8 @@
 // Segments are classed by length: <= 32 (one warp, one element per lane,
 // bitonic network across lanes), <= 256, 512, 1024, 2048 and 4096 (one CTA
 // of 32 to 512 threads: 8-element register sorts, then merge-path levels in
-// shared memory), longer (split into buckets by sample sort, below; past
+// shared memory), longer (a few of up to 16384 elements the same way by one
+// CTA each, else split into buckets by sample sort, below; past
 // three levels of splitting, 8192-element tiles sorted by one CTA the same
 // way, then merge-path passes over global memory that double the run length,
 // ping-ponging between the data and a scratch buffer).
@@ -69,22 +70,30 @@ __global__ void k_classify_count(Segs S, int64_t nseg, int64_t total,
   if (threadIdx.x < NCLASS + 2) c[threadIdx.x] = 0;
   __syncthreads();
   bool bad = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseg;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = S.b[i], e = S.e[i];
-    if (b < 0 || e < b || e > total) {
-      bad = true;
-      continue;
+  // lane k keeps the warp's count of class k, one ballot per class and step,
+  // and adds it once at the end (with a shared 64-bit atomic per segment, all
+  // to a few addresses, the nine calls of an R-MAT s20 build took 151 us, now 60)
+  const int lane = threadIdx.x & 31;
+  unsigned mine = 0;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < nseg;
+       i0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = i0 + lane;
+    const int64_t b = i < nseg ? S.b[i] : 0, e = i < nseg ? S.e[i] : 0;
+    const bool ok = b >= 0 && e >= b && e <= total;
+    bad |= !ok;
+    const int64_t len = ok ? e - b : 0;
+    const int cl = len <= 1 ? -1 : seg_class(len);
+#pragma unroll
+    for (int k = 0; k < NCLASS; ++k) {
+      const unsigned m = __ballot_sync(0xffffffffu, cl == k);
+      if (lane == k) mine += __popc(m);
     }
-    const int64_t len = e - b;
-    if (len <= 1) continue;
-    const int cl = seg_class(len);
-    atomicAdd(&c[cl], 1ull);
     if (cl == LONGC) {
       atomicAdd(&c[NCLASS], (unsigned long long)((len + TILE - 1) / TILE));
       atomicMax(&c[NCLASS + 1], (unsigned long long)len);
     }
   }
+  if (lane < NCLASS && mine) atomicAdd(&c[lane], (unsigned long long)mine);
   __syncthreads();
   if (threadIdx.x < NCLASS + 1 && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], c[threadIdx.x]);
   if (threadIdx.x == NCLASS + 1 && c[threadIdx.x]) atomicMax(&counts[threadIdx.x], c[threadIdx.x]);
@@ -243,6 +252,100 @@ __device__ __forceinline__ void merge_out(const uint64_t* ks, const int32_t* vs,
     va = take_a ? vn : va;
     kb = take_a ? kb : kn;
     vb = take_a ? vb : vn;
+  }
+}
+
+// The same outputs into registers, for tiles that fill shared memory with one
+// buffer: the caller writes them back once every thread has read its inputs.
+template <int R, int RI>
+__device__ __forceinline__ void merge_regs(const uint64_t* ks, const int32_t* vs, int a0, int la,
+                                           int b0, int lb, int d, uint64_t (&K)[RI],
+                                           int32_t (&V)[RI]) {
+  int ia = smem_merge_path_p<R>(ks, vs, a0, la, b0, lb, d);
+  int ib = d - ia;
+#pragma unroll
+  for (int q = 0; q < RI; ++q) {
+    const int pa = pslot<R>(a0 + (ia < la ? ia : 0)), pb = pslot<R>(b0 + (ib < lb ? ib : 0));
+    const bool take_a = ib >= lb || (ia < la && !before_at(ks, vs, pb, pa));
+    const int p = take_a ? pa : pb;
+    K[q] = ks[p];
+    V[q] = vs[p];
+    ia += take_a ? 1 : 0;
+    ib += take_a ? 0 : 1;
+  }
+}
+
+// Whole segments of up to HUGE elements by one CTA, in one shared buffer.
+// Taken when no segment of a level is longer and a multiprocessor each is
+// enough for those beyond 4096: the sample-sort split of such a few segments
+// is some 25 launches of two levels, each waiting for the one before (the
+// core order of an SBM graph of 10k vertices has a dozen segments of 1e4: 71 us
+// here, and 16 launches fewer; the build 1.00 -> 0.72 ms with the wider grids
+// of the other kernels).
+constexpr int HUGE_T = 1024, HUGE_RI = 16;
+constexpr int HUGE_LEN = HUGE_T * HUGE_RI;
+constexpr size_t HUGE_SMEM = (size_t)(HUGE_LEN + HUGE_LEN / HUGE_RI) * 12;
+
+__global__ void __launch_bounds__(HUGE_T, 1)
+k_sort_huge(const uint64_t* ik, const int32_t* iv, uint64_t* key, int32_t* val, Segs S,
+            const int64_t* __restrict__ list, int64_t cnt) {
+  extern __shared__ uint64_t hsm[];
+  uint64_t* ks = hsm;
+  int32_t* vs = (int32_t*)(hsm + HUGE_LEN + HUGE_LEN / HUGE_RI);
+  const int t = threadIdx.x;
+  for (int64_t u = blockIdx.x; u < cnt; u += gridDim.x) {
+    const int64_t sg = list[u];
+    const int64_t b = S.b[sg];
+    const int len = (int)(S.e[sg] - b);
+    const int lr = (len + HUGE_RI - 1) / HUGE_RI * HUGE_RI;
+    for (int i = t; i < lr; i += HUGE_T) {
+      const int p = pslot<HUGE_RI>(i);
+      ks[p] = i < len ? ik[b + i] : 0;
+      vs[p] = i < len ? iv[b + i] : SENT_V;
+    }
+    __syncthreads();
+    const int o = HUGE_RI * t;
+    uint64_t K[HUGE_RI];
+    int32_t V[HUGE_RI];
+    if (o < lr) {
+#pragma unroll
+      for (int r = 0; r < HUGE_RI; ++r) {
+        const int p = pslot<HUGE_RI>(o + r);
+        K[r] = ks[p];
+        V[r] = vs[p];
+      }
+      sort_regs(K, V);
+#pragma unroll
+      for (int r = 0; r < HUGE_RI; ++r) {
+        const int p = pslot<HUGE_RI>(o + r);
+        ks[p] = K[r];
+        vs[p] = V[r];
+      }
+    }
+    __syncthreads();
+    for (int w = HUGE_RI; w < lr; w <<= 1) {
+      if (o < lr) {
+        const int a0 = (o / (2 * w)) * (2 * w);
+        const int la = min(w, lr - a0), lb = max(0, min(w, lr - a0 - w));
+        merge_regs<HUGE_RI, HUGE_RI>(ks, vs, a0, la, a0 + w, lb, o - a0, K, V);
+      }
+      __syncthreads();
+      if (o < lr) {
+#pragma unroll
+        for (int r = 0; r < HUGE_RI; ++r) {
+          const int p = pslot<HUGE_RI>(o + r);
+          ks[p] = K[r];
+          vs[p] = V[r];
+        }
+      }
+      __syncthreads();
+    }
+    for (int i = t; i < len; i += HUGE_T) {
+      const int p = pslot<HUGE_RI>(i);
+      key[b + i] = ks[p];
+      val[b + i] = vs[p];
+    }
+    __syncthreads();
   }
 }
 
@@ -1019,7 +1122,15 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
   const int64_t max_long = (int64_t)hc[NCLASS + 1];
   // long segments are split into buckets, sorted one level down; below
   // BKT_DEPTH levels they take the tiles and merge passes
-  const bool bucketed = nlong && depth < BKT_DEPTH;
+  const bool whole = nlong && max_long <= HUGE_LEN && nlong <= sm_count();
+  const bool bucketed = nlong && !whole && depth < BKT_DEPTH;
+  if (whole) {
+    GS_CUDA(cudaFuncSetAttribute(k_sort_huge, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)HUGE_SMEM));
+    k_sort_huge<<<(unsigned)nlong, HUGE_T, HUGE_SMEM, s>>>(ik, iv, key, val, S,
+                                                           list + base[LONGC], nlong);
+    GS_LAUNCH();
+  }
   if (bucketed)
     GS_TRY(bucket_level(key, val, alt_k, alt_v, S, total, list + base[LONGC], nlong, in_alt, pool,
                         s, depth));
@@ -1069,7 +1180,7 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
         ik, iv, key, val, S, list + base[5], counts + 5, nullptr, 0, nullptr, nullptr);
     GS_LAUNCH();
   }
-  if (nlong && !bucketed) {
+  if (nlong && !bucketed && !whole) {
     const int64_t* llist = list + base[LONGC];
     if (in_alt) {  // the tiles and merge passes work in (key, val)
       k_copy_segments<<<grid_of(nlong, 1), 256, 0, s>>>(alt_k, alt_v, key, val, S, llist, nlong);

@@ -606,7 +606,9 @@ k_triangles(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
 // Warp kernel for rows of at most warp_deg positions with out-lists of at
 // most SMALL_OD entries: each warp owns one
 // vertex at a time, with its own table of out(v) (no CTA barrier). Warps take
-// 32 vertices per atomic fetch.
+// `batch` <= 32 vertices per atomic fetch: 32 on a large graph, fewer where 32
+// would leave warps of the grid without any (10k vertices are 313 batches of
+// 32 for 4864 warps: 125 us on an SBM graph of 10k vertices, now 22).
 template <typename IT, bool WT, int R>
 __global__ void __launch_bounds__(SW_WARPS * 32, 8)
 k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
@@ -614,7 +616,7 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
             const int32_t* __restrict__ oadj, const int32_t* __restrict__ opos,
             const uint64_t* __restrict__ okey,
             const int64_t* __restrict__ odp, int64_t n, unsigned long long* __restrict__ work,
-            int lsh_T, int warp_deg, int long_list, uint32_t* __restrict__ tcnt,
+            int batch, int lsh_T, int warp_deg, int long_list, uint32_t* __restrict__ tcnt,
             uint32_t* __restrict__ tc16,
             int32_t* __restrict__ twin_rel, unsigned* status, const double* __restrict__ ow,
             double* __restrict__ tsum) {
@@ -632,15 +634,16 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
   unsigned bad = 0;
   for (;;) {
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(work, 32ull);
+    if (lane == 0) base = atomicAdd(work, (unsigned long long)batch);
     base = __shfl_sync(FULL, base, 0);
     if ((int64_t)base >= n) break;
-    // the lanes read the 32 vertices' degrees at once; the warp then visits
+    // the lanes read the batch's degrees at once; the warp then visits
     // only its vertices with in-neighbours (most have none: their
     // neighbours all rank above them)
     const int64_t vl = (int64_t)base + lane;
-    const int32_t dl = vl < n ? deg[vl] : 0;
-    const int32_t ol = vl < n ? odeg[vl] : 0;
+    const bool inb = lane < batch && vl < n;
+    const int32_t dl = inb ? deg[vl] : 0;
+    const int32_t ol = inb ? odeg[vl] : 0;
     const bool mine = dl > 0 && warp_vertex(dl, ol, warp_deg) && dl - ol > 0;
     const int64_t offl = mine ? off[vl] : 0, odpl = mine ? odp[vl] : 0;
     unsigned todo = __ballot_sync(FULL, mine);
@@ -694,9 +697,12 @@ __device__ __forceinline__ double sim_of(int kind, int64_t c, int64_t du, int64_
 // Every oriented edge a->b writes sigma to both of its CSR arcs. Threads run
 // over the oriented edges in order (odp = exclusive prefix of the
 // out-degrees, so edge k is the (k - odp[a])-th out-arc of the vertex a with
-// odp[a] <= k < odp[a+1]); a CTA's EXPAND_T * EXPAND_ITEMS edges span the
+// odp[a] <= k < odp[a+1]); a CTA's EXPAND_T * per edges span the
 // vertices between two binary searches, and each edge finds its own vertex
 // by a search inside that bracket.
+// per: up to EXPAND_ITEMS edges per thread, fewer when the graph would not
+// give every multiprocessor a CTA (44 us for the 69k edges of an SBM graph of
+// 10k vertices on 34 CTAs, now 14 on 271).
 constexpr int EXPAND_T = 256;
 constexpr int EXPAND_ITEMS = 8;
 
@@ -747,11 +753,11 @@ k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ 
          const int64_t* __restrict__ odp, const int32_t* __restrict__ oadj,
          const int32_t* __restrict__ opos, const uint32_t* __restrict__ tcnt,
          const uint32_t* __restrict__ tc16,
-         const int32_t* __restrict__ twin_rel, int64_t n, int lsh_T,
+         const int32_t* __restrict__ twin_rel, int64_t n, int per, int lsh_T,
          double* __restrict__ sim_csr, unsigned* status) {
   __shared__ int64_t s_bracket[2];
   const int64_t m = odp[n];
-  constexpr int64_t CH = (int64_t)EXPAND_T * EXPAND_ITEMS;
+  const int64_t CH = (int64_t)EXPAND_T * per;
   unsigned bad = 0;
   for (int64_t k0 = (int64_t)blockIdx.x * CH; k0 < m; k0 += (int64_t)gridDim.x * CH) {
     const int64_t k1 = min(m, k0 + CH);
@@ -899,10 +905,10 @@ k_expand_w(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
            const double* __restrict__ ow, const double* __restrict__ tsum,
            const int32_t* __restrict__ twin_rel, const double* __restrict__ wcsr,
            const double* __restrict__ norm, const int32_t* __restrict__ deg, int64_t n,
-           int lsh_T, double* __restrict__ sim_csr, unsigned* status) {
+           int per, int lsh_T, double* __restrict__ sim_csr, unsigned* status) {
   __shared__ int64_t s_bracket[2];
   const int64_t m = odp[n];
-  constexpr int64_t CH = (int64_t)EXPAND_T * EXPAND_ITEMS;
+  const int64_t CH = (int64_t)EXPAND_T * per;
   unsigned bad = 0;
   for (int64_t k0 = (int64_t)blockIdx.x * CH; k0 < m; k0 += (int64_t)gridDim.x * CH) {
     const int64_t k1 = min(m, k0 + CH);
@@ -992,10 +998,11 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
   if (small_per_sm < 1) small_per_sm = 1;
   // the warp kernel takes its vertices from work[2] (set to the range's
   // first vertex) up to small_end
+  const int64_t small_warps = (int64_t)sms * small_per_sm * SW_WARPS;
+  const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(32, n / (2 * small_warps)));
   k_tri_small<IT, WT, R><<<sms * small_per_sm, SW_WARPS * 32, 0, s>>>(
-      off, adj, deg, odeg, oadj, opos, okey, odp, small_end, work + 2, lsh_T, cfg.warp_deg, cfg.long_list,
-      tcnt,
-      tc16, twin, status, ow, tsum);
+      off, adj, deg, odeg, oadj, opos, okey, odp, small_end, work + 2, batch, lsh_T, cfg.warp_deg,
+      cfg.long_list, tcnt, tc16, twin, status, ow, tsum);
   GS_LAUNCH();
   // items with out-lists too long for the shared table, and items deferred
   // by the CTA kernel (normally none: the launch then ends at once)
@@ -1102,11 +1109,13 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
   }
   GS_CUDA(cudaEventRecord(e0, s));
   // the rank and weight passes walk 32 rows per warp (EXPAND_T / 32 warps a
-  // CTA); the similarity pass takes EXPAND_T * EXPAND_ITEMS edges per CTA
+  // CTA); the similarity pass takes EXPAND_T * per edges per CTA
   const unsigned wgrid =
       (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + EXPAND_T - 1) / EXPAND_T,
                                                        sm_count() * 32));
-  const int64_t ch = (int64_t)EXPAND_T * EXPAND_ITEMS;
+  const int per = (int)std::max<int64_t>(
+      1, std::min<int64_t>(EXPAND_ITEMS, edges / ((int64_t)sm_count() * 4 * EXPAND_T)));
+  const int64_t ch = (int64_t)EXPAND_T * per;
   const unsigned egrid =
       (unsigned)std::max<int64_t>(1, std::min<int64_t>((edges + ch - 1) / ch, sm_count() * 32));
   if (n > 0 && m > 0) {
@@ -1150,10 +1159,10 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
                                                                                       norm);
       GS_LAUNCH();
       k_expand_w<<<egrid, EXPAND_T, 0, s>>>(off, adj, odp, oadj, opos, ow, tsum, twin, wcsr, norm,
-                                            deg, n, lsh_T, sim_csr, status);
+                                            deg, n, per, lsh_T, sim_csr, status);
     } else {
       k_expand<<<egrid, EXPAND_T, 0, s>>>(kind, off, deg, odp, oadj, opos, tcnt, tc16, twin, n,
-                                          lsh_T, sim_csr, status);
+                                          per, lsh_T, sim_csr, status);
     }
     GS_LAUNCH();
   }
