@@ -603,6 +603,438 @@ k_triangles(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
   if (bad) atomicOr(status, (unsigned)DEV_BADGRAPH);
 }
 
+// ---- Hubs: the vertices of highest degree, at most HUB_MAX of them, whole
+// degree classes, numbered 0, 1, ... from the highest rank (d, id) down. When
+// the middle vertex v is a hub, so is every third vertex w > v, and out(v) is
+// kept as a bitmap over the hub numbers below v's instead of a hash table:
+//  - a stream element is a 16-bit number (half the bytes of an id), read two
+//    to a 32-bit word (rounds in flight, s24 ms of the CTA kernels: 1 round of
+//    64 elements 71.7, 2 63.9, 3 63.3, 4 62.6);
+//  - its test is one shared load. The stream is in descending numbers, so
+//    the words of neighbouring lanes are neighbours: few bank conflicts, where
+//    the two hash slots of every lane are random banks (some 7 wavefronts);
+//  - the two elements of a word share one word of 16-bit (u,w) counters, so
+//    two hits are one global atomic;
+//  - the table takes 8 bytes per 32 hub numbers and 4 per out-arc, under 25 KB
+//    on R-MAT s24 instead of 57: six 256-thread CTAs per multiprocessor, and
+//    so twice as many middle vertices walk the same in-neighbours' lists and
+//    counters at a time, which are read from L2 instead of HBM.
+// The position of w in out(v) follows from its word's prefix count.
+// R-MAT s24: CTA kernels 88.5 -> 62.6 ms (46 here, bound by instruction issue,
+// 17 in the hash-table kernel for the middle vertices below the hubs), DRAM
+// traffic 465 -> 260 GB; s20: 2.3 -> 1.4 ms.
+constexpr int HUB_MAX = 65535;          // numbers 0..65534; 0xffff: not a hub
+constexpr int HUB_MIN_DEG = 64;         // no hubs below this degree
+constexpr int HUB_T = 256;
+constexpr int HUB_WARPS = HUB_T / 32;
+constexpr int HUB_WORDS = 2048;         // 32 numbers each
+constexpr int HUB_PAIRS = 4;            // 64-element rounds in flight of a long suffix
+
+struct HubInfo {
+  int32_t min_deg;     // hubs: the vertices of at least this degree
+  int32_t count;
+  int64_t items;       // leading items of the degree order whose vertex is a hub
+};
+
+// vertices per degree, bins of descending degree, degrees >= HUB_MIN_DEG
+__global__ void k_hub_hist(const int32_t* __restrict__ deg, int64_t n, int32_t maxdeg,
+                           unsigned long long* __restrict__ hist) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t d = deg[v];
+    if (d < HUB_MIN_DEG) continue;
+    // lanes of one degree add once (a regular graph has one bin)
+    const unsigned peers = __match_any_sync(__activemask(), d);
+    if ((threadIdx.x & 31) == __ffs(peers) - 1)
+      atomicAdd(&hist[maxdeg - d], (unsigned long long)__popc(peers));
+  }
+}
+
+// pre: exclusive prefix of the bins 0 .. nbins - 1. The lowest degree down to
+// which all classes together hold at most HUB_MAX vertices.
+__global__ void k_hub_cut(const int64_t* __restrict__ pre, int64_t nbins, int32_t maxdeg,
+                          HubInfo* info) {
+  if (blockIdx.x || threadIdx.x) return;
+  int64_t lo = 0, hi = nbins;  // bins taken
+  while (lo < hi) {
+    const int64_t mid = (lo + hi + 1) >> 1;
+    if (pre[mid] <= HUB_MAX) lo = mid; else hi = mid - 1;
+  }
+  info->min_deg = (int32_t)(maxdeg - lo + 1);
+  info->count = (int32_t)pre[lo];
+  info->items = 0;
+}
+
+__global__ void k_hub_place(const int32_t* __restrict__ deg, int64_t n, int32_t maxdeg,
+                            const HubInfo* __restrict__ info, const int64_t* __restrict__ pre,
+                            unsigned long long* __restrict__ fill, int32_t* __restrict__ list) {
+  const int32_t cut = info->min_deg;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x)
+    if (deg[v] >= cut) {
+      const int64_t b = maxdeg - deg[v];
+      list[pre[b] + (int64_t)atomicAdd(&fill[b], 1ull)] = (int32_t)v;
+    }
+}
+
+// number of a hub = hubs of higher degree + those of its degree with a larger
+// id, counted by a warp (the squares of the class sizes add up to at most
+// HUB_MAX^2 tests)
+__global__ void k_hub_number(const int32_t* __restrict__ deg, int32_t maxdeg,
+                             const HubInfo* __restrict__ info, const int64_t* __restrict__ pre,
+                             const int32_t* __restrict__ list, uint16_t* __restrict__ num) {
+  const int lane = threadIdx.x & 31;
+  const int w0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+  const int cnt = info->count;
+  for (int i = w0; i < cnt; i += nw) {
+    const int32_t v = list[i];
+    const int64_t b = maxdeg - deg[v];
+    const int c0 = (int)pre[b], c1 = (int)pre[b + 1];
+    int larger = 0;
+    for (int j = c0 + lane; j < c1; j += 32) larger += list[j] > v ? 1 : 0;
+    larger = __reduce_add_sync(0xffffffffu, larger);
+    if (lane == 0) num[v] = (uint16_t)(c0 + larger);
+  }
+}
+
+// items of the hubs in the degree order of the CTA kernel (start: vertices
+// with items before each bin, item_off: items before each vertex); the
+// hash-table kernel begins after them
+__global__ void k_hub_items(HubInfo* info, int32_t maxdeg, const int64_t* __restrict__ start,
+                            const int64_t* __restrict__ item_off,
+                            unsigned long long* __restrict__ work) {
+  if (blockIdx.x || threadIdx.x) return;
+  const int64_t bins = (int64_t)maxdeg - info->min_deg + 1;
+  info->items = item_off[start[bins]];
+  work[0] = (unsigned long long)info->items;
+}
+
+// The bitmap of out(v): words[i].x holds the numbers 32 i .. 32 i + 31,
+// words[i].y is 4 times the out-arcs of numbers below 32 (i + 1), plus vbase,
+// the shared-space address of the counters (0 in weighted mode): the address
+// of a number's counter is one multiply-add away.
+struct HubTable {
+  const uint2* words;
+  uint32_t vbase;
+  uint32_t own;   // v's number: every number of out(v) is smaller, its bit is clear
+};
+
+// Number (x >> SHIFT) mod 2^16 among out(v)'s: its word shifted down to its
+// bit (bit 0: it is there), and the address of its counter if it is.
+template <int SHIFT>
+__device__ __forceinline__ uint32_t hub_probe(const HubTable& t, uint32_t x, uint32_t& addr) {
+  const uint2 w = *reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(t.words) +
+                                                  ((x >> (SHIFT + 2)) & 0x3ff8u));
+  const uint32_t above = __funnelshift_r(w.x, 0u, x >> SHIFT);  // by the number mod 32
+  addr = w.y - 4u * (uint32_t)__popc(above);
+  return above;
+}
+
+// Predicated reductions: the compiler would branch around them.
+__device__ __forceinline__ void red_shared_if(uint32_t bit, uint32_t addr) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %0, 0;\n"
+               "@p red.shared.add.u32 [%1], 1;\n}" ::"r"(bit), "r"(addr) : "memory");
+}
+__device__ __forceinline__ void red_global_nz(uint32_t* p, uint32_t add) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %0, 0;\n"
+               "@p red.global.add.u32 [%1], %0;\n}" ::"r"(add), "l"(p) : "memory");
+}
+
+// process_slice for a hub v. o16[j] is the number of out-arc j's head (0xffff
+// for other vertices, which rank below every hub): every out-list descends.
+template <typename IT, bool WT, int R>
+__device__ __forceinline__ void hub_slice(
+    int64_t p0, int64_t p_end, int64_t rb, int32_t od, int64_t ob, int long_list,
+    const int32_t* __restrict__ opos, const int32_t* __restrict__ deg,
+    const int64_t* __restrict__ off, const int32_t* __restrict__ odeg,
+    const int32_t* __restrict__ oadj, const uint16_t* __restrict__ o16, int lsh_T,
+    const HubTable& tab, const SliceSmem& sm, uint32_t* __restrict__ tcnt,
+    uint32_t* __restrict__ tc16, int32_t* __restrict__ twin_rel, unsigned& bad,
+    const Weights& wt) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t p = p0 + lane;
+  int32_t u = -1;
+  bool is_in = false;
+  if (p < p_end) {
+    u = oadj[rb + p];
+    is_in = !(lsh_T >= 0 && deg[u] > lsh_T);  // (v's degree is above the threshold as well)
+  }
+  const unsigned m = __ballot_sync(FULL, is_in);
+  if (!m) return;
+  const int k = __popc(m);
+  if (is_in) {
+    const int r = __popc(m & ((1u << lane) - 1u));
+    sm.u[r] = u;
+    sm.p[r] = opos[rb + p];
+  }
+  __syncwarp();
+  int32_t cp = 0, clen = 0;  // suffix length after v
+  IT cub = 0, jv = 0;        // suffix start; position of v in out(u)
+  bool found = false;
+  if (lane < k) {
+    const int32_t cu = sm.u[lane];
+    cp = sm.p[lane];
+    const IT ub = (IT)off[cu];
+    const int32_t len = odeg[cu];
+    int lo = 0, hi = len;  // first entry <= own
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (o16[ub + mid] > tab.own) lo = mid + 1; else hi = mid;
+    }
+    found = lo < len && o16[ub + lo] == tab.own;
+    if (found) {
+      jv = ub + (IT)lo;
+      cub = jv + 1;
+      clen = len - lo - 1;
+    } else {
+      bad = 1;  // v lists u but u does not list v
+    }
+  }
+  if (od == 0) {
+    if (found) twin_rel[jv] = cp;
+    __syncwarp();
+    return;
+  }
+  sm.acc[lane] = 0;
+  int wcnt = 0;
+  __syncwarp();
+
+  // 1. long suffixes, one at a time, two elements per lane and round
+  const uint32_t none = tab.own | (tab.own << 16);
+  // the out-arc of the counter at addr (ascending numbers, descending ranks)
+  const IT qlast = (IT)(ob + od - 1);
+  auto out_arc = [&](uint32_t addr) { return qlast - (IT)((addr - tab.vbase) >> 2); };
+  const uint32_t* o32 = reinterpret_cast<const uint32_t*>(o16);
+  unsigned lm = __ballot_sync(FULL, lane < k && clen >= long_list);
+  while (lm) {
+    const int i = __ffs(lm) - 1;
+    lm &= lm - 1;
+    const IT s0 = __shfl_sync(FULL, cub, i);
+    const int32_t slen = __shfl_sync(FULL, clen, i);
+    const IT jvi = WT ? __shfl_sync(FULL, jv, i) : (IT)0;
+    // word t of the suffix holds elements 2 t - odd and 2 t + 1 - odd of it
+    const int odd = (int)(s0 & 1);
+    const uint32_t* px = o32 + (s0 >> 1) + lane;
+    uint32_t* pc = (sizeof(IT) == 4 ? tc16 : tcnt) + (s0 >> 1) * (sizeof(IT) == 4 ? 1 : 2) +
+                   lane * (sizeof(IT) == 4 ? 1 : 2);
+    unsigned hits = 0;  // of this lane: even elements low half, odd elements high half
+    int left = slen + odd - 2 * lane;  // elements from this lane's word on
+    for (int rest = slen + odd; rest > 0; rest -= 64 * HUB_PAIRS) {
+      uint32_t xs[HUB_PAIRS];
+#pragma unroll
+      for (int rr = 0; rr < HUB_PAIRS; ++rr) {
+        xs[rr] = none;
+        if (left > 64 * rr) xs[rr] = px[32 * rr];
+        if (left == 64 * rr + 1) xs[rr] = (xs[rr] & 0xffffu) | (tab.own << 16);
+      }
+      if (odd && left == slen + odd) xs[0] = (xs[0] & 0xffff0000u) | tab.own;  // the first word
+#pragma unroll
+      for (int rr = 0; rr < HUB_PAIRS; ++rr) {
+        if (rr > 0 && rest <= 64 * rr) break;
+        uint32_t a0, a1;
+        const uint32_t b0 = hub_probe<0>(tab, xs[rr], a0), b1 = hub_probe<16>(tab, xs[rr], a1);
+        if (WT) {
+          const IT j = 2 * (IT)(px - o32 + 32 * rr);
+          wt_push<IT>(b0 & 1u, j, out_arc(a0), jvi, wcnt, wt);
+          wt_push<IT>(b1 & 1u, j + 1, out_arc(a1), jvi, wcnt, wt);
+        } else {
+          red_shared_if(b0 & 1u, a0);
+          red_shared_if(b1 & 1u, a1);
+          const uint32_t add = (b0 & 1u) | ((b1 & 1u) << 16);
+          if (sizeof(IT) == 4) {
+            red_global_nz(pc + 32 * rr, add);
+          } else {
+            red_global_nz(pc + 64 * rr, b0 & 1u);
+            red_global_nz(pc + 64 * rr + 1, b1 & 1u);
+          }
+          hits += add;
+        }
+      }
+      px += 32 * HUB_PAIRS;
+      pc += 32 * HUB_PAIRS * (sizeof(IT) == 4 ? 1 : 2);
+      left -= 64 * HUB_PAIRS;
+    }
+    if (!WT) hits = (hits & 0xffffu) + (hits >> 16);
+    if (!WT) {
+      hits = __reduce_add_sync(FULL, hits);
+      if (lane == 0) sm.acc[i] += hits;
+    }
+  }
+
+  // 2. short non-empty suffixes, concatenated (as in process_slice)
+  const bool is_short = lane < k && clen > 0 && clen < long_list;
+  const unsigned shm = __ballot_sync(FULL, is_short);
+  if (shm) {
+    const int k2 = __popc(shm);
+    if (is_short) sm.u[__popc(shm & ((1u << lane) - 1u))] = lane;
+    __syncwarp();
+    const int orig = lane < k2 ? sm.u[lane] : 0;
+    const IT sub = __shfl_sync(FULL, cub, orig);
+    const int32_t sl = __shfl_sync(FULL, clen, orig);
+    const int32_t slen = lane < k2 ? sl : 0;
+    int32_t incl = slen;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    const int32_t cstart = incl - slen;
+    const int32_t W = __shfl_sync(FULL, incl, 31);
+    for (int32_t rbase = 0; rbase < W; rbase += 32 * R) {
+      uint32_t xs[R];
+      IT js[R];
+      int owns[R];
+#pragma unroll
+      for (int rr = 0; rr < R; ++rr) {
+        const int32_t r0 = rbase + 32 * rr;
+        const int32_t t = r0 + lane;
+        const bool starts_here = lane < k2 && cstart >= r0 && cstart < r0 + 32;
+        const unsigned smask = __reduce_or_sync(FULL, starts_here ? (1u << (cstart - r0)) : 0u);
+        const int before = __popc(__ballot_sync(FULL, lane < k2 && cstart < r0));
+        const int owner = before + __popc(smask & ((2u << lane) - 1u)) - 1;
+        const int own = owner < 0 ? 0 : owner;
+        const IT ub_o = __shfl_sync(FULL, sub, own);
+        const int32_t st_o = __shfl_sync(FULL, cstart, own);
+        owns[rr] = __shfl_sync(FULL, orig, own);
+        js[rr] = t < W ? ub_o + (IT)(t - st_o) : (IT)-1;
+        xs[rr] = t < W ? o16[js[rr]] : tab.own;
+      }
+#pragma unroll
+      for (int rr = 0; rr < R; ++rr) {
+        const int own = owns[rr];
+        uint32_t addr;
+        const uint32_t bit = hub_probe<0>(tab, xs[rr], addr) & 1u;
+        if (WT) {
+          const IT jo = __shfl_sync(FULL, jv, own);
+          wt_push<IT>(bit, js[rr], out_arc(addr), jo, wcnt, wt);
+        } else {
+          const IT j = js[rr];
+          red_shared_if(bit, addr);
+          if (sizeof(IT) == 4) red_global_nz(tc16 + (j >> 1), bit << ((j & 1) << 4));
+          else red_global_nz(tcnt + j, bit);
+          const unsigned hm = __ballot_sync(FULL, bit);
+          if (hm) {
+            const unsigned peers = __match_any_sync(FULL, own);
+            if ((hm & peers) && lane == __ffs(peers) - 1) sm.acc[own] += __popc(hm & peers);
+          }
+        }
+      }
+    }
+  }
+  __syncwarp();
+  if (WT) wt_drain<IT>(wcnt, wt);
+  if (found) {
+    if (!WT) {
+      const uint32_t acc = sm.acc[lane];
+      if (acc) atomicAdd(&tcnt[jv], acc);
+    }
+    twin_rel[jv] = cp;
+  }
+  __syncwarp();
+}
+
+template <typename IT, bool WT, int R>
+__global__ void __launch_bounds__(HUB_T, 6)
+k_tri_hub(const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
+          const int32_t* __restrict__ odeg, const int32_t* __restrict__ oadj,
+          const int32_t* __restrict__ opos, const uint16_t* __restrict__ o16,
+          const uint16_t* __restrict__ num, const HubInfo* __restrict__ info, int64_t n,
+          const int64_t* __restrict__ item_off, const int32_t* __restrict__ order,
+          unsigned long long* __restrict__ work, int lsh_T, int item_chunk, int long_list,
+          uint32_t* __restrict__ tcnt, uint32_t* __restrict__ tc16,
+          int32_t* __restrict__ twin_rel, unsigned* status, const double* __restrict__ ow,
+          double* __restrict__ tsum) {
+  extern __shared__ uint4 smem4[];  // words[HUB_WORDS], then vcnt (unweighted)
+  __shared__ long long s_item;
+  __shared__ int s_next;
+  __shared__ int s_sum[HUB_WARPS];
+  __shared__ int32_t s_u[HUB_WARPS][32];
+  __shared__ int32_t s_p[HUB_WARPS][32];
+  __shared__ uint32_t s_acc[HUB_WARPS][32];
+  __shared__ IT s_hb[WT ? HUB_WARPS : 1][WT ? 3 * WT_BUF : 1];
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t total = info->items;
+  uint2* words = reinterpret_cast<uint2*>(smem4);
+  uint32_t* vcnt = reinterpret_cast<uint32_t*>(words + HUB_WORDS);
+  const uint32_t vbase = WT ? 0u : (uint32_t)__cvta_generic_to_shared(vcnt);
+  const Weights wt{ow, tsum, WT ? (void*)s_hb[wid] : nullptr};
+  const SliceSmem sm{s_u[wid], s_p[wid], s_acc[wid]};
+  unsigned bad = 0;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      s_item = (long long)atomicAdd(work, 1ull);
+      s_next = 0;
+    }
+    __syncthreads();
+    const int64_t item = s_item;
+    if (item >= total) break;
+    const int64_t idx = find_item_vertex(item_off, n, item);
+    const int32_t v = order[idx];
+    const int64_t chunk = item - item_off[idx];
+    const int32_t dv = deg[v], od = odeg[v];
+    const int64_t ob = off[v];
+    if (od > SMEM_OD_MAX) {  // left to the binary-search kernel
+      __syncthreads();
+      continue;
+    }
+    const uint32_t own = num[v];
+    const int nwords = (int)(own >> 5) + 1;
+    for (int i = threadIdx.x; i < nwords; i += HUB_T) words[i] = make_uint2(0u, 0u);
+    if (!WT)
+      for (int i = threadIdx.x; i < od; i += HUB_T) vcnt[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < od; i += HUB_T) {
+      const uint32_t x = o16[ob + i];
+      if (x < own) atomicOr(&words[x >> 5].x, 1u << (x & 31));
+      else bad = 1;  // (an out-arc to a vertex of lower rank: not a symmetric graph)
+    }
+    __syncthreads();
+    // prefix counts: a thread takes consecutive words
+    const int per = (nwords + HUB_T - 1) / HUB_T;
+    const int i0 = min(nwords, (int)threadIdx.x * per), i1 = min(nwords, i0 + per);
+    int mine = 0;
+    for (int i = i0; i < i1; ++i) mine += __popc(words[i].x);
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_sum[wid] = inc;
+    __syncthreads();
+    int before = inc - mine;
+    for (int w = 0; w < wid; ++w) before += s_sum[w];
+    for (int i = i0; i < i1; ++i) {
+      before += __popc(words[i].x);
+      words[i].y = vbase + 4u * (uint32_t)before;
+    }
+    __syncthreads();
+    const HubTable tab{words, vbase, own};
+    const int64_t p_begin = chunk * item_chunk;
+    const int64_t p_end = min((int64_t)(dv - od), p_begin + item_chunk);
+    for (;;) {
+      int slice = 0;
+      if (lane == 0) slice = atomicAdd(&s_next, 32);
+      slice = __shfl_sync(FULL, slice, 0);
+      const int64_t pos0 = p_begin + slice;
+      if (pos0 >= p_end) break;
+      hub_slice<IT, WT, R>(pos0, p_end, ob + od, od, ob, long_list, opos, deg, off, odeg, oadj, o16,
+                           dv > lsh_T ? lsh_T : -1, tab, sm, tcnt, tc16, twin_rel, bad, wt);
+    }
+    __syncthreads();
+    if (!WT)
+      for (int i = threadIdx.x; i < od; i += HUB_T) {
+        const uint32_t c = vcnt[i];
+        if (c) atomicAdd(&tcnt[ob + od - 1 - i], c);  // ascending numbers, descending ranks
+      }
+    __syncthreads();
+  }
+  if (bad) atomicOr(status, (unsigned)DEV_BADGRAPH);
+}
+
 // Warp kernel for rows of at most warp_deg positions with out-lists of at
 // most SMALL_OD entries: each warp owns one
 // vertex at a time, with its own table of out(v) (no CTA barrier). Warps take
@@ -811,10 +1243,13 @@ k_rank_keys(const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
 __global__ void __launch_bounds__(EXPAND_T)
 k_rank_scatter(const int64_t* __restrict__ off, const int64_t* __restrict__ odp, int64_t n,
                const uint64_t* __restrict__ okey, const int32_t* __restrict__ oval,
-               int32_t* __restrict__ oadj, int32_t* __restrict__ opos) {
+               int32_t* __restrict__ oadj, int32_t* __restrict__ opos,
+               const uint16_t* __restrict__ num, uint16_t* __restrict__ o16) {
   walk_out_arcs(off, odp, n, [&](int64_t k, int64_t, int64_t j) {
-    oadj[j] = (int32_t)(uint32_t)~okey[k];
+    const int32_t x = (int32_t)(uint32_t)~okey[k];
+    oadj[j] = x;
     opos[j] = oval[k];
+    if (o16) o16[j] = num[x];  // hub numbers
   });
 }
 
@@ -964,6 +1399,12 @@ __global__ void k_fill_i32(int32_t* p, int64_t n, int32_t v) {
 // accumulates weighted-cosine numerators (ow, tsum) instead of counts; R is
 // the number of 32-element rounds of loads in flight for the concatenated
 // short suffixes (a tuning parameter: 4 or 8).
+struct Hubs {
+  const uint16_t* num = nullptr;  // hub number of every vertex; null: no hub kernel
+  const uint16_t* o16 = nullptr;  // and of every out-arc's head
+  const HubInfo* info = nullptr;
+};
+
 template <typename IT, bool WT, int R>
 int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, const int32_t* odeg,
                     const int32_t* oadj, const int32_t* opos, const uint64_t* okey,
@@ -972,7 +1413,8 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
                     unsigned long long* work, int lsh_T, int32_t max_od, int64_t* deferred,
                     unsigned long long* n_deferred, uint32_t* tcnt, uint32_t* tc16, int32_t* twin,
                     unsigned* status, const double* ow, double* tsum, const CountCfg& cfg,
-                    cudaStream_t s, cudaEvent_t k0, cudaEvent_t k1, int64_t small_end) {
+                    cudaStream_t s, cudaEvent_t k0, cudaEvent_t k1, int64_t small_end,
+                    const Hubs& hubs) {
   int od_cap = 16;
   while (od_cap < max_od && od_cap < SMEM_OD_MAX) od_cap <<= 1;
   // the table (12 bytes per slot, 2 * od_cap slots) and the counters (4 bytes)
@@ -987,6 +1429,21 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
                                                         TRI_THREADS, smem));
   if (per_sm < 1) per_sm = 1;
   if (k0) GS_CUDA(cudaEventRecord(k0, s));
+  if (hubs.num) {
+    // two elements per lane and round: a suffix fills a round of half the
+    // hash-table kernel's bound (a quarter and the whole of it were slower)
+    const size_t hsmem = HUB_WORDS * sizeof(uint2) + (WT ? 0 : 4 * (size_t)od_cap);
+    GS_CUDA(cudaFuncSetAttribute(k_tri_hub<IT, WT, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(HUB_WORDS * sizeof(uint2) + 4 * SMEM_OD_MAX)));
+    int hub_per_sm = 1;
+    GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hub_per_sm, k_tri_hub<IT, WT, R>, HUB_T,
+                                                          hsmem));
+    if (hub_per_sm < 1) hub_per_sm = 1;
+    k_tri_hub<IT, WT, R><<<sms * hub_per_sm, HUB_T, hsmem, s>>>(
+        off, deg, odeg, oadj, opos, hubs.o16, hubs.num, hubs.info, n, item_off, order, work + 4,
+        lsh_T, cfg.cta_chunk, std::max(1, cfg.long_list / 2), tcnt, tc16, twin, status, ow, tsum);
+    GS_LAUNCH();
+  }
   k_triangles<false, IT, WT, R><<<sms * per_sm, TRI_THREADS, smem, s>>>(
       off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off, order, work, lsh_T, cfg.cta_chunk,
       cfg.long_list, od_cap, deferred, n_deferred, false, tcnt, tc16, twin, status, ow, tsum);
@@ -1025,14 +1482,15 @@ int launch_counting_cfg(const int64_t* off, const int32_t* adj, const int32_t* d
                         int64_t* deferred, unsigned long long* n_deferred, uint32_t* tcnt,
                         uint32_t* tc16, int32_t* twin, unsigned* status, const double* ow,
                         double* tsum, const CountCfg& cfg, cudaStream_t s, cudaEvent_t k0,
-                        cudaEvent_t k1, int64_t small_end) {
+                        cudaEvent_t k1, int64_t small_end,
+                        const Hubs& hubs) {
   if (!WT && cfg.rounds == 8)
     return launch_counting<IT, WT, 8>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off, order,
                                       work, lsh_T, max_od, deferred, n_deferred, tcnt, tc16, twin,
-                                      status, ow, tsum, cfg, s, k0, k1, small_end);
+                                      status, ow, tsum, cfg, s, k0, k1, small_end, hubs);
   return launch_counting<IT, WT, 4>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off, order,
                                     work, lsh_T, max_od, deferred, n_deferred, tcnt, tc16, twin,
-                                    status, ow, tsum, cfg, s, k0, k1, small_end);
+                                    status, ow, tsum, cfg, s, k0, k1, small_end, hubs);
 }
 
 int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* adj,
@@ -1067,7 +1525,9 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
   int64_t* item_off = pool.get<int64_t>(n + 1);
   unsigned long long* hist = pool.get<unsigned long long>(2 * nbins);  // counts | fill cursors
   int64_t* start = pool.get<int64_t>(nbins + 1);
-  unsigned long long* work = pool.get<unsigned long long>(4);  // 3 counters + deferred count
+  // counters of the hash-table, binary-search and warp kernels, deferred
+  // items, counter of the hub kernel
+  unsigned long long* work = pool.get<unsigned long long>(5);
   // items: at most one per vertex plus one per cta_chunk arcs
   int64_t* deferred = pool.get<int64_t>(n + m / cfg.cta_chunk + 1);
   if (!tcnt || (narrow && !tc16) || !twin || !items || !items_sorted || !order || !item_off ||
@@ -1076,7 +1536,7 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(tcnt, 0, m * sizeof(uint32_t), s));
   if (narrow) GS_CUDA(cudaMemsetAsync(tc16, 0, (m / 2 + 1) * sizeof(uint32_t), s));
-  GS_CUDA(cudaMemsetAsync(work, 0, 4 * sizeof(unsigned long long), s));
+  GS_CUDA(cudaMemsetAsync(work, 0, 5 * sizeof(unsigned long long), s));
   if (v0 > 0) {  // the warp kernel's first vertex
     const unsigned long long first = (unsigned long long)v0;
     GS_CUDA(cudaMemcpyAsync(work + 2, &first, sizeof(first), cudaMemcpyHostToDevice, s));
@@ -1100,6 +1560,38 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     GS_LAUNCH();
   }
   GS_TRY(exclusive_scan_i32_to_i64(items_sorted, item_off, n, pool, s));
+  // hub numbers, when some vertex is beyond the warp kernel
+  Hubs hubs;
+  uint16_t *num = nullptr, *o16 = nullptr;
+  int32_t* hub_list = nullptr;
+  HubInfo* hub_info = nullptr;
+  if (n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG && !warp_vertex(maxdeg, max_od, cfg.warp_deg)) {
+    num = pool.get<uint16_t>(n);
+    o16 = pool.get<uint16_t>(m + 2);
+    hub_list = pool.get<int32_t>(HUB_MAX);
+    hub_info = pool.get<HubInfo>(1);
+    unsigned long long* hh = pool.get<unsigned long long>(2 * nbins);
+    int64_t* pre = pool.get<int64_t>(nbins + 1);
+    if (!num || !o16 || !hub_list || !hub_info || !hh || !pre) return SCAN_ENOMEM;
+    const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 64);
+    GS_CUDA(cudaMemsetAsync(hh, 0, 2 * nbins * sizeof(unsigned long long), s));
+    GS_CUDA(cudaMemsetAsync(num, 0xff, n * sizeof(uint16_t), s));
+    const int64_t hbins = (int64_t)maxdeg - HUB_MIN_DEG + 1;
+    k_hub_hist<<<g, 256, 0, s>>>(deg, n, maxdeg, hh);
+    GS_LAUNCH();
+    GS_TRY(exclusive_scan_i64(reinterpret_cast<const int64_t*>(hh), pre, hbins, pool, s));
+    k_hub_cut<<<1, 32, 0, s>>>(pre, hbins, maxdeg, hub_info);
+    GS_LAUNCH();
+    k_hub_place<<<g, 256, 0, s>>>(deg, n, maxdeg, hub_info, pre, hh + nbins, hub_list);
+    GS_LAUNCH();
+    k_hub_number<<<sm_count() * 8, 256, 0, s>>>(deg, maxdeg, hub_info, pre, hub_list, num);
+    GS_LAUNCH();
+    k_hub_items<<<1, 32, 0, s>>>(hub_info, maxdeg, start, item_off, work);
+    GS_LAUNCH();
+    pool.put(hh);
+    pool.put(pre);
+    hubs = Hubs{num, o16, hub_info};
+  }
   cudaEvent_t e0, e1, k0 = nullptr, k1 = nullptr;
   GS_CUDA(cudaEventCreate(&e0));
   GS_CUDA(cudaEventCreate(&e1));
@@ -1125,7 +1617,7 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     k_rank_keys<<<wgrid, EXPAND_T, 0, s>>>(off, deg, odp, oadj, opos, n, okey, oval);
     GS_LAUNCH();
     GS_TRY(segmented_sort_desc(okey, oval, odp, n, edges, max_od, pool, s));
-    k_rank_scatter<<<wgrid, EXPAND_T, 0, s>>>(off, odp, n, okey, oval, oadj, opos);
+    k_rank_scatter<<<wgrid, EXPAND_T, 0, s>>>(off, odp, n, okey, oval, oadj, opos, num, o16);
     GS_LAUNCH();
     if (weighted) {
       k_out_weights<<<wgrid, EXPAND_T, 0, s>>>(off, odp, n, opos, wcsr, ow, status);
@@ -1133,20 +1625,20 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
       if (narrow) {
         GS_TRY((launch_counting_cfg<int32_t, true>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off,
                                                order, work, lsh_T, max_od, deferred, work + 3,
-                                               tcnt, tc16, twin, status, ow, tsum, cfg, s, k0, k1, v1)));
+                                               tcnt, tc16, twin, status, ow, tsum, cfg, s, k0, k1, v1, hubs)));
       } else {
         GS_TRY((launch_counting_cfg<int64_t, true>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off,
                                                order, work, lsh_T, max_od, deferred, work + 3,
-                                               tcnt, nullptr, twin, status, ow, tsum, cfg, s, k0, k1, v1)));
+                                               tcnt, nullptr, twin, status, ow, tsum, cfg, s, k0, k1, v1, hubs)));
       }
     } else if (narrow) {
       GS_TRY((launch_counting_cfg<int32_t, false>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off,
                                               order, work, lsh_T, max_od, deferred, work + 3, tcnt,
-                                              tc16, twin, status, nullptr, nullptr, cfg, s, k0, k1, v1)));
+                                              tc16, twin, status, nullptr, nullptr, cfg, s, k0, k1, v1, hubs)));
     } else {
       GS_TRY((launch_counting_cfg<int64_t, false>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off,
                                               order, work, lsh_T, max_od, deferred, work + 3, tcnt,
-                                              nullptr, twin, status, nullptr, nullptr, cfg, s, k0, k1, v1)));
+                                              nullptr, twin, status, nullptr, nullptr, cfg, s, k0, k1, v1, hubs)));
     }
   }
   GS_CUDA(cudaEventRecord(e1, s));
@@ -1191,6 +1683,12 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
   pool.put(start);
   pool.put(item_off);
   pool.put(work);
+  if (num) {
+    pool.put(num);
+    pool.put(o16);
+    pool.put(hub_list);
+    pool.put(hub_info);
+  }
   pool.put(odp);
   pool.put(okey);
   pool.put(oval);
