@@ -234,7 +234,7 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
     if (row) pool.put(row);
     GS_TRY(ev.mark(s));
     GS_TRY(segmented_sort_desc((uint64_t*)ix->no_sim, ix->no_id, ix->off, n, arcs, ix->maxdeg, pool,
-                               s));
+                               s, true));
     GS_TRY(ev.mark(s));
     return SCAN_OK;
   }
@@ -282,7 +282,8 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
   if (row) pool.put(row);
   GS_TRY(ev.mark(s));
   // ---- neighbour order (Algorithm 2)
-  GS_TRY(segmented_sort_desc((uint64_t*)ix->no_sim, ix->no_id, ix->off, n, arcs, ix->maxdeg, pool, s));
+  GS_TRY(segmented_sort_desc((uint64_t*)ix->no_sim, ix->no_id, ix->off, n, arcs, ix->maxdeg, pool, s,
+                             true));
   GS_TRY(ev.mark(s));
   return SCAN_OK;
 }

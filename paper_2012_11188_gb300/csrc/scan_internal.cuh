@@ -166,9 +166,12 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
 
 // Sort every segment [seg_off[i], seg_off[i+1]) of (key, val) pairs by key
 // descending, then val ascending. Keys are non-negative doubles viewed as
-// uint64. max_len bounds every segment length.
+// uint64. max_len bounds every segment length. ascending_vals: the vals of
+// every segment ascend (as in an id-sorted CSR row), so that ties may be kept
+// in place.
 int segmented_sort_desc(uint64_t* key, int32_t* val, const int64_t* seg_off, int64_t nseg,
-                        int64_t total, int64_t max_len, Pool& pool, cudaStream_t s);
+                        int64_t total, int64_t max_len, Pool& pool, cudaStream_t s,
+                        bool ascending_vals = false);
 
 // Core order from the neighbour order (Algorithm 2, MakeCoreOrder).
 int build_core_order(IndexData& ix, Pool& pool, cudaStream_t s);

@@ -349,6 +349,86 @@ k_sort_huge(const uint64_t* ik, const int32_t* iv, uint64_t* key, int32_t* val, 
   }
 }
 
+// ---- Segments as 64-bit words.
+// A merge level on pairs moves 12 bytes per element and compares a 64-bit
+// key, then a val on ties. Where the segment's key range leaves room, an
+// element is packed into one word that orders as the pair does and gives it
+// back: (max key - key), then
+//  - the val's difference from the smallest, or
+//  - where the caller says that the vals ascend in every segment, the position
+//    (8 to 12 bits; the val is fetched by it at the end).
+// No key bit is dropped: similarities that are equal in exact arithmetic often
+// differ by one unit in the last place, and thousands of them would share the
+// leading bits. Builds, before and after: R-MAT s24 162.5 -> 155.5 ms, s20
+// 10.27 -> 10.04, dense 25,825 vertices 28.9 -> 27.0, 512 SBM graphs 85.9 -> 83.0.
+__device__ __forceinline__ void cas64(uint64_t& a, uint64_t& b) {
+  const uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
+  a = lo;
+  b = hi;
+}
+
+__device__ __forceinline__ void sort_regs64(uint64_t (&K)[8]) {
+#define GS_CAS64(i, j) cas64(K[i], K[j])
+  GS_CAS64(0, 1); GS_CAS64(2, 3); GS_CAS64(4, 5); GS_CAS64(6, 7);
+  GS_CAS64(0, 2); GS_CAS64(1, 3); GS_CAS64(4, 6); GS_CAS64(5, 7);
+  GS_CAS64(1, 2); GS_CAS64(5, 6);
+  GS_CAS64(0, 4); GS_CAS64(1, 5); GS_CAS64(2, 6); GS_CAS64(3, 7);
+  GS_CAS64(2, 4); GS_CAS64(3, 5);
+  GS_CAS64(1, 2); GS_CAS64(3, 4); GS_CAS64(5, 6);
+#undef GS_CAS64
+}
+
+// 8 outputs from diagonal d of the ascending runs [a, a + la) and [a + la,
+// a + la + lb) of ks, to slots o .. of kd (padded by pslot; o a multiple of 8).
+__device__ __forceinline__ void merge_words(const uint64_t* ks, int a, int la, int lb, int d,
+                                            uint64_t* kd, int o) {
+  int lo = max(0, d - lb), hi = min(d, la);
+  const int bd = a + la + d - 1;
+  while (lo < hi) {
+    const int i = (lo + hi) >> 1;
+    if (ks[pslot<8>(bd - i)] < ks[pslot<8>(a + i)]) hi = i;
+    else lo = i + 1;
+  }
+  int ia = a + lo, ib = a + la + d - lo;
+  const int ea = a + la, eb = a + la + lb;
+  // an exhausted run's head is the largest word, as the padding's
+  uint64_t ka = ia < ea ? ks[pslot<8>(ia)] : ~0ull;
+  uint64_t kb = ib < eb ? ks[pslot<8>(ib)] : ~0ull;
+  kd += pslot<8>(o);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const bool ta = ka <= kb;
+    kd[q] = ta ? ka : kb;
+    const int nx = (ta ? ia : ib) + 1, e = ta ? ea : eb;
+    const uint64_t kn = nx < e ? ks[pslot<8>(nx)] : ~0ull;
+    ia = ta ? nx : ia;
+    ib = ta ? ib : nx;
+    ka = ta ? kn : ka;
+    kb = ta ? kb : kn;
+  }
+}
+
+// Extremes of a segment's keys and vals (vals with the sign bit turned, so
+// that they order as unsigned).
+struct SegRange {
+  uint64_t kmin, kmax;
+  unsigned vmin, vmax;
+};
+
+__device__ __forceinline__ SegRange warp_range(SegRange x) {
+  constexpr unsigned FULL = 0xffffffffu;
+  SegRange r;
+  const unsigned hx = __reduce_max_sync(FULL, (unsigned)(x.kmax >> 32));
+  const unsigned hn = __reduce_min_sync(FULL, (unsigned)(x.kmin >> 32));
+  const unsigned lx = __reduce_max_sync(FULL, (unsigned)(x.kmax >> 32) == hx ? (unsigned)x.kmax : 0u);
+  const unsigned ln = __reduce_min_sync(FULL, (unsigned)(x.kmin >> 32) == hn ? (unsigned)x.kmin : ~0u);
+  r.kmax = (uint64_t)hx << 32 | lx;
+  r.kmin = (uint64_t)hn << 32 | ln;
+  r.vmin = __reduce_min_sync(FULL, x.vmin);
+  r.vmax = __reduce_max_sync(FULL, x.vmax);
+  return r;
+}
+
 // One CTA of TT threads sorts a tile of up to TT*RI elements (RI = 8 or 16):
 // the tile is loaded into shared memory with coalesced reads (padded with
 // sentinels that sort last up to a multiple of RI), each thread sorts RI
@@ -365,7 +445,10 @@ __global__ void __launch_bounds__(TT, TT * RI >= 8192 ? 1 : (TT >= 1024 ? 1 : 10
 k_sort_tile(const uint64_t* ik, const int32_t* iv, uint64_t* key, int32_t* val, Segs S,
             const int64_t* __restrict__ list, const unsigned long long* __restrict__ count_ptr,
             const int64_t* __restrict__ tile_prefix, int64_t nlong, uint64_t* __restrict__ tk,
-            int32_t* __restrict__ tv) {
+            int32_t* __restrict__ tv, bool ascending) {
+  constexpr bool WORDS = !TILED && RI == 8;
+  constexpr int IB = 31 - __builtin_clz(TT * RI);  // bits of a position
+  __shared__ SegRange s_range[WORDS ? TT / 32 : 1];
   constexpr int CAP = TT * RI;
   constexpr int PCAP = CAP + CAP / RI;  // padded slots per buffer
   extern __shared__ uint64_t tsm[];
@@ -398,10 +481,93 @@ k_sort_tile(const uint64_t* ik, const int32_t* iv, uint64_t* key, int32_t* val, 
     // merge levels clip their last run pair there, so the work follows len
     const int lr = len <= RI ? RI : (int)((len + RI - 1) / RI) * RI;
     // 1. coalesced load, sentinels past the end
-    for (int i = t; i < lr; i += TT) {
-      const int p = pslot<RI>(i);
-      if (i < len) { k0[p] = ik[b + i]; v0[p] = iv[b + i]; }
-      else { k0[p] = 0; v0[p] = SENT_V; }
+    if (WORDS) {
+      uint64_t K[RI];
+      int32_t V[RI];
+      SegRange rg{~0ull, 0, ~0u, 0};
+#pragma unroll
+      for (int r = 0; r < RI; ++r) {
+        const int i = t + r * TT;
+        K[r] = 0;
+        V[r] = SENT_V;
+        if (i < len) {
+          K[r] = ik[b + i];
+          V[r] = iv[b + i];
+          rg.kmin = min(rg.kmin, K[r]);
+          rg.kmax = max(rg.kmax, K[r]);
+          rg.vmin = min(rg.vmin, (unsigned)V[r] ^ 0x80000000u);
+          rg.vmax = max(rg.vmax, (unsigned)V[r] ^ 0x80000000u);
+        }
+      }
+      rg = warp_range(rg);
+      if (TT > 32) {
+        if ((t & 31) == 0) s_range[t >> 5] = rg;
+        __syncthreads();
+        rg = warp_range(s_range[t & (TT / 32 - 1)]);
+      }
+      const int kbits = 64 - __clzll((long long)(rg.kmax - rg.kmin));
+      const int vbits = 32 - __clz((int)(rg.vmax - rg.vmin));
+      const bool by_val = kbits + vbits <= 64;
+      if (by_val || (ascending && kbits + IB <= 64)) {
+        // the words fill k0, k1 and, by position, the vals v0
+        const int low = by_val ? vbits : IB;
+#pragma unroll
+        for (int r = 0; r < RI; ++r) {
+          const int i = t + r * TT;
+          if (i < lr) {
+            const uint64_t d = low < 64 ? (rg.kmax - K[r]) << low : 0;
+            const uint64_t x = by_val ? (uint64_t)(((unsigned)V[r] ^ 0x80000000u) - rg.vmin)
+                                      : (uint64_t)i;
+            k0[pslot<8>(i)] = i < len ? d | x : ~0ull;
+            if (!by_val) v0[i] = V[r];
+          }
+        }
+        __syncthreads();
+        const int o = 8 * t;
+        if (o < lr) {
+          uint64_t W[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) W[r] = k0[pslot<8>(o) + r];
+          sort_regs64(W);
+#pragma unroll
+          for (int r = 0; r < 8; ++r) k0[pslot<8>(o) + r] = W[r];
+        }
+        __syncwarp();
+        uint64_t *ks = k0, *kd = k1;
+        for (int w = 8; w < lr; w <<= 1) {  // up to 256 words a run is one warp's
+          if (o < lr) {
+            const int a = o & ~(2 * w - 1);
+            const int la = min(w, lr - a), lb = max(0, min(w, lr - a - w));
+            merge_words(ks, a, la, lb, o - a, kd, o);
+          }
+          if (w < 128 || TT == 32) __syncwarp();
+          else __syncthreads();
+          uint64_t* x = ks;
+          ks = kd;
+          kd = x;
+        }
+        if (lr <= 256 && TT > 32) __syncthreads();
+        const uint64_t mask = (1ull << low) - 1;  // low <= 32
+        for (int i = t; i < len; i += TT) {
+          const uint64_t x = ks[pslot<8>(i)];
+          ok[b + i] = rg.kmax - (x >> low);
+          ov[b + i] = by_val ? (int32_t)(((unsigned)(x & mask) + rg.vmin) ^ 0x80000000u)
+                             : v0[x & mask];
+        }
+        __syncthreads();
+        continue;
+      }
+#pragma unroll
+      for (int r = 0; r < RI; ++r) {
+        const int i = t + r * TT;
+        if (i < lr) { const int p = pslot<RI>(i); k0[p] = K[r]; v0[p] = V[r]; }
+      }
+    } else {
+      for (int i = t; i < lr; i += TT) {
+        const int p = pslot<RI>(i);
+        if (i < len) { k0[p] = ik[b + i]; v0[p] = iv[b + i]; }
+        else { k0[p] = 0; v0[p] = SENT_V; }
+      }
     }
     __syncthreads();
     // 2. each thread sorts its RI consecutive elements in registers
@@ -999,9 +1165,11 @@ unsigned grid_of(int64_t units, int per) {
 
 // Sorts every segment of S into (key, val). The data is in (key, val), or
 // in the copy (alt_k, alt_v) when in_alt; alt_k may be null until a level
-// needs it (it then holds total elements).
+// needs it (it then holds total elements). ascending: the vals of every
+// segment ascend.
 int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Segs S, int64_t nseg,
-               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth);
+               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth,
+               bool ascending = false);
 
 // Moves the elements of the nlong long segments (device list llist) into
 // their buckets in the other array pair and sorts the buckets, as segments of
@@ -1094,7 +1262,7 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
 }
 
 int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Segs S, int64_t nseg,
-               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth) {
+               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth, bool ascending) {
   if (nseg <= 0 || total <= 1) return SCAN_OK;
   unsigned long long* counts = pool.get<unsigned long long>(2 * NCNT);
   if (!counts) return SCAN_ENOMEM;
@@ -1145,7 +1313,7 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
     // networks and merge levels: compact code, unlike fully unrolled bitonic
     // networks, whose instruction footprint stalls the warp on fetches)
     k_sort_tile<32, 8, false><<<grid_of((int64_t)hc[1], 1), 32, tile_smem_bytes<32, 8>(), s>>>(
-        ik, iv, key, val, S, list + base[1], counts + 1, nullptr, 0, nullptr, nullptr);
+        ik, iv, key, val, S, list + base[1], counts + 1, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
   GS_CUDA(cudaFuncSetAttribute(k_merge_pass, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1161,23 +1329,23 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
                                (int)tile_smem_bytes<T4K_T, 8>()));
   if (hc[2]) {
     k_sort_tile<64, 8, false><<<grid_of((int64_t)hc[2], 1), 64, tile_smem_bytes<64, 8>(), s>>>(
-        ik, iv, key, val, S, list + base[2], counts + 2, nullptr, 0, nullptr, nullptr);
+        ik, iv, key, val, S, list + base[2], counts + 2, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
   if (hc[3]) {
     k_sort_tile<128, 8, false><<<grid_of((int64_t)hc[3], 1), 128, tile_smem_bytes<128, 8>(), s>>>(
-        ik, iv, key, val, S, list + base[3], counts + 3, nullptr, 0, nullptr, nullptr);
+        ik, iv, key, val, S, list + base[3], counts + 3, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
   if (hc[4]) {
     k_sort_tile<256, 8, false><<<grid_of((int64_t)hc[4], 1), 256, tile_smem_bytes<256, 8>(), s>>>(
-        ik, iv, key, val, S, list + base[4], counts + 4, nullptr, 0, nullptr, nullptr);
+        ik, iv, key, val, S, list + base[4], counts + 4, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
   if (hc[5]) {
     k_sort_tile<T4K_T, 8, false><<<grid_of((int64_t)hc[5], 1), T4K_T, tile_smem_bytes<T4K_T, 8>(),
                                  s>>>(
-        ik, iv, key, val, S, list + base[5], counts + 5, nullptr, 0, nullptr, nullptr);
+        ik, iv, key, val, S, list + base[5], counts + 5, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
   if (nlong && !bucketed && !whole) {
@@ -1202,7 +1370,7 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
     // tile sort (count = ntiles, read from counts[NCLASS])
     k_sort_tile<TLONG_T, TLONG_RI, true><<<grid_of(ntiles, 1), TLONG_T,
                                           tile_smem_bytes<TLONG_T, TLONG_RI>(), s>>>(
-        key, val, key, val, S, llist, counts + NCLASS, tile_prefix, nlong, tk, tv);
+        key, val, key, val, S, llist, counts + NCLASS, tile_prefix, nlong, tk, tv, false);
     GS_LAUNCH();
     const int64_t total_chunks_ub = (total + MERGE_CHUNK - 1) / MERGE_CHUNK + nlong;
     MergeDesc* desc = pool.get<MergeDesc>((size_t)total_chunks_ub);
@@ -1236,10 +1404,11 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
 }  // namespace
 
 int segmented_sort_desc(uint64_t* key, int32_t* val, const int64_t* seg_off, int64_t nseg,
-                        int64_t total, int64_t max_len, Pool& pool, cudaStream_t s) {
+                        int64_t total, int64_t max_len, Pool& pool, cudaStream_t s,
+                        bool ascending_vals) {
   if (nseg <= 0 || total <= 1 || max_len <= 1) return SCAN_OK;
   return sort_level(key, val, nullptr, nullptr, Segs{seg_off, seg_off + 1}, nseg, total, false, pool,
-                    s, 0);
+                    s, 0, ascending_vals);
 }
 
 }  // namespace gscan

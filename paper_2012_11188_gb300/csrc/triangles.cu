@@ -1616,7 +1616,7 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     GS_TRY(exclusive_scan_i32_to_i64(odeg, odp, n, pool, s));
     k_rank_keys<<<wgrid, EXPAND_T, 0, s>>>(off, deg, odp, oadj, opos, n, okey, oval);
     GS_LAUNCH();
-    GS_TRY(segmented_sort_desc(okey, oval, odp, n, edges, max_od, pool, s));
+    GS_TRY(segmented_sort_desc(okey, oval, odp, n, edges, max_od, pool, s, true));
     k_rank_scatter<<<wgrid, EXPAND_T, 0, s>>>(off, odp, n, okey, oval, oadj, opos, num, o16);
     GS_LAUNCH();
     if (weighted) {
