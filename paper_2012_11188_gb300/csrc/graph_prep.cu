@@ -97,36 +97,32 @@ int scan_impl(const T* in, int64_t* out, int64_t n, Pool& pool, cudaStream_t s) 
   return SCAN_OK;
 }
 
-// deg[v], per-row checks, max degree. One warp per vertex row.
-// Degrees and CSR checks, 32 rows per warp: lane j reads the bounds of row
-// v0 + j, then the warp walks the group's arcs [off[v0], off[v0 + 32]) --
-// contiguous -- 32 positions at a time, each lane finding its row among the
-// group's by a five-step search over the lanes' row starts. (One warp per row
-// would leave most lanes idle on the many short rows.) Rows longer than
-// DEG_LONG are listed for k_degrees_long and jumped over (one warp would walk
+// Degrees and CSR checks, 32 rows per warp (RowGroup). Rows longer than
+// DEG_LONG are listed for k_degrees_long and left out (one warp would walk
 // a hub's row alone, one dependent load at a time). A group with a bad row
 // bound is not walked.
 constexpr int DEG_LONG = 4096;
 
-__global__ void k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                          int64_t n, int64_t arcs, int32_t* __restrict__ deg, int32_t* maxdeg,
-                          unsigned* status, int32_t* __restrict__ long_rows,
-                          unsigned* __restrict__ n_long) {
+__global__ void __launch_bounds__(256)
+k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+          int64_t n, int64_t arcs, int32_t* __restrict__ deg, int32_t* maxdeg,
+          unsigned* status, int32_t* __restrict__ long_rows,
+          unsigned* __restrict__ n_long) {
   constexpr unsigned FULL = 0xffffffffu;
+  __shared__ int scratch[8][64];
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int32_t local_max = 0;
   unsigned bad = 0;
   for (int64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
-    const int cnt = (int)min((int64_t)32, n - v0);  // rows in this group
     const int64_t v = v0 + lane;
     int64_t b = 0, e = 0;
-    if (lane < cnt) { b = off[v]; e = off[v + 1]; }
+    if (v < n) { b = off[v]; e = off[v + 1]; }
     // rows must lie inside [0, arcs] before adj is touched
-    const bool row_bad = lane < cnt && (b < 0 || e > arcs || e - b < 0 || e - b > 0x7fffffff);
+    const bool row_bad = b < 0 || e > arcs || e - b < 0 || e - b > 0x7fffffff;
     const bool is_long = !row_bad && e - b > DEG_LONG;
-    if (lane < cnt) {
+    if (v < n) {
       deg[v] = row_bad ? 0 : (int32_t)(e - b);
       if (!row_bad) local_max = max(local_max, (int32_t)(e - b));
       if (is_long) long_rows[atomicAdd(n_long, 1u)] = (int32_t)v;
@@ -135,34 +131,26 @@ __global__ void k_degrees(const int64_t* __restrict__ off, const int32_t* __rest
       bad = 1;
       continue;
     }
-    const int64_t gb = __shfl_sync(FULL, b, 0), ge = __shfl_sync(FULL, e, cnt - 1);
-    int32_t carry = 0;  // adj[i - 1] for lane 0
-    for (int64_t i0 = gb; i0 < ge;) {
-      const int64_t i = i0 + lane;
-      // row of position i: the last row of the group starting at or before it
-      int j = 0;
-#pragma unroll
-      for (int step = 16; step; step >>= 1) {
-        const int64_t bs = __shfl_sync(FULL, b, (j + step) & 31);
-        if (j + step < cnt && bs <= i) j += step;
-      }
-      const bool row_long = __shfl_sync(FULL, is_long, j);
-      const int j0 = __shfl_sync(FULL, j, 0);
-      if (__shfl_sync(FULL, row_long, 0)) {  // the chunk starts inside a long row: skip it
-        i0 = __shfl_sync(FULL, e, j0);
-        continue;
-      }
-      const bool act = i < ge && !row_long;
-      const int32_t x = act ? adj[i] : 0;
-      const int64_t bj = __shfl_sync(FULL, b, j);
+    RowGroup g;
+    g.init(is_long ? 0 : (int)(e - b), scratch[threadIdx.x >> 5]);
+    // element of a virtual position: adj[base of its row + position]
+    const int64_t base = __shfl_sync(FULL, b, g.row) - g.vs;
+    int32_t carry = 0;  // the element before the chunk
+    for (int i0 = 0; i0 < g.total; i0 += 32) {
+      const int k = g.chunk(i0);
+      const int i = i0 + lane;
+      const int64_t bk = __shfl_sync(FULL, base, k);
+      const int32_t own = (int32_t)v0 + __shfl_sync(FULL, g.row, k);
+      const bool act = i < g.total;
+      const int32_t x = act ? adj[bk + i] : 0;
       int32_t prev = __shfl_up_sync(FULL, x, 1);
       if (lane == 0) prev = carry;
       carry = __shfl_sync(FULL, x, 31);
       if (act) {
-        if (x < 0 || x >= n || x == v0 + j) bad = 1;
-        if (i > bj && prev >= x) bad = 1;  // strictly ascending: sorted, no duplicates
+        if (x < 0 || x >= n || x == own) bad = 1;
+        // strictly ascending inside a row: sorted, no duplicates
+        if (!(g.starts >> lane & 1u) && prev >= x) bad = 1;
       }
-      i0 += 32;
     }
   }
   for (int o = 16; o; o >>= 1) local_max = max(local_max, __shfl_xor_sync(FULL, local_max, o));
@@ -200,21 +188,23 @@ __device__ __forceinline__ bool lower(int32_t du, int32_t u, int32_t dv, int32_t
 // are compacted, in id order, to the front of v's own CSR slot range, so
 // out(v) = oadj[off[v] .. off[v] + od[v]) needs no separate offsets; the
 // in-arcs fill the row from its end; opos holds each arc's position in the
-// row. 32 rows per warp, as in k_degrees: lane j keeps row v0 + j's bounds
-// and its running out- and in-arc counts, the warp walks the group's arcs 32
-// positions at a time, and each lane finds its row by a five-step search and
-// its place by ballots masked to its row's lanes. Rows longer than LONG_ROW
-// are listed in long_rows for k_orient_long and jumped over.
+// row. 32 rows per warp (RowGroup): lane k keeps the out-arcs placed so far
+// of the k-th non-empty row, and a position finds its place by ballots masked
+// to its row's lower lanes; the in-arcs before it are the other positions
+// before it. Rows longer than LONG_ROW are listed in long_rows for
+// k_orient_long and left out.
 constexpr int LONG_ROW = 4096;
 constexpr int LONG_T = 1024;
 
-__global__ void k_orient_inplace(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                 const int32_t* __restrict__ deg, int64_t n,
-                                 int32_t* __restrict__ od, int32_t* __restrict__ oadj,
-                                 int32_t* __restrict__ opos, int32_t* max_od,
-                                 unsigned long long* sum_od, int32_t* __restrict__ long_rows,
-                                 unsigned* __restrict__ n_long) {
+__global__ void __launch_bounds__(256)
+k_orient_inplace(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                 const int32_t* __restrict__ deg, int64_t n,
+                 int32_t* __restrict__ od, int32_t* __restrict__ oadj,
+                 int32_t* __restrict__ opos, int32_t* max_od,
+                 unsigned long long* sum_od, int32_t* __restrict__ long_rows,
+                 unsigned* __restrict__ n_long) {
   constexpr unsigned FULL = 0xffffffffu;
+  __shared__ int scratch[8][64];
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;  // lanes below this one
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -222,60 +212,47 @@ __global__ void k_orient_inplace(const int64_t* __restrict__ off, const int32_t*
   unsigned long long local_sum = 0;
   int32_t local_max = 0;
   for (int64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
-    const int cnt = (int)min((int64_t)32, n - v0);  // rows in this group
     const int64_t v = v0 + lane;
-    int64_t b = 0, e = 0;
+    int64_t b = 0;
     int32_t d = 0;
-    if (lane < cnt) { b = off[v]; e = off[v + 1]; d = deg[v]; }
+    if (v < n) { b = off[v]; d = deg[v]; }
     const bool is_long = d > LONG_ROW;
     if (is_long) long_rows[atomicAdd(n_long, 1u)] = (int32_t)v;
-    int32_t w = 0, wi = 0;  // this lane's row: out-arcs placed from the front, in-arcs from the back
-    const int64_t gb = __shfl_sync(FULL, b, 0), ge = __shfl_sync(FULL, e, cnt - 1);
-    for (int64_t i0 = gb; i0 < ge;) {
-      const int64_t i = i0 + lane;
-      int j = 0;  // row of position i: the last row of the group starting at or before it
-#pragma unroll
-      for (int step = 16; step; step >>= 1) {
-        const int64_t bs = __shfl_sync(FULL, b, (j + step) & 31);
-        if (j + step < cnt && bs <= i) j += step;
-      }
-      const bool row_long = __shfl_sync(FULL, is_long, j);
-      const int j0 = __shfl_sync(FULL, j, 0);
-      if (__shfl_sync(FULL, row_long, 0)) {  // the chunk starts inside a long row: skip it
-        i0 = __shfl_sync(FULL, e, j0);
-        continue;
-      }
-      const int64_t bj = __shfl_sync(FULL, b, j), ej = __shfl_sync(FULL, e, j);
-      const int32_t dj = __shfl_sync(FULL, d, j);
-      const int32_t wj = __shfl_sync(FULL, w, j), wij = __shfl_sync(FULL, wi, j);
-      const bool act = i < ge && !row_long;
+    if (v < n && d == 0) od[v] = 0;
+    RowGroup g;
+    g.init(is_long ? 0 : d, scratch[threadIdx.x >> 5]);
+    const int64_t start = __shfl_sync(FULL, b, g.row);  // of lane's compacted row
+    int32_t w = 0;                                      // its out-arcs placed so far
+    for (int i0 = 0; i0 < g.total; i0 += 32) {
+      const int k = g.chunk(i0);
+      const int i = i0 + lane;
+      const int64_t rb = __shfl_sync(FULL, start, k);
+      const int vsk = __shfl_sync(FULL, g.vs, k), vek = __shfl_sync(FULL, g.ve, k);
+      const int wk = __shfl_sync(FULL, w, k);
+      const int32_t own = (int32_t)v0 + __shfl_sync(FULL, g.row, k);
+      const bool act = i < g.total;
+      const int p = i - vsk;  // position in the row
       int32_t x = 0;
       bool up = false;
-      if (act) { x = adj[i]; up = lower(dj, (int32_t)(v0 + j), deg[x], x); }
-      const unsigned m = __ballot_sync(FULL, up), am = __ballot_sync(FULL, act);
-      // lanes of row j in this chunk: [bj - i0, ej - i0) clipped to [0, 32)
-      const int lo = (int)max((int64_t)0, bj - i0), hi = (int)min((int64_t)32, ej - i0);
-      const unsigned rowm = (hi >= 32 ? FULL : ((1u << hi) - 1u)) & ~((1u << lo) - 1u);
-      if (up) {
-        const int64_t dst = bj + wj + __popc(m & rowm & lt);
+      if (act) { x = adj[rb + p]; up = lower(vek - vsk, own, deg[x], x); }
+      const unsigned m = __ballot_sync(FULL, up);
+      // out-arcs of the row before this position: placed ones and lower lanes
+      // from the row's first position in the chunk on
+      const unsigned st = g.starts & (lt | (lt + 1u));
+      const unsigned from = st ? ~((1u << (31 - __clz(st))) - 1u) : FULL;
+      const int ups = wk + __popc(m & lt & from);
+      if (act) {
+        const int64_t dst = up ? rb + ups : rb + (vek - vsk) - 1 - (p - ups);
         oadj[dst] = x;
-        opos[dst] = (int32_t)(i - bj);
-      } else if (act) {
-        const int64_t dst = ej - 1 - (wij + __popc(~m & am & rowm & lt));
-        oadj[dst] = x;
-        opos[dst] = (int32_t)(i - bj);
+        opos[dst] = p;
       }
-      // each row's owner lane adds its row's counts of this chunk
-      const int mlo = (int)max((int64_t)0, b - i0), mhi = (int)min((int64_t)32, e - i0);
-      if (lane < cnt && mlo < mhi) {
-        const unsigned own = (mhi >= 32 ? FULL : ((1u << mhi) - 1u)) & ~((1u << mlo) - 1u);
-        w += __popc(m & own);
-        wi += __popc(~m & am & own);
-      }
-      i0 += 32;
+      // each row's owner lane adds its row's out-arcs of this chunk
+      const int mlo = max(0, g.vs - i0), mhi = min(32, g.ve - i0);
+      if (lane < g.cnt && mlo < mhi)
+        w += __popc(m & (FULL >> (32 - mhi)) & (FULL << mlo));
     }
-    if (lane < cnt && !is_long) {
-      od[v] = w;
+    if (lane < g.cnt) {
+      od[v0 + g.row] = w;
       local_sum += (unsigned long long)w;
       local_max = max(local_max, w);
     }

@@ -1149,33 +1149,35 @@ __device__ __forceinline__ int64_t row_of(const int64_t* __restrict__ odp, int64
 }
 
 // Every out-arc in compact order (k = odp[a] + i, i < od[a], at CSR
-// position j = off[a] + i), 32 rows per warp: lane l holds row v0 + l's odp
-// and off, the warp walks the group's out-arcs [odp[v0], odp[v0 + 32]) --
-// contiguous -- 32 at a time, and each lane finds its row by a five-step
-// search over the lanes' odp values (no dependent global loads, unlike a
-// binary search of odp). f(k, a, j) runs for every out-arc.
+// position j = off[a] + i), 32 rows per warp (RowGroup; EXPAND_T threads per
+// CTA): f(k, a, j) runs for every out-arc.
 template <class F>
 __device__ __forceinline__ void walk_out_arcs(const int64_t* __restrict__ off,
                                               const int64_t* __restrict__ odp, int64_t n, F f) {
   constexpr unsigned FULL = 0xffffffffu;
+  __shared__ int scratch[EXPAND_T / 32][64];
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
-    const int cnt = (int)min((int64_t)32, n - v0);
+    const int64_t v = v0 + lane;
     int64_t kb = 0, rb = 0;
-    if (lane < cnt) { kb = odp[v0 + lane]; rb = off[v0 + lane]; }
-    const int64_t g0 = __shfl_sync(FULL, kb, 0), g1 = odp[v0 + cnt];
-    for (int64_t k0 = g0; k0 < g1; k0 += 32) {
-      const int64_t k = k0 + lane;
-      int r = 0;
-#pragma unroll
-      for (int step = 16; step; step >>= 1) {
-        const int64_t bs = __shfl_sync(FULL, kb, (r + step) & 31);
-        if (r + step < cnt && bs <= k) r += step;
-      }
-      const int64_t kbr = __shfl_sync(FULL, kb, r), rbr = __shfl_sync(FULL, rb, r);
-      if (k < g1) f(k, v0 + r, rbr + (k - kbr));
+    int len = 0;
+    if (v < n) {
+      kb = odp[v];
+      rb = off[v];
+      len = (int)(odp[v + 1] - kb);
+    }
+    const int64_t g0 = __shfl_sync(FULL, kb, 0);
+    RowGroup g;
+    g.init(len, scratch[threadIdx.x >> 5]);
+    const int64_t base = __shfl_sync(FULL, rb, g.row) - g.vs;
+    for (int i0 = 0; i0 < g.total; i0 += 32) {
+      const int k = g.chunk(i0);
+      const int64_t bk = __shfl_sync(FULL, base, k);
+      const int row = __shfl_sync(FULL, g.row, k);
+      const int i = i0 + lane;
+      if (i < g.total) f(g0 + i, v0 + row, bk + i);
     }
   }
 }
