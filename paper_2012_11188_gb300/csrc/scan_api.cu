@@ -129,6 +129,19 @@ size_t build_footprint(int64_t n, int64_t arcs) {
 
 namespace {
 
+// A pointer that kernels of the current device may use as 4-byte (or `align`)
+// words: device memory of this device. Copies take any other kind.
+bool kernel_reads(const void* p, size_t align) {
+  if ((uintptr_t)p % align) return false;
+  int dev = 0;
+  cudaPointerAttributes at;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 __global__ void k_off32_to_64(const int32_t* __restrict__ in, int64_t n1, int64_t* __restrict__ out) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n1;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -398,42 +411,79 @@ __device__ __forceinline__ int64_t last_le(const int64_t* a, int64_t cnt, int64_
   return lo;
 }
 
-// union offsets: off[u] = ab_g + raw[u + g] for u in graph g; off[N] = A.
-// raw holds each graph's own n_g+1 offsets, graph g starting at vb_g + g.
-__global__ void k_pack_offsets(const int64_t* __restrict__ raw, const int64_t* __restrict__ vb,
-                               const int64_t* __restrict__ ab, int G, int64_t N,
-                               int64_t* __restrict__ off, unsigned* status) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u <= N;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    if (u == N) { off[N] = ab[G]; continue; }
-    const int64_t g = last_le(vb, G, u);
-    const int64_t o = raw[u + g];
-    const int64_t na = ab[g + 1] - ab[g];
-    if (o < 0 || o > na) { atomicOr(status, (unsigned)DEV_BADGRAPH); off[u] = ab[g]; continue; }
-    off[u] = ab[g] + o;
-  }
+// Where a graph's CSR is on the device while it is packed (one in host memory
+// is first copied to the arena).
+struct PackSrc {
+  const void* off;  // n_g + 1 offsets
+  const int32_t* adj;
+  int off64;
+};
+
+__device__ __forceinline__ int64_t src_offset(const PackSrc& p, int64_t i) {
+  return p.off64 ? static_cast<const int64_t*>(p.off)[i] : static_cast<const int32_t*>(p.off)[i];
 }
 
-__global__ void k_check_ends(const int64_t* __restrict__ raw, const int64_t* __restrict__ vb,
-                             const int64_t* __restrict__ ab, int G, unsigned* status) {
+// A CTA's chunk of the union's arcs or vertices: the graph of each element is
+// found by walking on from that of the chunk's first (one search per CTA and
+// chunk; a search per element was 1.4 ms of each pass over the 190M arcs of
+// 512 SBM graphs).
+constexpr int PACK_CH = 4096;
+struct GraphWalk {
+  const int64_t* base;  // ascending bases, G + 1 entries
+  int64_t g;
+  __device__ __forceinline__ GraphWalk(const int64_t* a, int G, int64_t first)
+      : base(a), g(last_le(a, G, first)) {}
+  __device__ __forceinline__ int64_t at(int64_t i) {  // i must not descend
+    while (base[g + 1] <= i) ++g;
+    return g;
+  }
+};
+
+// union offsets: off[u] = ab_g + o_g[u - vb_g] for u in graph g; off[N] = A;
+// every graph's first and last offset are checked.
+__global__ void __launch_bounds__(256)
+k_pack_offsets(const PackSrc* __restrict__ src, const int64_t* __restrict__ vb,
+               const int64_t* __restrict__ ab, int G, int64_t N, int64_t* __restrict__ off,
+               unsigned* status) {
+  bool bad = false;
+  for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < N; c0 += (int64_t)gridDim.x * PACK_CH) {
+    GraphWalk w(vb, G, c0);
+    const int64_t c1 = min(N, c0 + PACK_CH);
+    for (int64_t u = c0 + threadIdx.x; u < c1; u += blockDim.x) {
+      const int64_t g = w.at(u);
+      const int64_t o = src_offset(src[g], u - vb[g]);
+      const int64_t na = ab[g + 1] - ab[g];
+      const bool ok = o >= 0 && o <= na;
+      bad |= !ok;
+      off[u] = ab[g] + (ok ? o : 0);
+    }
+  }
   for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = vb[g] + g, ng = vb[g + 1] - vb[g];
-    if (raw[b] != 0 || raw[b + ng] != ab[g + 1] - ab[g]) atomicOr(status, (unsigned)DEV_BADGRAPH);
-  }
+       g += (int64_t)gridDim.x * blockDim.x)
+    bad |= src_offset(src[g], 0) != 0 ||
+           src_offset(src[g], vb[g + 1] - vb[g]) != ab[g + 1] - ab[g];
+  if (blockIdx.x == 0 && threadIdx.x == 0) off[N] = ab[G];
+  if (bad) atomicOr(status, (unsigned)DEV_BADGRAPH);
 }
 
-// local ids -> union ids (checked against the graph's own n)
-__global__ void k_shift_adj(int32_t* __restrict__ adj, const int64_t* __restrict__ vb,
-                            const int64_t* __restrict__ ab, int G, int64_t A, unsigned* status) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < A;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t g = last_le(ab, G, i);
-    const int32_t x = adj[i];
-    const int64_t ng = vb[g + 1] - vb[g];
-    if (x < 0 || x >= ng) { atomicOr(status, (unsigned)DEV_BADGRAPH); adj[i] = (int32_t)vb[g]; continue; }
-    adj[i] = (int32_t)(x + vb[g]);
+// adjacency into the union, local ids -> union ids (checked against the
+// graph's own n); a graph whose source is the arena is shifted in place
+__global__ void __launch_bounds__(256)
+k_pack_adj(const PackSrc* __restrict__ src, const int64_t* __restrict__ vb,
+           const int64_t* __restrict__ ab, int G, int64_t A, int32_t* adj, unsigned* status) {
+  bool bad = false;
+  for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < A; c0 += (int64_t)gridDim.x * PACK_CH) {
+    GraphWalk w(ab, G, c0);
+    const int64_t c1 = min(A, c0 + PACK_CH);
+    for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
+      const int64_t g = w.at(i);
+      const int32_t x = src[g].adj[i - ab[g]];
+      const bool ok = x >= 0 && x < vb[g + 1] - vb[g];
+      bad |= !ok;
+      adj[i] = (int32_t)((ok ? x : 0) + vb[g]);
+    }
   }
+  if (bad) atomicOr(status, (unsigned)DEV_BADGRAPH);
 }
 
 __global__ void k_graph_maxdeg(const int32_t* __restrict__ deg, const int64_t* __restrict__ vb, int G,
@@ -446,14 +496,17 @@ __global__ void k_graph_maxdeg(const int32_t* __restrict__ deg, const int64_t* _
 }
 
 // union ids -> local ids in adj and NO
-__global__ void k_rebase_ids(int32_t* __restrict__ adj, int32_t* __restrict__ no_id,
-                             const int64_t* __restrict__ vb, const int64_t* __restrict__ ab, int G,
-                             int64_t A) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < A;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t b = (int32_t)vb[last_le(ab, G, i)];
-    adj[i] -= b;
-    no_id[i] -= b;
+__global__ void __launch_bounds__(256)
+k_rebase_ids(int32_t* __restrict__ adj, int32_t* __restrict__ no_id,
+             const int64_t* __restrict__ vb, const int64_t* __restrict__ ab, int G, int64_t A) {
+  for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < A; c0 += (int64_t)gridDim.x * PACK_CH) {
+    GraphWalk w(ab, G, c0);
+    const int64_t c1 = min(A, c0 + PACK_CH);
+    for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
+      const int32_t b = (int32_t)vb[w.at(i)];
+      adj[i] -= b;
+      no_id[i] -= b;
+    }
   }
 }
 
@@ -501,9 +554,9 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   u.no_id = pool.get<int32_t>(A > 0 ? A : 1);
   u.no_sim = pool.get<double>(A > 0 ? A : 1);
   u.status = pool.get<unsigned>(8);
-  int64_t* raw = pool.get<int64_t>(N + G);
   int64_t* meta = pool.get<int64_t>(2 * (size_t)(G + 1));
-  if (!u.off || !u.deg || !u.adj || !u.no_id || !u.no_sim || !u.status || !raw || !meta)
+  PackSrc* d_src = pool.get<PackSrc>(G);
+  if (!u.off || !u.deg || !u.adj || !u.no_id || !u.no_sim || !u.status || !meta || !d_src)
     return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(u.status, 0, 8 * sizeof(unsigned), s));
   std::vector<int64_t> hmeta(2 * (size_t)(G + 1));
@@ -512,40 +565,48 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   GS_CUDA(cudaMemcpyAsync(meta, hmeta.data(), hmeta.size() * 8, cudaMemcpyHostToDevice, s));
   const int64_t* d_vb = meta;
   const int64_t* d_ab = meta + (G + 1);
-  // ---- pack: raw offsets (int64) and adjacency of every graph into the arena
-  std::vector<std::vector<int64_t>> staged;
+  // ---- pack: two kernels read every graph's arrays where they are, through a
+  // table (a pair of copies per graph kept the GPU waiting for 1024 of them
+  // on 512 graphs); arrays that a kernel cannot read are copied in first
+  std::vector<PackSrc> src(G);
+  std::vector<char> staged(G);
+  int64_t staged_n = 0;
   for (int g = 0; g < G; ++g) {
     const scan_csr& c = graphs[g];
-    const cudaMemcpyKind k = c.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    int64_t* dst = raw + vb[g] + g;
-    if (c.offsets_64) {
-      GS_CUDA(cudaMemcpyAsync(dst, c.offsets, (c.n + 1) * 8, k, s));
-    } else if (c.on_device) {
-      k_off32_to_64<<<(unsigned)std::min<int64_t>((c.n + 256) / 256, 4096), 256, 0, s>>>(
-          (const int32_t*)c.offsets, c.n + 1, dst);
-      GS_LAUNCH();
-    } else {
-      staged.emplace_back(c.n + 1);
-      const int32_t* o32 = (const int32_t*)c.offsets;
-      for (int64_t i = 0; i <= c.n; ++i) staged.back()[i] = o32[i];
-      GS_CUDA(cudaMemcpyAsync(dst, staged.back().data(), (c.n + 1) * 8, cudaMemcpyHostToDevice, s));
-    }
-    if (c.num_arcs > 0) GS_CUDA(cudaMemcpyAsync(u.adj + ab[g], c.adj, c.num_arcs * 4, k, s));
+    if (!c.offsets) return SCAN_ECUDA;  // (a graph without vertices has one offset too)
+    staged[g] = !c.on_device || !kernel_reads(c.offsets, c.offsets_64 ? 8 : 4) ||
+                (c.num_arcs > 0 && !kernel_reads(c.adj, 4));
+    if (staged[g]) staged_n += c.n + 1;
   }
+  char* staged_off = staged_n ? (char*)pool.get<int64_t>(staged_n) : nullptr;
+  if (staged_n && !staged_off) return SCAN_ENOMEM;
+  char* at = staged_off;
+  for (int g = 0; g < G; ++g) {
+    const scan_csr& c = graphs[g];
+    src[g] = PackSrc{c.offsets, c.adj, c.offsets_64};
+    if (!staged[g]) continue;
+    const cudaMemcpyKind k = c.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    const size_t ob = (size_t)(c.n + 1) * (c.offsets_64 ? 8 : 4);
+    GS_CUDA(cudaMemcpyAsync(at, c.offsets, ob, k, s));
+    src[g].off = at;
+    at += (size_t)(c.n + 1) * 8;
+    if (c.num_arcs > 0) GS_CUDA(cudaMemcpyAsync(u.adj + ab[g], c.adj, c.num_arcs * 4, k, s));
+    src[g].adj = u.adj + ab[g];
+  }
+  GS_CUDA(cudaMemcpyAsync(d_src, src.data(), src.size() * sizeof(PackSrc), cudaMemcpyHostToDevice,
+                          s));
   const unsigned gN = (unsigned)std::max<int64_t>(1, std::min<int64_t>((N + 256) / 256, sm_count() * 16));
-  const unsigned gA = (unsigned)std::max<int64_t>(1, std::min<int64_t>((A + 255) / 256, sm_count() * 16));
-  const unsigned gG = (unsigned)std::max<int64_t>(1, std::min<int64_t>((G + 255) / 256, sm_count() * 16));
-  k_check_ends<<<gG, 256, 0, s>>>(raw, d_vb, d_ab, G, u.status);
-  GS_LAUNCH();
-  k_pack_offsets<<<gN, 256, 0, s>>>(raw, d_vb, d_ab, G, N, u.off, u.status);
+  const unsigned cN = (unsigned)std::max<int64_t>(1, std::min<int64_t>(N / PACK_CH + 1, sm_count() * 16));
+  const unsigned cA = (unsigned)std::max<int64_t>(1, std::min<int64_t>(A / PACK_CH + 1, sm_count() * 16));
+  k_pack_offsets<<<cN, 256, 0, s>>>(d_src, d_vb, d_ab, G, N, u.off, u.status);
   GS_LAUNCH();
   if (A > 0) {
-    k_shift_adj<<<gA, 256, 0, s>>>(u.adj, d_vb, d_ab, G, A, u.status);
+    k_pack_adj<<<cA, 256, 0, s>>>(d_src, d_vb, d_ab, G, A, u.adj, u.status);
     GS_LAUNCH();
   }
-  GS_CUDA(cudaStreamSynchronize(s));  // staged host offsets must outlive their copies
-  staged.clear();
-  pool.put(raw);
+  GS_CUDA(cudaStreamSynchronize(s));  // the host arrays must outlive their copies
+  if (staged_off) pool.put(staged_off);
+  pool.put(d_src);
   // ---- the shared pipeline over the union (every step is local to a vertex)
   float count_ms = 0;
   GS_TRY(run_pipeline(&u, kind, lsh, pool, s, ev, &count_ms, SCAN_COUNTS_SPARSE, cfg));
@@ -584,7 +645,7 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   std::copy(sb.begin(), sb.end(), hm2.begin() + 3 * (G + 1));
   GS_CUDA(cudaMemcpyAsync(meta2, hm2.data(), hm2.size() * 8, cudaMemcpyHostToDevice, s));
   if (A > 0) {
-    k_rebase_ids<<<gA, 256, 0, s>>>(u.adj, u.no_id, d_vb, d_ab, G, A);
+    k_rebase_ids<<<cA, 256, 0, s>>>(u.adj, u.no_id, d_vb, d_ab, G, A);
     GS_LAUNCH();
   }
   k_rebase_offsets<<<gN, 256, 0, s>>>(u.off, meta2 + (G + 1), meta2, d_ab, G, N + G, off_rel);
@@ -715,6 +776,27 @@ int copy_out(void* dst, const void* src, size_t bytes, cudaStream_t s) {
   return SCAN_OK;
 }
 
+// Small index arrays copied out by one kernel: five copies of a few hundred
+// kilobytes cost their five enqueues (the build and the export of 512 SBM
+// graphs: 82.1 ms, with the packing above 70.2).
+constexpr size_t EXPORT_ONE = 8u << 20;  // bytes in all
+struct ExportParts {
+  void* dst[5];
+  const void* src[5];
+  size_t words[5];  // of 4 bytes
+};
+
+__global__ void __launch_bounds__(256) k_export(ExportParts p) {
+  const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t nt = (size_t)gridDim.x * blockDim.x;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const uint32_t* src = static_cast<const uint32_t*>(p.src[k]);
+    uint32_t* dst = static_cast<uint32_t*>(p.dst[k]);
+    for (size_t i = t0; i < p.words[k]; i += nt) dst[i] = src[i];
+  }
+}
+
 int query_impl(scan_index* index, int q, const int* mu, const double* eps, int32_t* labels,
                int flags, cudaStream_t s) {
   if (!index || q < 0 || (q > 0 && (!mu || !eps || !labels))) return SCAN_EINVAL;
@@ -835,11 +917,27 @@ int scan_index_export(scan_index* index, double* sim, int32_t* no_id, double* no
   const IndexData& ix = index->d;
   cudaStream_t s = ix.home;
   const size_t A = (size_t)ix.arcs;
-  GS_TRY(copy_out(no_id, ix.no_id, A * 4, s));
-  GS_TRY(copy_out(no_sim, ix.no_sim, A * 8, s));
-  GS_TRY(copy_out(co_id, ix.co_id, A * 4, s));
-  GS_TRY(copy_out(co_thr, ix.co_thr, A * 8, s));
-  GS_TRY(copy_out(co_off, ix.co_off, ((size_t)ix.maxdeg + 1) * 8, s));
+  void* dst[5] = {no_id, no_sim, co_id, co_thr, co_off};
+  const void* src[5] = {ix.no_id, ix.no_sim, ix.co_id, ix.co_thr, ix.co_off};
+  const size_t bytes[5] = {A * 4, A * 8, A * 4, A * 8, ((size_t)ix.maxdeg + 1) * 8};
+  ExportParts parts{};
+  size_t total = 0;
+  for (int k = 0; k < 5; ++k) {
+    if (!dst[k] || bytes[k] == 0) continue;
+    if (A * 24 <= EXPORT_ONE && kernel_reads(dst[k], 4)) {
+      parts.dst[k] = dst[k];
+      parts.src[k] = src[k];
+      parts.words[k] = bytes[k] / 4;
+      total += bytes[k];
+    } else {
+      GS_TRY(copy_out(dst[k], src[k], bytes[k], s));
+    }
+  }
+  if (total) {
+    k_export<<<(unsigned)std::min<size_t>((total / 4 + 1023) / 1024, sm_count() * 8), 256, 0, s>>>(
+        parts);
+    GS_LAUNCH();
+  }
   if (sim && A > 0) {
     Pool pool(s);
     const bool dev = is_device_ptr(sim);
