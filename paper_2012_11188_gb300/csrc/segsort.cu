@@ -11,8 +11,8 @@
 // Segments are classed by length: <= 32 (one warp, one element per lane,
 // bitonic network across lanes), <= 256, 512, 1024, 2048 and 4096 (one CTA
 // of 32 to 512 threads: 8-element register sorts, then merge-path levels in
-// shared memory), longer (a few of up to 16384 elements the same way by one
-// CTA each, else split into buckets by sample sort, below; past
+// shared memory), longer (up to 8192 elements the same way when there are many
+// of them, up to 16384 when few, else split into buckets by sample sort; past
 // three levels of splitting, 8192-element tiles sorted by one CTA the same
 // way, then merge-path passes over global memory that double the run length,
 // ping-ponging between the data and a scratch buffer).
@@ -24,8 +24,9 @@ namespace {
 
 constexpr int WTILE = 256;   // rows up to this length are sorted by a one-warp CTA
 constexpr int TILE = 8192;   // tiles of long segments (one CTA of 1024 threads each)
-constexpr int NCLASS = 7;    // <=32, <=256, <=512, <=1024, <=2048, <=4096, >4096
+constexpr int NCLASS = 8;    // <=32, <=256, <=512, <=1024, <=2048, <=4096, <=8192, >8192
 constexpr int LONGC = NCLASS - 1;  // the long class
+constexpr int EIGHTC = LONGC - 1;  // up to 8192: long as well where there are few
 
 // Segments as begin/end arrays: segment i is [b[i], e[i]). A contiguous
 // segmentation by offsets is {off, off + 1}; the buckets of long segments
@@ -56,7 +57,7 @@ constexpr int32_t SENT_V = 0x7fffffff;  // sorts after every real element (key 0
 // elements each), so that a segment keeps at least half of its CTA busy.
 __device__ __forceinline__ int seg_class(int64_t len) {
   return len <= 32 ? 0 : len <= WTILE ? 1 : len <= 512 ? 2 : len <= 1024 ? 3 : len <= 2048 ? 4
-       : len <= 4096 ? 5 : LONGC;
+       : len <= 4096 ? 5 : len <= 8192 ? 6 : LONGC;
 }
 
 // Count segments per class and number of tiles of long segments.
@@ -88,7 +89,7 @@ __global__ void k_classify_count(Segs S, int64_t nseg, int64_t total,
       const unsigned m = __ballot_sync(0xffffffffu, cl == k);
       if (lane == k) mine += __popc(m);
     }
-    if (cl == LONGC) {
+    if (cl >= EIGHTC) {
       atomicAdd(&c[NCLASS], (unsigned long long)((len + TILE - 1) / TILE));
       atomicMax(&c[NCLASS + 1], (unsigned long long)len);
     }
@@ -620,10 +621,8 @@ constexpr int TLONG_T = TILE / TLONG_RI;
 
 // Tiles per long segment (prefix computed by the caller).
 __global__ void k_long_tiles(Segs S, const int64_t* __restrict__ list,
-                             const unsigned long long* __restrict__ count_ptr,
-                             int64_t* __restrict__ tiles, int64_t* __restrict__ outchunks,
-                             int chunk) {
-  const int64_t cnt = (int64_t)*count_ptr;
+                             int64_t cnt, int64_t* __restrict__ tiles,
+                             int64_t* __restrict__ outchunks, int chunk) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t sg = list[i];
@@ -1286,7 +1285,14 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
   unsigned long long* fill = counts + NCNT;
   k_classify_fill<<<g_seg, 256, 0, s>>>(S, nseg, base_dev, fill, list);
   GS_LAUNCH();
-  const int64_t nlong = (int64_t)hc[LONGC];
+  // Segments of 4097 to 8192 elements are sorted by one CTA each when there
+  // are many of them: the split into buckets reads and writes every element
+  // twice more (dense graph of 25,825 vertices, rows of 5400: 27.0 ms per build
+  // with the split, 25.2 without). A few leave most multiprocessors idle for
+  // as long as one CTA takes (R-MAT s20: 1% slower), and count as long.
+  const bool eights = depth < BKT_DEPTH && hc[EIGHTC] >= 16ull * sm_count();
+  const int first_long = eights ? LONGC : EIGHTC;
+  const int64_t nlong = (int64_t)(hc[LONGC] + (eights ? 0 : hc[EIGHTC]));
   const int64_t max_long = (int64_t)hc[NCLASS + 1];
   // long segments are split into buckets, sorted one level down; below
   // BKT_DEPTH levels they take the tiles and merge passes
@@ -1296,11 +1302,11 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
     GS_CUDA(cudaFuncSetAttribute(k_sort_huge, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)HUGE_SMEM));
     k_sort_huge<<<(unsigned)nlong, HUGE_T, HUGE_SMEM, s>>>(ik, iv, key, val, S,
-                                                           list + base[LONGC], nlong);
+                                                           list + base[first_long], nlong);
     GS_LAUNCH();
   }
   if (bucketed)
-    GS_TRY(bucket_level(key, val, alt_k, alt_v, S, total, list + base[LONGC], nlong, in_alt, pool,
+    GS_TRY(bucket_level(key, val, alt_k, alt_v, S, total, list + base[first_long], nlong, in_alt, pool,
                         s, depth));
   // per-class counts on the device for the grid-stride kernels: counts[c]
   if (hc[0]) {
@@ -1348,8 +1354,16 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
         ik, iv, key, val, S, list + base[5], counts + 5, nullptr, 0, nullptr, nullptr, ascending);
     GS_LAUNCH();
   }
+  if (eights) {
+    GS_CUDA(cudaFuncSetAttribute(k_sort_tile<1024, 8, false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)tile_smem_bytes<1024, 8>()));
+    k_sort_tile<1024, 8, false><<<grid_of((int64_t)hc[EIGHTC], 1), 1024, tile_smem_bytes<1024, 8>(), s>>>(
+        ik, iv, key, val, S, list + base[EIGHTC], counts + EIGHTC, nullptr, 0, nullptr, nullptr, ascending);
+    GS_LAUNCH();
+  }
   if (nlong && !bucketed && !whole) {
-    const int64_t* llist = list + base[LONGC];
+    const int64_t* llist = list + base[first_long];
     if (in_alt) {  // the tiles and merge passes work in (key, val)
       k_copy_segments<<<grid_of(nlong, 1), 256, 0, s>>>(alt_k, alt_v, key, val, S, llist, nlong);
       GS_LAUNCH();
@@ -1361,7 +1375,7 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
     uint64_t* tk = pool.get<uint64_t>(total);
     int32_t* tv = pool.get<int32_t>(total);
     if (!tiles || !tile_prefix || !chunks || !chunk_prefix || !tk || !tv) return SCAN_ENOMEM;
-    k_long_tiles<<<grid_of(nlong, 256), 256, 0, s>>>(S, llist, counts + LONGC, tiles, chunks,
+    k_long_tiles<<<grid_of(nlong, 256), 256, 0, s>>>(S, llist, nlong, tiles, chunks,
                                                      MERGE_CHUNK);
     GS_LAUNCH();
     GS_TRY(exclusive_scan_i64(tiles, tile_prefix, nlong, pool, s));

@@ -39,9 +39,12 @@ def test_whole_segments(pattern, longest):
     check(keys, ids, lens)
 
 
-@pytest.mark.parametrize("count", [1, 100, 400])
+@pytest.mark.parametrize("count", [1, 100, 400, 3000])
 def test_counts_of_long_segments(count):
+    """Few enough for a CTA each, split into buckets, and so many that those
+    of up to 8192 are sorted by one CTA each again."""
     rng = np.random.default_rng(6)
-    lens = rng.integers(4097, 6000, count)
+    lens = rng.integers(4097, 8194, count)
+    lens[:3] = [8192, 8193, 4097][:count]
     total = int(lens.sum())
     check(rng.random(total), rng.permutation(total).astype(np.int32), lens)
