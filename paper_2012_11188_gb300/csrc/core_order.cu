@@ -243,17 +243,17 @@ int build_core_order_multi(int64_t N, int64_t A, const int64_t* off, const int32
     GS_CUDA(cudaMemsetAsync(co_off_all, 0, sizeof(int64_t), s));
     return SCAN_OK;
   }
-  int64_t* meta = pool.get<int64_t>(3 * (size_t)(G + 1));
-  unsigned long long* hist = pool.get<unsigned long long>(H);
-  unsigned long long* fill = pool.get<unsigned long long>(H);
-  int64_t* Sx = pool.get<int64_t>(H + 1);
-  int64_t* sizes = pool.get<int64_t>(S);
-  int64_t* qt = pool.get<int64_t>(G);
-  int64_t* qtb = pool.get<int64_t>(G + 1);
+  int64_t* meta = pool.tmp<int64_t>(3 * (size_t)(G + 1));
+  unsigned long long* hist = pool.tmp<unsigned long long>(H);
+  unsigned long long* fill = pool.tmp<unsigned long long>(H);
+  int64_t* Sx = pool.tmp<int64_t>(H + 1);
+  int64_t* sizes = pool.tmp<int64_t>(S);
+  int64_t* qt = pool.tmp<int64_t>(G);
+  int64_t* qtb = pool.tmp<int64_t>(G + 1);
   const int64_t Tub = N / 32 + G + 1;  // q-tiles upper bound
-  int64_t* rt = pool.get<int64_t>(Tub);
-  int64_t* rt_prefix = pool.get<int64_t>(Tub + 1);
-  int32_t* perm = pool.get<int32_t>(N > 0 ? N : 1);
+  int64_t* rt = pool.tmp<int64_t>(Tub);
+  int64_t* rt_prefix = pool.tmp<int64_t>(Tub + 1);
+  int32_t* perm = pool.tmp<int32_t>(N > 0 ? N : 1);
   if (!meta || !hist || !fill || !Sx || !sizes || !qt || !qtb || !rt || !rt_prefix || !perm)
     return SCAN_ENOMEM;
   std::vector<int64_t> hmeta(3 * (size_t)(G + 1));

@@ -469,37 +469,21 @@ bool dense_counts_pay(int64_t n, int64_t arcs, const CountCfg& cfg) {
 
 int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, const int32_t* deg,
                           int64_t n, int lsh_T, double* sim_csr, unsigned* status, Pool& pool,
-                          cudaStream_t s, float* count_ms) {
+                          cudaStream_t s, CountTimer* timer) {
   if (n > DENSE_MAX_N) return SCAN_EINVAL;
   if (n == 0) return SCAN_OK;
   const int64_t np = (n + DENSE_PAD - 1) / DENSE_PAD * DENSE_PAD;
   const int64_t nb = np / 128;
   const size_t nn = (size_t)np * (size_t)np;
   const std::vector<uint32_t> tiles = upper_tiles(np);
-  __nv_bfloat16* M = pool.get<__nv_bfloat16>(nn);
-  int64_t* bpos = pool.get<int64_t>((size_t)n * (size_t)(nb + 1));
-  uint32_t* tiles_d = pool.get<uint32_t>(tiles.size());
+  __nv_bfloat16* M = pool.tmp<__nv_bfloat16>(nn);
+  int64_t* bpos = pool.tmp<int64_t>((size_t)n * (size_t)(nb + 1));
+  uint32_t* tiles_d = pool.tmp<uint32_t>(tiles.size());
   if (!M || !bpos || !tiles_d) return SCAN_ENOMEM;
   CUtensorMap map_a, map_b;
   GS_TRY(encode_map(&map_a, M, np, BM));
   GS_TRY(encode_map(&map_b, M, np, BN));
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (count_ms) {
-    GS_CUDA(cudaEventCreate(&e0));
-    if (cudaEventCreate(&e1) != cudaSuccess) {
-      cudaEventDestroy(e0);
-      return SCAN_ECUDA;
-    }
-  }
-  // events are released on every return path
-  struct EvGuard {
-    cudaEvent_t a, b;
-    ~EvGuard() {
-      if (a) cudaEventDestroy(a);
-      if (b) cudaEventDestroy(b);
-    }
-  } guard{e0, e1};
-  if (e0) GS_CUDA(cudaEventRecord(e0, s));
+  if (timer) GS_TRY(CountTimer::mark(&timer->step[0], s));
   GS_CUDA(cudaMemcpyAsync(tiles_d, tiles.data(), tiles.size() * sizeof(uint32_t),
                           cudaMemcpyHostToDevice, s));
   GS_CUDA(cudaMemsetAsync(M, 0, nn * sizeof(__nv_bfloat16), s));
@@ -511,8 +495,7 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
   GS_LAUNCH();
   // the epilogue pairs every arc with its reverse: check symmetry first
   unsigned hst = 0;
-  GS_CUDA(cudaMemcpyAsync(&hst, status, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaStreamSynchronize(s));
+  GS_TRY(read_back(&hst, status, sizeof(hst), s));
   if (hst & DEV_BADGRAPH) return SCAN_EBADGRAPH;
   GS_CUDA(cudaFuncSetAttribute(k_dense_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)SMEM_BYTES));
@@ -521,11 +504,7 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
   const unsigned mgrid = (unsigned)std::min<int64_t>((int64_t)tiles.size(), sm_count());
   k_dense_mma<<<mgrid, THREADS, SMEM_BYTES, s>>>(map_a, map_b, da);
   GS_LAUNCH();
-  if (e1) {
-    GS_CUDA(cudaEventRecord(e1, s));
-    GS_CUDA(cudaEventSynchronize(e1));
-    GS_CUDA(cudaEventElapsedTime(count_ms, e0, e1));
-  }
+  if (timer) GS_TRY(CountTimer::mark(&timer->step[1], s));
   pool.put(M);
   pool.put(bpos);
   pool.put(tiles_d);

@@ -84,8 +84,8 @@ int scan_impl(const T* in, int64_t* out, int64_t n, Pool& pool, cudaStream_t s) 
     GS_LAUNCH();
     return SCAN_OK;
   }
-  int64_t* sums = pool.get<int64_t>(tiles);
-  int64_t* base = pool.get<int64_t>(tiles + 1);
+  int64_t* sums = pool.tmp<int64_t>(tiles);
+  int64_t* base = pool.tmp<int64_t>(tiles + 1);
   if (!sums || !base) return SCAN_ENOMEM;
   k_tile_sums<T><<<(unsigned)tiles, SCAN_T, 0, s>>>(in, n, sums);
   GS_LAUNCH();
@@ -114,7 +114,7 @@ k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int32_t local_max = 0;
-  unsigned bad = 0;
+  unsigned bad = warp == 0 && (off[0] != 0 || off[n] != arcs) ? 1 : 0;
   for (int64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
     const int64_t v = v0 + lane;
     int64_t b = 0, e = 0;
@@ -202,9 +202,10 @@ k_orient_inplace(const int64_t* __restrict__ off, const int32_t* __restrict__ ad
                  int32_t* __restrict__ od, int32_t* __restrict__ oadj,
                  int32_t* __restrict__ opos, int32_t* max_od,
                  unsigned long long* sum_od, int32_t* __restrict__ long_rows,
-                 unsigned* __restrict__ n_long) {
+                 unsigned* __restrict__ n_long, const unsigned* __restrict__ status) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ int scratch[8][64];
+  if (*status & DEV_BADGRAPH) return;  // ids may be out of range
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;  // lanes below this one
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -347,8 +348,8 @@ int launch_degrees(const int64_t* off, const int32_t* adj, int64_t n, int64_t ar
                    int32_t* maxdeg_dev, unsigned* status, Pool& pool, cudaStream_t s) {
   if (n == 0) return SCAN_OK;
   const int64_t max_long = arcs / DEG_LONG + 1;
-  int32_t* long_rows = pool.get<int32_t>(max_long);
-  unsigned* n_long = pool.get<unsigned>(1);
+  int32_t* long_rows = pool.tmp<int32_t>(max_long);
+  unsigned* n_long = pool.tmp<unsigned>(1);
   if (!long_rows || !n_long) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(n_long, 0, sizeof(unsigned), s));
   k_degrees<<<grid_for(n, 256), 256, 0, s>>>(off, adj, n, arcs, deg, maxdeg_dev, status, long_rows,
@@ -365,19 +366,19 @@ int launch_degrees(const int64_t* off, const int32_t* adj, int64_t n, int64_t ar
 int launch_orient(const int64_t* off, const int32_t* adj, const int32_t* deg, int64_t n,
                   int64_t arcs, Pool& pool, int32_t** od_out, int32_t** oadj_out,
                   int32_t** opos_out, int32_t* max_od_dev, unsigned long long* sum_od_dev,
-                  cudaStream_t s) {
-  int32_t* od = pool.get<int32_t>(n > 0 ? n : 1);
-  int32_t* oadj = pool.get<int32_t>(arcs > 0 ? arcs : 1);
-  int32_t* opos = pool.get<int32_t>(arcs > 0 ? arcs : 1);
+                  const unsigned* status, cudaStream_t s) {
+  int32_t* od = pool.tmp<int32_t>(n > 0 ? n : 1);
+  int32_t* oadj = pool.tmp<int32_t>(arcs > 0 ? arcs : 1);
+  int32_t* opos = pool.tmp<int32_t>(arcs > 0 ? arcs : 1);
   // rows longer than LONG_ROW: at most arcs / LONG_ROW of them
   const int64_t max_long = arcs / LONG_ROW + 1;
-  int32_t* long_rows = pool.get<int32_t>(max_long);
-  unsigned* n_long = pool.get<unsigned>(1);
+  int32_t* long_rows = pool.tmp<int32_t>(max_long);
+  unsigned* n_long = pool.tmp<unsigned>(1);
   if (!od || !oadj || !opos || !long_rows || !n_long) return SCAN_ENOMEM;
   if (n > 0) {
     GS_CUDA(cudaMemsetAsync(n_long, 0, sizeof(unsigned), s));
     k_orient_inplace<<<grid_for(n, 256), 256, 0, s>>>(off, adj, deg, n, od, oadj, opos, max_od_dev,
-                                                    sum_od_dev, long_rows, n_long);
+                                                    sum_od_dev, long_rows, n_long, status);
     GS_LAUNCH();
     k_orient_long<<<(unsigned)std::min<int64_t>(max_long, sm_count() * 2), LONG_T, 0, s>>>(
         off, adj, deg, long_rows, n_long, od, oadj, opos, max_od_dev, sum_od_dev);

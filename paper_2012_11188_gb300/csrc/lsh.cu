@@ -555,8 +555,8 @@ int launch_sims(const int64_t* off, const int32_t* adj, const int32_t* row, cons
 
 int lsh_select(const int64_t* off, const int32_t* adj, const int32_t* deg, int64_t n, int T,
                int32_t* row, int64_t* nH_host, Pool& pool, cudaStream_t s) {
-  int32_t* flag = pool.get<int32_t>(n > 0 ? n : 1);
-  int64_t* pre = pool.get<int64_t>(n + 1);
+  int32_t* flag = pool.tmp<int32_t>(n > 0 ? n : 1);
+  int64_t* pre = pool.tmp<int64_t>(n + 1);
   if (!flag || !pre) return SCAN_ENOMEM;
   if (n > 0) {
     k_select_flags<<<(unsigned)std::min<int64_t>((n + 7) / 8, sm_count() * 32), 256, 0, s>>>(off, adj, deg,
@@ -581,9 +581,9 @@ int lsh_apply(const scan_lsh_params& p, int kind, const int64_t* off, const int3
               double* sim_csr, Pool& pool, cudaStream_t s, const double* wcsr) {
   (void)arcs;
   if (nH <= 0) return SCAN_OK;
-  int32_t* hlist = pool.get<int32_t>(nH);
-  int32_t* pieces = pool.get<int32_t>(nH);
-  int64_t* ipre = pool.get<int64_t>(nH + 1);
+  int32_t* hlist = pool.tmp<int32_t>(nH);
+  int32_t* pieces = pool.tmp<int32_t>(nH);
+  int64_t* ipre = pool.tmp<int64_t>(nH + 1);
   if (!hlist || !pieces || !ipre) return SCAN_ENOMEM;
   k_hlist<<<(unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 32), 256, 0, s>>>(
       row, deg, n, hlist, pieces);
@@ -593,8 +593,8 @@ int lsh_apply(const scan_lsh_params& p, int kind, const int64_t* off, const int3
   if (kind == SCAN_COSINE) {
     const int k = p.simhash_bits, W = k / 64;
     const uint64_t key = mix64(p.seed ^ 0x53494D48ULL);  // "SIMH"
-    uint64_t* sig = pool.get<uint64_t>((size_t)nH * W);
-    double* tab = pool.get<double>((size_t)k + 1);
+    uint64_t* sig = pool.tmp<uint64_t>((size_t)nH * W);
+    double* tab = pool.tmp<double>((size_t)k + 1);
     if (!sig || !tab) return SCAN_ENOMEM;
     std::vector<double> htab((size_t)k + 1);
     for (int h = 0; h <= k; ++h) {
@@ -628,7 +628,7 @@ int lsh_apply(const scan_lsh_params& p, int kind, const int64_t* off, const int3
     int L = 0;
     while ((1 << L) < k) ++L;
     const uint64_t key = mix64(p.seed ^ 0x4D494E48ULL);  // "MINH"
-    uint32_t* mh = pool.get<uint32_t>((size_t)nH * k);
+    uint32_t* mh = pool.tmp<uint32_t>((size_t)nH * k);
     if (!mh) return SCAN_ENOMEM;
     k_minhash<<<gh, 256, 0, s>>>(off, adj, hlist, nH, k, L, p.minhash_kpartition, key, mh);
     GS_LAUNCH();

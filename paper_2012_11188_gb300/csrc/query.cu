@@ -35,8 +35,6 @@
 // R-MAT s22 1.78 -> 1.41 ms, 594 pairs of a sweep on R-MAT s20 438 -> 72 ms.
 #include <cooperative_groups.h>
 
-#include <mutex>
-
 #include "scan_internal.cuh"
 
 namespace gscan {
@@ -467,39 +465,6 @@ k_query_one(QArgs a, int mu, double eps, int hubs) {
   phase_hubs(a, a.labels, t0 >> 5, nt >> 5);
 }
 
-// Words of pinned host memory that kernels write their status to: one page
-// for the process, words handed out and taken back under a lock.
-constexpr int STATUS_WORDS = 256;
-std::mutex g_word_mu;
-unsigned* g_words = nullptr;
-bool g_word_used[STATUS_WORDS];
-
-struct HostWord {
-  unsigned* p = nullptr;
-  HostWord() {
-    std::lock_guard<std::mutex> lk(g_word_mu);
-    if (!g_words &&
-        cudaHostAlloc((void**)&g_words, STATUS_WORDS * sizeof(unsigned),
-                      cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-      cudaGetLastError();
-      g_words = nullptr;
-      return;
-    }
-    for (int i = 0; i < STATUS_WORDS; ++i)
-      if (!g_word_used[i]) {
-        g_word_used[i] = true;
-        p = g_words + i;
-        *p = 0;
-        return;
-      }
-  }
-  ~HostWord() {
-    if (!p) return;
-    std::lock_guard<std::mutex> lk(g_word_mu);
-    g_word_used[p - g_words] = false;
-  }
-};
-
 // Resident CTAs of k_query_one per multiprocessor (0: no cooperative launch).
 int query_one_per_sm() {
   static std::atomic<int> cached[64];  // 1 + the value, zero until looked up
@@ -582,8 +547,10 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   *done = false;
   const int64_t n = ix.n;
   const int per_sm = query_one_per_sm();
-  HostWord status;
-  if (per_sm == 0 || !status.p) return SCAN_OK;
+  PinnedSlot slot;  // the kernel's status word
+  unsigned* status = static_cast<unsigned*>(slot.p);
+  if (per_sm == 0 || !status) return SCAN_OK;
+  *status = 0;
   const size_t qb = query_queue_bytes(ix, 1);
   const size_t head = ((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255;
   char* scratch = pool.get<char>(head + (qb ? qb : 16));
@@ -592,7 +559,7 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   int32_t* parent = reinterpret_cast<int32_t*>(scratch);
   unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + head);
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
-          n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status.p,
+          n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status,
           qb ? reinterpret_cast<QPiece*>(scratch + head + 16) : nullptr, queued,
           queue_capacity(ix, 1)};
   // a warp per core at most, and no more CTAs than are resident at once
@@ -606,7 +573,7 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
     GS_CUDA(cudaMemcpyAsync(host_labels, labels, (size_t)n * sizeof(int32_t),
                             cudaMemcpyDeviceToHost, s));
   GS_CUDA(cudaStreamSynchronize(s));
-  if (*(volatile unsigned*)status.p & DEV_LIMIT) return SCAN_ETIMEOUT;
+  if (*(volatile unsigned*)status & DEV_LIMIT) return SCAN_ETIMEOUT;
   return SCAN_OK;
 }
 

@@ -102,6 +102,44 @@ void dev_free(void* p, size_t bytes, cudaStream_t s) {
   cudaFreeAsync(p, s);
 }
 
+namespace {
+constexpr int PINNED_SLOTS = 64;
+std::mutex g_slot_mu;
+char* g_slots = nullptr;
+bool g_slot_used[PINNED_SLOTS];
+}  // namespace
+
+PinnedSlot::PinnedSlot() {
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  if (!g_slots && cudaHostAlloc((void**)&g_slots, PINNED_SLOTS * BYTES,
+                                cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    g_slots = nullptr;
+    return;
+  }
+  for (int i = 0; i < PINNED_SLOTS; ++i)
+    if (!g_slot_used[i]) {
+      g_slot_used[i] = true;
+      p = g_slots + i * BYTES;
+      return;
+    }
+}
+
+PinnedSlot::~PinnedSlot() {
+  if (!p) return;
+  std::lock_guard<std::mutex> lk(g_slot_mu);
+  g_slot_used[((char*)p - g_slots) / BYTES] = false;
+}
+
+int read_back(void* dst, const void* src_dev, size_t bytes, cudaStream_t s) {
+  PinnedSlot slot;
+  void* to = slot.p && bytes <= PinnedSlot::BYTES ? slot.p : dst;
+  GS_CUDA(cudaMemcpyAsync(to, src_dev, bytes, cudaMemcpyDeviceToHost, s));
+  GS_CUDA(cudaStreamSynchronize(s));
+  if (to != dst) std::memcpy(dst, to, bytes);
+  return SCAN_OK;
+}
+
 void record_kernel_ms(double ms) { g_timings[7] = ms; }
 
 void record_timings(const double* ms7) {
@@ -208,39 +246,35 @@ int validate_lsh(const scan_lsh_params* p, int kind) {
 // ix holds n, arcs, off (absolute, int64), adj and allocated deg, no_id,
 // no_sim and an 8-word status block; on return ix->maxdeg is set.
 int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool, cudaStream_t s,
-                 Events& ev, float* count_ms, int counts_mode, const CountCfg& cfg,
+                 Events& ev, CountTimer& timer, int counts_mode, const CountCfg& cfg,
                  const double* wcsr = nullptr) {
   const int64_t n = ix->n, arcs = ix->arcs;
   const bool use_lsh = lsh && lsh->enabled;
   unsigned* scalars = ix->status;  // [0] status, [1] maxdeg, [2] max out-degree
   GS_TRY(launch_degrees(ix->off, ix->adj, n, arcs, ix->deg, (int32_t*)scalars + 1, scalars, pool,
                         s));
-  unsigned hs[4];
-  GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaStreamSynchronize(s));
-  if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
-  ix->maxdeg = (int32_t)hs[1];
   // weighted similarities take the sparse enumeration only
   const bool dense = arcs > 0 && !wcsr && (counts_mode == SCAN_COUNTS_DENSE ||
                                   (counts_mode == SCAN_COUNTS_AUTO && dense_counts_pay(n, arcs, cfg)));
+  unsigned hs[8];  // status, maximum degree, maximum out-degree, -, out-arcs (2 words)
   if (dense) {
+    GS_TRY(read_back(hs, scalars, sizeof(hs), s));
+    if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
+    ix->maxdeg = (int32_t)hs[1];
     // closed counts of every arc from one matrix product (Section 4.1.1)
     if (n > DENSE_MAX_N) return SCAN_EINVAL;
     GS_TRY(ev.mark(s));
     int32_t* row = nullptr;
     int64_t nH = 0;
     if (use_lsh) {
-      row = pool.get<int32_t>(n);
+      row = pool.tmp<int32_t>(n);
       if (!row) return SCAN_ENOMEM;
       GS_TRY(lsh_select(ix->off, ix->adj, ix->deg, n, lsh->degree_threshold, row, &nH, pool, s));
     }
     GS_CUDA(cudaMemcpyAsync(ix->no_id, ix->adj, arcs * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     GS_TRY(dense_counts_and_sims(kind, ix->off, ix->adj, ix->deg, n,
                                  use_lsh ? lsh->degree_threshold : -1, ix->no_sim, scalars, pool,
-                                 s, count_ms));
-    GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    GS_CUDA(cudaStreamSynchronize(s));
-    if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
+                                 s, &timer));
     GS_TRY(ev.mark(s));
     if (use_lsh && nH > 0)
       GS_TRY(lsh_apply(*lsh, kind, ix->off, ix->adj, ix->deg, n, arcs, row, nH, ix->no_sim, pool, s));
@@ -253,24 +287,22 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
   }
   // ---- orientation (Section 6.1)
   int32_t *od = nullptr, *oadj = nullptr, *opos = nullptr;
-  if (arcs > 0) {
-    unsigned long long* sum_od = (unsigned long long*)(scalars + 4);
+  if (arcs > 0)
     GS_TRY(launch_orient(ix->off, ix->adj, ix->deg, n, arcs, pool, &od, &oadj, &opos,
-                         (int32_t*)scalars + 2, sum_od, s));
-    unsigned long long hsum = 0;
-    GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    GS_CUDA(cudaMemcpyAsync(&hsum, sum_od, sizeof(hsum), cudaMemcpyDeviceToHost, s));
-    GS_CUDA(cudaStreamSynchronize(s));
-    // a symmetric graph orients exactly arcs/2 edges
-    if ((int64_t)hsum != arcs / 2) return SCAN_EBADGRAPH;
-  }
+                         (int32_t*)scalars + 2, (unsigned long long*)(scalars + 4), scalars, s));
+  // one wait for the checks and the orientation (which leaves a bad graph alone)
+  GS_TRY(read_back(hs, scalars, sizeof(hs), s));
+  if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
+  ix->maxdeg = (int32_t)hs[1];
+  // a symmetric graph orients exactly arcs/2 edges
+  if (arcs > 0 && (int64_t)((uint64_t)hs[5] << 32 | hs[4]) != arcs / 2) return SCAN_EBADGRAPH;
   const int32_t max_od = (int32_t)hs[2];
   GS_TRY(ev.mark(s));
   // ---- LSH selection (Section 6.3)
   int32_t* row = nullptr;
   int64_t nH = 0;
   if (use_lsh && arcs > 0) {
-    row = pool.get<int32_t>(n);
+    row = pool.tmp<int32_t>(n);
     if (!row) return SCAN_ENOMEM;
     GS_TRY(lsh_select(ix->off, ix->adj, ix->deg, n, lsh->degree_threshold, row, &nH, pool, s));
   }
@@ -279,11 +311,9 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
     GS_CUDA(cudaMemcpyAsync(ix->no_id, ix->adj, arcs * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
     GS_TRY(launch_closed_counts_and_sims(kind, ix->off, ix->adj, ix->deg, n, arcs, od, oadj, opos,
                                          ix->maxdeg, max_od, use_lsh ? lsh->degree_threshold : -1,
-                                         wcsr, ix->no_sim, scalars, pool, s, count_ms, cfg));
-    GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
-    GS_CUDA(cudaStreamSynchronize(s));
-    if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
-    if (hs[0] & DEV_BADWEIGHT) return SCAN_EINVAL;
+                                         wcsr, ix->no_sim, scalars, pool, s, &timer, cfg));
+    // (what the counting finds wrong is read with the build's final status:
+    // the sorts take any bits for keys)
     pool.put(od);
     pool.put(oadj);
     pool.put(opos);
@@ -301,8 +331,10 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
   return SCAN_OK;
 }
 
-void store_timings(Events& ev, float count_ms) {
+void store_timings(Events& ev, const CountTimer& timer) {
   double t[7];
+  const float count_ms = CountTimer::ms(timer.step);
+  if (timer.step[0]) record_kernel_ms(CountTimer::ms(timer.kernel));
   t[0] = ev.ms(0, 1);
   t[1] = count_ms;
   t[2] = ev.ms(1, 2) - count_ms;
@@ -314,11 +346,11 @@ void store_timings(Events& ev, float count_ms) {
 }
 
 int check_final_status(const unsigned* scalars, cudaStream_t s) {
-  unsigned hs[4];
-  GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaStreamSynchronize(s));
-  if (hs[0] & DEV_BADGRAPH) return SCAN_EBADGRAPH;
-  if (hs[0] & DEV_LIMIT) return SCAN_ETIMEOUT;
+  unsigned hs = 0;
+  GS_TRY(read_back(&hs, scalars, sizeof(hs), s));
+  if (hs & DEV_BADGRAPH) return SCAN_EBADGRAPH;
+  if (hs & DEV_BADWEIGHT) return SCAN_EINVAL;
+  if (hs & DEV_LIMIT) return SCAN_ETIMEOUT;
   return SCAN_OK;
 }
 
@@ -360,41 +392,42 @@ int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStr
   // ---- inputs into the index's own arrays
   const bool dev_in = csr->on_device != 0;
   const cudaMemcpyKind k_in = dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  std::vector<int64_t> off_host;
   if (csr->offsets_64) {
     GS_CUDA(cudaMemcpyAsync(ix->off, csr->offsets, (n + 1) * sizeof(int64_t), k_in, s));
-  } else if (dev_in) {
-    k_off32_to_64<<<(unsigned)std::min<int64_t>((n + 256) / 256, 4096), 256, 0, s>>>(
-        (const int32_t*)csr->offsets, n + 1, ix->off);
-    GS_LAUNCH();
   } else {
-    off_host.resize(n + 1);
     const int32_t* o32 = (const int32_t*)csr->offsets;
-    for (int64_t i = 0; i <= n; ++i) off_host[i] = o32[i];
-    GS_CUDA(cudaMemcpyAsync(ix->off, off_host.data(), (n + 1) * sizeof(int64_t),
-                            cudaMemcpyHostToDevice, s));
+    if (!dev_in) {
+      int32_t* d32 = pool.tmp<int32_t>(n + 1);
+      if (!d32) return SCAN_ENOMEM;
+      GS_CUDA(cudaMemcpyAsync(d32, csr->offsets, (n + 1) * sizeof(int32_t), k_in, s));
+      o32 = d32;
+    }
+    k_off32_to_64<<<(unsigned)std::min<int64_t>((n + 256) / 256, 4096), 256, 0, s>>>(o32, n + 1,
+                                                                                    ix->off);
+    GS_LAUNCH();
+    if (!dev_in) pool.put(const_cast<int32_t*>(o32));
   }
   if (arcs > 0) GS_CUDA(cudaMemcpyAsync(ix->adj, csr->adj, arcs * sizeof(int32_t), k_in, s));
   double* wcsr = nullptr;  // arc weights, released with the build's scratch
   if (weights && arcs > 0) {
-    wcsr = pool.get<double>(arcs);
+    wcsr = pool.tmp<double>(arcs);
     if (!wcsr) return SCAN_ENOMEM;
     GS_CUDA(cudaMemcpyAsync(wcsr, weights, arcs * sizeof(double), k_in, s));
   }
-  int64_t ends[2] = {0, 0};
-  GS_CUDA(cudaMemcpyAsync(&ends[0], ix->off, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaMemcpyAsync(&ends[1], ix->off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaStreamSynchronize(s));
-  if (ends[0] != 0 || ends[1] != arcs) return SCAN_EBADGRAPH;
-  float count_ms = 0;
+  if (n == 0) {  // (with vertices, the degree pass checks the first and last offset)
+    int64_t end = 0;
+    GS_TRY(read_back(&end, ix->off, sizeof(end), s));
+    if (end != 0 || arcs != 0) return SCAN_EBADGRAPH;
+  }
+  CountTimer timer;
   const CountCfg cfg = cfg_in ? *cfg_in : count_config_for(n, n, arcs);
-  GS_TRY(run_pipeline(ix, kind, lsh, pool, s, ev, &count_ms, counts_mode, cfg, wcsr));
+  GS_TRY(run_pipeline(ix, kind, lsh, pool, s, ev, timer, counts_mode, cfg, wcsr));
   if (wcsr) pool.put(wcsr);
   // ---- core order (Algorithm 2)
   GS_TRY(build_core_order(*ix, pool, s));
   GS_TRY(ev.mark(s));
   GS_TRY(check_final_status(ix->status, s));
-  store_timings(ev, count_ms);
+  store_timings(ev, timer);
   ix->blocks = pool.detach();
   ix->bytes = 0;
   for (auto& b : ix->blocks) ix->bytes += b.b;
@@ -554,8 +587,8 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   u.no_id = pool.get<int32_t>(A > 0 ? A : 1);
   u.no_sim = pool.get<double>(A > 0 ? A : 1);
   u.status = pool.get<unsigned>(8);
-  int64_t* meta = pool.get<int64_t>(2 * (size_t)(G + 1));
-  PackSrc* d_src = pool.get<PackSrc>(G);
+  int64_t* meta = pool.tmp<int64_t>(2 * (size_t)(G + 1));
+  PackSrc* d_src = pool.tmp<PackSrc>(G);
   if (!u.off || !u.deg || !u.adj || !u.no_id || !u.no_sim || !u.status || !meta || !d_src)
     return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(u.status, 0, 8 * sizeof(unsigned), s));
@@ -578,7 +611,7 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
                 (c.num_arcs > 0 && !kernel_reads(c.adj, 4));
     if (staged[g]) staged_n += c.n + 1;
   }
-  char* staged_off = staged_n ? (char*)pool.get<int64_t>(staged_n) : nullptr;
+  char* staged_off = staged_n ? (char*)pool.tmp<int64_t>(staged_n) : nullptr;
   if (staged_n && !staged_off) return SCAN_ENOMEM;
   char* at = staged_off;
   for (int g = 0; g < G; ++g) {
@@ -608,10 +641,10 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   if (staged_off) pool.put(staged_off);
   pool.put(d_src);
   // ---- the shared pipeline over the union (every step is local to a vertex)
-  float count_ms = 0;
-  GS_TRY(run_pipeline(&u, kind, lsh, pool, s, ev, &count_ms, SCAN_COUNTS_SPARSE, cfg));
+  CountTimer timer;
+  GS_TRY(run_pipeline(&u, kind, lsh, pool, s, ev, timer, SCAN_COUNTS_SPARSE, cfg));
   // ---- per-graph core orders
-  int32_t* md_dev = pool.get<int32_t>(G);
+  int32_t* md_dev = pool.tmp<int32_t>(G);
   if (!md_dev) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(md_dev, 0, G * 4, s));
   k_graph_maxdeg<<<gN, 256, 0, s>>>(u.deg, d_vb, G, N, md_dev);
@@ -627,12 +660,12 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
     cb[g + 1] = cb[g] + md[g] + 1;
   }
   const int64_t S = sb[G];
-  int64_t* co_off_all = pool.get<int64_t>(S + 1);
+  int64_t* co_off_all = pool.tmp<int64_t>(S + 1);
   int32_t* co_id = pool.get<int32_t>(A > 0 ? A : 1);
   double* co_thr = pool.get<double>(A > 0 ? A : 1);
   int64_t* off_rel = pool.get<int64_t>(N + G);
   int64_t* co_off_rel = pool.get<int64_t>(S + G);
-  int64_t* meta2 = pool.get<int64_t>(4 * (size_t)(G + 1));
+  int64_t* meta2 = pool.tmp<int64_t>(4 * (size_t)(G + 1));
   if (!co_off_all || !co_id || !co_thr || !off_rel || !co_off_rel || !meta2) return SCAN_ENOMEM;
   GS_TRY(build_core_order_multi(N, A, u.off, u.deg, (const uint64_t*)u.no_sim, vb, md, co_off_all,
                                 co_id, (uint64_t*)co_thr, pool, s));
@@ -655,7 +688,7 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
                                       S + G, co_off_rel);
   GS_LAUNCH();
   GS_TRY(check_final_status(u.status, s));
-  store_timings(ev, count_ms);
+  store_timings(ev, timer);
   pool.put(co_off_all);
   pool.put(u.off);
   pool.put(meta2);
@@ -1204,7 +1237,7 @@ int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end
   int32_t *od = nullptr, *oadj = nullptr, *opos = nullptr;
   unsigned long long* sum_od = (unsigned long long*)(scalars + 4);
   GS_TRY(gscan::launch_orient(off, adj, deg, n, arcs, pool, &od, &oadj, &opos,
-                              (int32_t*)scalars + 2, sum_od, s));
+                              (int32_t*)scalars + 2, sum_od, scalars, s));
   unsigned long long hsum = 0;
   GS_CUDA(cudaMemcpyAsync(hs, scalars, sizeof(hs), cudaMemcpyDeviceToHost, s));
   GS_CUDA(cudaMemcpyAsync(&hsum, sum_od, sizeof(hsum), cudaMemcpyDeviceToHost, s));

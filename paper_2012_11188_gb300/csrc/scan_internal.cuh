@@ -48,6 +48,48 @@ enum : unsigned {
   DEV_BADWEIGHT = 8u,  // a weight negative, not finite, or not symmetric
 };
 
+// ------------------------------------------------------------ pinned host words
+// A slot of pinned host memory that the device writes directly (one page for
+// the process, slots handed out and taken back under a lock); p is null when
+// none is left.
+struct PinnedSlot {
+  static constexpr size_t BYTES = 256;
+  void* p = nullptr;
+  PinnedSlot();
+  ~PinnedSlot();
+  PinnedSlot(const PinnedSlot&) = delete;
+  PinnedSlot& operator=(const PinnedSlot&) = delete;
+};
+
+// Waits for s and returns `bytes` (at most PinnedSlot::BYTES) of device memory.
+int read_back(void* dst, const void* src_dev, size_t bytes, cudaStream_t s);
+
+// Events around a build's counting step and its CTA kernels; read once the
+// build has finished, so that the host does not wait in the middle of it.
+struct CountTimer {
+  cudaEvent_t step[2] = {}, kernel[2] = {};
+  CountTimer() = default;
+  CountTimer(const CountTimer&) = delete;
+  CountTimer& operator=(const CountTimer&) = delete;
+  ~CountTimer() {
+    for (cudaEvent_t e : {step[0], step[1], kernel[0], kernel[1]})
+      if (e) cudaEventDestroy(e);
+  }
+  static int mark(cudaEvent_t* e, cudaStream_t s) {
+    if (!*e) GS_CUDA(cudaEventCreate(e));
+    GS_CUDA(cudaEventRecord(*e, s));
+    return SCAN_OK;
+  }
+  static float ms(const cudaEvent_t (&e)[2]) {
+    float t = 0;
+    if (e[0] && e[1] && cudaEventElapsedTime(&t, e[0], e[1]) != cudaSuccess) {
+      cudaGetLastError();
+      t = 0;
+    }
+    return t;
+  }
+};
+
 // ------------------------------------------------------------ device memory
 // All device allocations go through the installed hooks (or the stream-ordered
 // CUDA allocator). A Pool remembers what it handed out so a failed build can
@@ -55,10 +97,20 @@ enum : unsigned {
 void* dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void* p, size_t bytes, cudaStream_t s);
 
+//
+// tmp() is for scratch of one call: small requests are carved from slabs that
+// the Pool keeps until it ends (a build makes some 60 to 130 of them, and an
+// allocation and a release in stream order cost the host about 3 us together:
+// with the fewer waits for results below, an SBM graph of 10k vertices
+// 0.70 -> 0.61 ms), larger ones are blocks of their own. put() gives a block back
+// and leaves a slab piece where it is. What detach() hands over is get()'s.
 struct Pool {
   cudaStream_t s;
   struct Blk { void* p; size_t b; };
   std::vector<Blk> blocks;
+  static constexpr size_t TMP_BYTES = 256u << 10, SLAB = 4u << 20;
+  std::vector<void*> slabs;
+  size_t slab_used = SLAB;
   explicit Pool(cudaStream_t st) : s(st) {}
   ~Pool() { release_all(); }
   template <class T>
@@ -78,9 +130,26 @@ struct Pool {
         return;
       }
   }
+  template <class T>
+  T* tmp(size_t count) {
+    const size_t b = (count * sizeof(T) + 255) / 256 * 256;
+    if (b > TMP_BYTES) return get<T>(count);
+    if (slab_used + b > SLAB) {
+      void* p = dev_alloc(SLAB, s);
+      if (!p) return get<T>(count);
+      slabs.push_back(p);
+      slab_used = 0;
+    }
+    char* p = (char*)slabs.back() + slab_used;
+    slab_used += b > 0 ? b : 256;
+    return (T*)p;
+  }
   void release_all() {
     for (auto& b : blocks) dev_free(b.p, b.b, s);
     blocks.clear();
+    for (void* p : slabs) dev_free(p, SLAB, s);
+    slabs.clear();
+    slab_used = SLAB;
   }
   // hand ownership of every block to the caller (the index)
   std::vector<Blk> detach() {
@@ -173,7 +242,8 @@ struct IndexData {
 // ------------------------------------------------------------ kernels' host launchers
 // Each returns a scan_status; all work is enqueued on `s`.
 
-// Degrees, CSR checks (sorted, in range, no self-loops), max degree.
+// Degrees, CSR checks (sorted, in range, no self-loops, offsets from 0 to
+// arcs), max degree.
 int launch_degrees(const int64_t* off, const int32_t* adj, int64_t n, int64_t arcs, int32_t* deg,
                    int32_t* maxdeg_dev, unsigned* status, Pool& pool, cudaStream_t s);
 
@@ -182,9 +252,11 @@ int launch_degrees(const int64_t* off, const int32_t* adj, int64_t n, int64_t ar
 // oadj[off[v]+od[v] .. off[v+1]), in descending id order; opos = position of
 // each arc inside v's CSR row.
 // max_od_dev receives the largest out-degree, sum_od_dev the number of out-arcs.
+// With DEV_BADGRAPH set in *status (device) by then, nothing is touched.
 int launch_orient(const int64_t* off, const int32_t* adj, const int32_t* deg, int64_t n,
                   int64_t arcs, Pool& pool, int32_t** od, int32_t** oadj, int32_t** opos,
-                  int32_t* max_od_dev, unsigned long long* sum_od_dev, cudaStream_t s);
+                  int32_t* max_od_dev, unsigned long long* sum_od_dev, const unsigned* status,
+                  cudaStream_t s);
 
 // Counting strategy per degree bucket (a tuning point): a graph of at least
 // dense_min_n vertices with dense_div * arcs >= n^2 takes the dense GEMM
@@ -218,7 +290,7 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
                                   const int32_t* deg, int64_t n, int64_t arcs, const int32_t* od,
                                   int32_t* oadj, int32_t* opos, int32_t maxdeg,
                                   int32_t max_od, int lsh_T, const double* wcsr, double* sim_csr,
-                                  unsigned* status, Pool& pool, cudaStream_t s, float* count_ms,
+                                  unsigned* status, Pool& pool, cudaStream_t s, CountTimer* timer,
                                   const CountCfg& cfg, int64_t v0 = 0, int64_t v1 = -1,
                                   uint32_t* counts_out = nullptr);
 
@@ -248,7 +320,7 @@ constexpr int64_t DENSE_MAX_N = 65536;
 bool dense_counts_pay(int64_t n, int64_t arcs, const CountCfg& cfg);
 int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, const int32_t* deg,
                           int64_t n, int lsh_T, double* sim_csr, unsigned* status, Pool& pool,
-                          cudaStream_t s, float* count_ms);
+                          cudaStream_t s, CountTimer* timer);
 
 // Queries (Algorithms 3-5). status_dev: a zeroed device word that receives
 // DEV_LIMIT if a bounded union-find loop gave up.

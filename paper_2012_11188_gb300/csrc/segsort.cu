@@ -1178,8 +1178,8 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
                  cudaStream_t s, int depth) {
   const bool own_alt = alt_k == nullptr;
   if (own_alt) {
-    alt_k = pool.get<uint64_t>(total);
-    alt_v = pool.get<int32_t>(total);
+    alt_k = pool.tmp<uint64_t>(total);
+    alt_v = pool.tmp<int32_t>(total);
     if (!alt_k || !alt_v) return SCAN_ENOMEM;
   }
   const uint64_t* ck = in_alt ? alt_k : key;  // where the data is
@@ -1191,14 +1191,14 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
   const int64_t B_ub = std::min<int64_t>(total / BKT_TARGET + 2 * nlong, nlong * BKT_FAN);
   const int64_t S_ub = B_ub * BKT_OS;
   const int64_t G_ub = total / ((int64_t)BKT_CH * BKT_G) + nlong;
-  int64_t* nb = pool.get<int64_t>(nlong);
-  int64_t* ns = pool.get<int64_t>(nlong);
-  int64_t* ngr = pool.get<int64_t>(nlong);
-  int64_t* boff = pool.get<int64_t>(nlong + 1);
-  int64_t* soff = pool.get<int64_t>(nlong + 1);
-  int64_t* gpre = pool.get<int64_t>(nlong + 1);
-  uint64_t* skey = pool.get<uint64_t>(S_ub);
-  int32_t* sval = pool.get<int32_t>(S_ub);
+  int64_t* nb = pool.tmp<int64_t>(nlong);
+  int64_t* ns = pool.tmp<int64_t>(nlong);
+  int64_t* ngr = pool.tmp<int64_t>(nlong);
+  int64_t* boff = pool.tmp<int64_t>(nlong + 1);
+  int64_t* soff = pool.tmp<int64_t>(nlong + 1);
+  int64_t* gpre = pool.tmp<int64_t>(nlong + 1);
+  uint64_t* skey = pool.tmp<uint64_t>(S_ub);
+  int32_t* sval = pool.tmp<int32_t>(S_ub);
   if (!nb || !ns || !ngr || !boff || !soff || !gpre || !skey || !sval) return SCAN_ENOMEM;
   k_bucket_plan<<<grid_of(nlong, 256), 256, 0, s>>>(S, llist, nlong, nb, ns, ngr);
   GS_LAUNCH();
@@ -1210,11 +1210,11 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
   GS_LAUNCH();
   GS_TRY(sort_level(skey, sval, nullptr, nullptr, Segs{soff, soff + 1}, nlong, S_ub, false, pool, s,
                     depth + 1));
-  unsigned long long* bcount = pool.get<unsigned long long>(B_ub);
-  unsigned long long* bfill = pool.get<unsigned long long>(B_ub);
-  int64_t* bscan = pool.get<int64_t>(B_ub + 1);
-  uint16_t* bid = pool.get<uint16_t>(total);
-  unsigned* ghist = pool.get<unsigned>((size_t)G_ub * BKT_FAN);
+  unsigned long long* bcount = pool.tmp<unsigned long long>(B_ub);
+  unsigned long long* bfill = pool.tmp<unsigned long long>(B_ub);
+  int64_t* bscan = pool.tmp<int64_t>(B_ub + 1);
+  uint16_t* bid = pool.tmp<uint16_t>(total);
+  unsigned* ghist = pool.tmp<unsigned>((size_t)G_ub * BKT_FAN);
   if (!bcount || !bfill || !bscan || !bid || !ghist) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(bcount, 0, B_ub * sizeof(unsigned long long), s));
   GS_CUDA(cudaMemsetAsync(bfill, 0, B_ub * sizeof(unsigned long long), s));
@@ -1237,8 +1237,8 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
   pool.put(bcount);
   pool.put(bfill);
   // the buckets as segments of their own
-  int64_t* bb = pool.get<int64_t>(B_ub);
-  int64_t* be = pool.get<int64_t>(B_ub);
+  int64_t* bb = pool.tmp<int64_t>(B_ub);
+  int64_t* be = pool.tmp<int64_t>(B_ub);
   if (!bb || !be) return SCAN_ENOMEM;
   k_bucket_bounds<<<grid_of(B_ub, 256), 256, 0, s>>>(S, llist, nlong, boff, bscan, B_ub, bb, be);
   GS_LAUNCH();
@@ -1263,21 +1263,20 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
 int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Segs S, int64_t nseg,
                int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth, bool ascending) {
   if (nseg <= 0 || total <= 1) return SCAN_OK;
-  unsigned long long* counts = pool.get<unsigned long long>(2 * NCNT);
+  unsigned long long* counts = pool.tmp<unsigned long long>(2 * NCNT);
   if (!counts) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(counts, 0, 2 * NCNT * sizeof(unsigned long long), s));
   const unsigned g_seg = (unsigned)std::min<int64_t>((nseg + 255) / 256, sm_count() * 16);
   k_classify_count<<<g_seg, 256, 0, s>>>(S, nseg, total, counts);
   GS_LAUNCH();
   unsigned long long hc[NCNT];
-  GS_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
-  GS_CUDA(cudaStreamSynchronize(s));
+  GS_TRY(read_back(hc, counts, sizeof(hc), s));
   if (hc[NCLASS + 2]) return SCAN_EINVAL;  // before any element is touched
   int64_t base[NCLASS + 1];
   base[0] = 0;
   for (int c = 0; c < NCLASS; ++c) base[c + 1] = base[c] + (int64_t)hc[c];
-  int64_t* list = pool.get<int64_t>(base[NCLASS] > 0 ? base[NCLASS] : 1);
-  int64_t* base_dev = pool.get<int64_t>(NCLASS + 1);
+  int64_t* list = pool.tmp<int64_t>(base[NCLASS] > 0 ? base[NCLASS] : 1);
+  int64_t* base_dev = pool.tmp<int64_t>(NCLASS + 1);
   if (!list || !base_dev) return SCAN_ENOMEM;
   GS_CUDA(cudaMemcpyAsync(base_dev, base, sizeof(base), cudaMemcpyHostToDevice, s));
   const uint64_t* ik = in_alt ? alt_k : key;  // where the data is
@@ -1368,12 +1367,12 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
       k_copy_segments<<<grid_of(nlong, 1), 256, 0, s>>>(alt_k, alt_v, key, val, S, llist, nlong);
       GS_LAUNCH();
     }
-    int64_t* tiles = pool.get<int64_t>(nlong);
-    int64_t* tile_prefix = pool.get<int64_t>(nlong + 1);
-    int64_t* chunks = pool.get<int64_t>(nlong);
-    int64_t* chunk_prefix = pool.get<int64_t>(nlong + 1);
-    uint64_t* tk = pool.get<uint64_t>(total);
-    int32_t* tv = pool.get<int32_t>(total);
+    int64_t* tiles = pool.tmp<int64_t>(nlong);
+    int64_t* tile_prefix = pool.tmp<int64_t>(nlong + 1);
+    int64_t* chunks = pool.tmp<int64_t>(nlong);
+    int64_t* chunk_prefix = pool.tmp<int64_t>(nlong + 1);
+    uint64_t* tk = pool.tmp<uint64_t>(total);
+    int32_t* tv = pool.tmp<int32_t>(total);
     if (!tiles || !tile_prefix || !chunks || !chunk_prefix || !tk || !tv) return SCAN_ENOMEM;
     k_long_tiles<<<grid_of(nlong, 256), 256, 0, s>>>(S, llist, nlong, tiles, chunks,
                                                      MERGE_CHUNK);
@@ -1387,7 +1386,7 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
         key, val, key, val, S, llist, counts + NCLASS, tile_prefix, nlong, tk, tv, false);
     GS_LAUNCH();
     const int64_t total_chunks_ub = (total + MERGE_CHUNK - 1) / MERGE_CHUNK + nlong;
-    MergeDesc* desc = pool.get<MergeDesc>((size_t)total_chunks_ub);
+    MergeDesc* desc = pool.tmp<MergeDesc>((size_t)total_chunks_ub);
     if (!desc) return SCAN_ENOMEM;
     // every pass reads each segment from the buffer its parity says and
     // writes the other; the last pass of every segment writes (key, val)

@@ -1415,7 +1415,7 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
                     unsigned long long* work, int lsh_T, int32_t max_od, int64_t* deferred,
                     unsigned long long* n_deferred, uint32_t* tcnt, uint32_t* tc16, int32_t* twin,
                     unsigned* status, const double* ow, double* tsum, const CountCfg& cfg,
-                    cudaStream_t s, cudaEvent_t k0, cudaEvent_t k1, int64_t small_end,
+                    cudaStream_t s, cudaEvent_t* k0, cudaEvent_t* k1, int64_t small_end,
                     const Hubs& hubs) {
   int od_cap = 16;
   while (od_cap < max_od && od_cap < SMEM_OD_MAX) od_cap <<= 1;
@@ -1430,7 +1430,7 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
   GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_triangles<false, IT, WT, R>,
                                                         TRI_THREADS, smem));
   if (per_sm < 1) per_sm = 1;
-  if (k0) GS_CUDA(cudaEventRecord(k0, s));
+  if (k0) GS_TRY(CountTimer::mark(k0, s));
   if (hubs.num) {
     // two elements per lane and round: a suffix fills a round of half the
     // hash-table kernel's bound (a quarter and the whole of it were slower)
@@ -1450,7 +1450,7 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
       off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off, order, work, lsh_T, cfg.cta_chunk,
       cfg.long_list, od_cap, deferred, n_deferred, false, tcnt, tc16, twin, status, ow, tsum);
   GS_LAUNCH();
-  if (k1) GS_CUDA(cudaEventRecord(k1, s));
+  if (k1) GS_TRY(CountTimer::mark(k1, s));
   int small_per_sm = 1;
   GS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k_tri_small<IT, WT, R>,
                                                         SW_WARPS * 32, 0));
@@ -1483,8 +1483,8 @@ int launch_counting_cfg(const int64_t* off, const int32_t* adj, const int32_t* d
                         const int32_t* order, unsigned long long* work, int lsh_T, int32_t max_od,
                         int64_t* deferred, unsigned long long* n_deferred, uint32_t* tcnt,
                         uint32_t* tc16, int32_t* twin, unsigned* status, const double* ow,
-                        double* tsum, const CountCfg& cfg, cudaStream_t s, cudaEvent_t k0,
-                        cudaEvent_t k1, int64_t small_end,
+                        double* tsum, const CountCfg& cfg, cudaStream_t s, cudaEvent_t* k0,
+                        cudaEvent_t* k1, int64_t small_end,
                         const Hubs& hubs) {
   if (!WT && cfg.rounds == 8)
     return launch_counting<IT, WT, 8>(off, adj, deg, odeg, oadj, opos, okey, odp, n, item_off, order,
@@ -1499,39 +1499,39 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
                                   const int32_t* deg, int64_t n, int64_t arcs, const int32_t* odeg,
                                   int32_t* oadj, int32_t* opos, int32_t maxdeg,
                                   int32_t max_od, int lsh_T, const double* wcsr, double* sim_csr,
-                                  unsigned* status, Pool& pool, cudaStream_t s, float* count_ms,
+                                  unsigned* status, Pool& pool, cudaStream_t s, CountTimer* timer,
                                   const CountCfg& cfg, int64_t v0, int64_t v1,
                                   uint32_t* counts_out) {
   if (v1 < 0) v1 = n;
   const bool weighted = wcsr != nullptr;
   const int64_t m = arcs;  // out-lists live in CSR slots: counts and twins are indexed by arc
   const int64_t edges = m / 2;  // oriented edges (the orientation checked sum od = arcs / 2)
-  int64_t* odp = pool.get<int64_t>(n + 1);
-  uint64_t* okey = pool.get<uint64_t>(edges > 0 ? edges : 1);
-  int32_t* oval = pool.get<int32_t>(edges > 0 ? edges : 1);
+  int64_t* odp = pool.tmp<int64_t>(n + 1);
+  uint64_t* okey = pool.tmp<uint64_t>(edges > 0 ? edges : 1);
+  int32_t* oval = pool.tmp<int32_t>(edges > 0 ? edges : 1);
   if (!odp || !okey || !oval) return SCAN_ENOMEM;
-  double* ow = weighted ? pool.get<double>(m) : nullptr;     // weight of every out-arc
-  double* tsum = weighted ? pool.get<double>(m) : nullptr;   // numerator sums per out-arc
-  double* norm = weighted ? pool.get<double>(n > 0 ? n : 1) : nullptr;
+  double* ow = weighted ? pool.tmp<double>(m) : nullptr;     // weight of every out-arc
+  double* tsum = weighted ? pool.tmp<double>(m) : nullptr;   // numerator sums per out-arc
+  double* norm = weighted ? pool.tmp<double>(n > 0 ? n : 1) : nullptr;
   if (weighted && (!ow || !tsum || !norm)) return SCAN_ENOMEM;
   if (weighted) GS_CUDA(cudaMemsetAsync(tsum, 0, m * sizeof(double), s));
   const int64_t nbins = (int64_t)maxdeg + 1;
-  uint32_t* tcnt = pool.get<uint32_t>(m);
+  uint32_t* tcnt = pool.tmp<uint32_t>(m);
   // 16-bit (u,w) counters, two per word, when positions fit in 32 bits
   const bool narrow = m < ((int64_t)1 << 31) - 1 && !force_wide_index();
-  uint32_t* tc16 = narrow ? pool.get<uint32_t>(m / 2 + 1) : nullptr;
-  int32_t* twin = pool.get<int32_t>(m);
-  int32_t* items = pool.get<int32_t>(n);
-  int32_t* items_sorted = pool.get<int32_t>(n);
-  int32_t* order = pool.get<int32_t>(n);
-  int64_t* item_off = pool.get<int64_t>(n + 1);
-  unsigned long long* hist = pool.get<unsigned long long>(2 * nbins);  // counts | fill cursors
-  int64_t* start = pool.get<int64_t>(nbins + 1);
+  uint32_t* tc16 = narrow ? pool.tmp<uint32_t>(m / 2 + 1) : nullptr;
+  int32_t* twin = pool.tmp<int32_t>(m);
+  int32_t* items = pool.tmp<int32_t>(n);
+  int32_t* items_sorted = pool.tmp<int32_t>(n);
+  int32_t* order = pool.tmp<int32_t>(n);
+  int64_t* item_off = pool.tmp<int64_t>(n + 1);
+  unsigned long long* hist = pool.tmp<unsigned long long>(2 * nbins);  // counts | fill cursors
+  int64_t* start = pool.tmp<int64_t>(nbins + 1);
   // counters of the hash-table, binary-search and warp kernels, deferred
   // items, counter of the hub kernel
-  unsigned long long* work = pool.get<unsigned long long>(5);
+  unsigned long long* work = pool.tmp<unsigned long long>(5);
   // items: at most one per vertex plus one per cta_chunk arcs
-  int64_t* deferred = pool.get<int64_t>(n + m / cfg.cta_chunk + 1);
+  int64_t* deferred = pool.tmp<int64_t>(n + m / cfg.cta_chunk + 1);
   if (!tcnt || (narrow && !tc16) || !twin || !items || !items_sorted || !order || !item_off ||
       !hist || !start ||
       !work || !deferred)
@@ -1568,12 +1568,12 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
   int32_t* hub_list = nullptr;
   HubInfo* hub_info = nullptr;
   if (n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG && !warp_vertex(maxdeg, max_od, cfg.warp_deg)) {
-    num = pool.get<uint16_t>(n);
-    o16 = pool.get<uint16_t>(m + 2);
-    hub_list = pool.get<int32_t>(HUB_MAX);
-    hub_info = pool.get<HubInfo>(1);
-    unsigned long long* hh = pool.get<unsigned long long>(2 * nbins);
-    int64_t* pre = pool.get<int64_t>(nbins + 1);
+    num = pool.tmp<uint16_t>(n);
+    o16 = pool.tmp<uint16_t>(m + 2);
+    hub_list = pool.tmp<int32_t>(HUB_MAX);
+    hub_info = pool.tmp<HubInfo>(1);
+    unsigned long long* hh = pool.tmp<unsigned long long>(2 * nbins);
+    int64_t* pre = pool.tmp<int64_t>(nbins + 1);
     if (!num || !o16 || !hub_list || !hub_info || !hh || !pre) return SCAN_ENOMEM;
     const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 64);
     GS_CUDA(cudaMemsetAsync(hh, 0, 2 * nbins * sizeof(unsigned long long), s));
@@ -1594,14 +1594,12 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     pool.put(pre);
     hubs = Hubs{num, o16, hub_info};
   }
-  cudaEvent_t e0, e1, k0 = nullptr, k1 = nullptr;
-  GS_CUDA(cudaEventCreate(&e0));
-  GS_CUDA(cudaEventCreate(&e1));
-  if (count_ms) {  // the CTA counting kernel alone, for its roofline
-    GS_CUDA(cudaEventCreate(&k0));
-    GS_CUDA(cudaEventCreate(&k1));
+  cudaEvent_t *k0 = nullptr, *k1 = nullptr;  // around the CTA kernels, for their roofline
+  if (timer) {
+    k0 = &timer->kernel[0];
+    k1 = &timer->kernel[1];
+    GS_TRY(CountTimer::mark(&timer->step[0], s));
   }
-  GS_CUDA(cudaEventRecord(e0, s));
   // the rank and weight passes walk 32 rows per warp (EXPAND_T / 32 warps a
   // CTA); the similarity pass takes EXPAND_T * per edges per CTA
   const unsigned wgrid =
@@ -1643,7 +1641,7 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
                                               nullptr, twin, status, nullptr, nullptr, cfg, s, k0, k1, v1, hubs)));
     }
   }
-  GS_CUDA(cudaEventRecord(e1, s));
+  if (timer) GS_TRY(CountTimer::mark(&timer->step[1], s));
   if (n > 0 && m > 0 && counts_out) {
     k_counts_out<<<wgrid, EXPAND_T, 0, s>>>(off, adj, odp, oadj, opos, tcnt, tc16, n, counts_out);
     GS_LAUNCH();
@@ -1660,20 +1658,6 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     }
     GS_LAUNCH();
   }
-  if (count_ms) {
-    GS_CUDA(cudaEventSynchronize(e1));
-    GS_CUDA(cudaEventElapsedTime(count_ms, e0, e1));
-    float kms = 0;
-    if (n > 0 && m > 0 && cudaEventElapsedTime(&kms, k0, k1) == cudaSuccess)
-      record_kernel_ms(kms);
-    else
-      record_kernel_ms(0);
-    cudaGetLastError();
-    cudaEventDestroy(k0);
-    cudaEventDestroy(k1);
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
   pool.put(tcnt);
   if (tc16) pool.put(tc16);
   pool.put(twin);
