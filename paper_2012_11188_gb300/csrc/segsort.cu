@@ -950,9 +950,13 @@ __device__ __forceinline__ void block_exclusive_scan(unsigned* h, unsigned* wsum
 // Bucket of every element of the long segments, written to bid, and the
 // bucket sizes per group of BKT_G chunks (ghist) and per segment (one global
 // atomic per bucket and group). The segment's splitters are held in shared
-// memory as a complete binary search tree in breadth-first order (node i's
-// children are 2i and 2i + 1; padded with entries that no element follows),
-// so that every lane descends the same number of levels without branches.
+// memory in order, with a table that divides their key range into BKT_CELLS
+// equal cells and gives the first splitter of each: an element looks its
+// cell up and searches only that cell's splitters, one or two for most keys,
+// all of them only where they share one key. (Descending a tree of up to 1024
+// splitters was ten dependent loads: 7.1 ms of an R-MAT s24 build, now 4.2.)
+constexpr int BKT_CELLS = 2048;
+
 __global__ void __launch_bounds__(BKT_T, 2)
 k_bucket_count(const uint64_t* __restrict__ ck, const int32_t* __restrict__ cv, Segs S,
                const int64_t* __restrict__ list, int64_t nlong, const int64_t* __restrict__ soff,
@@ -963,6 +967,7 @@ k_bucket_count(const uint64_t* __restrict__ ck, const int32_t* __restrict__ cv, 
   __shared__ uint64_t tkey[BKT_FAN];
   __shared__ int32_t tval[BKT_FAN];
   __shared__ unsigned hsum[BKT_FAN];
+  __shared__ uint16_t cell0[BKT_CELLS + 2];  // splitters before cell i
   constexpr int U = 8;  // elements per thread in flight
   const int t = threadIdx.x, lane = t & 31;
   const int64_t G = gpre[nlong];
@@ -972,20 +977,25 @@ k_bucket_count(const uint64_t* __restrict__ ck, const int32_t* __restrict__ cv, 
     const int64_t b = S.b[sg], len = S.e[sg] - b;
     const int nbx = (int)(boff[x + 1] - boff[x]);
     const int nsp = nbx - 1;
-    const int L = 32 - __clz(nsp);  // levels: 2^L - 1 >= nsp nodes
     const int64_t q0 = (g - gpre[x]) * BKT_CH * BKT_G;
     const int m = (int)(min(len, q0 + (int64_t)BKT_CH * BKT_G) - q0);
-    for (int i = t + 1; i < (1 << L); i += BKT_T) {
-      const int l = 31 - __clz(i), p = i - (1 << l);
-      const int r = ((2 * p + 1) << (L - 1 - l)) - 1;  // in-order rank of node i
-      if (r < nsp) {
-        const int64_t q = soff[x] + (int64_t)(r + 1) * BKT_OS;
-        tkey[i] = skey[q];
-        tval[i] = sval[q];
-      } else {
-        tkey[i] = 0;  // sorts after every element
-        tval[i] = SENT_V;
+    for (int i = t; i < nsp; i += BKT_T) {
+      const int64_t q = soff[x] + (int64_t)(i + 1) * BKT_OS;
+      tkey[i] = skey[q];
+      tval[i] = sval[q];
+    }
+    __syncthreads();
+    const uint64_t kmax = tkey[0], kmin = tkey[nsp - 1];  // splitters descend
+    // cell of key K: (kmax - K) >> shift, below BKT_CELLS for every splitter
+    const int shift = max(0, 64 - __clzll((long long)(kmax - kmin)) - 11);
+    static_assert(BKT_CELLS == 1 << 11, "");
+    for (int c = t; c <= BKT_CELLS; c += BKT_T) {
+      int lo = 0, hi = nsp;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((int)((kmax - tkey[mid]) >> shift) < c) lo = mid + 1; else hi = mid;
       }
+      cell0[c] = (uint16_t)lo;
     }
     for (int j = t; j < nbx; j += BKT_T) hsum[j] = 0;
     __syncthreads();
@@ -1004,13 +1014,21 @@ k_bucket_count(const uint64_t* __restrict__ ck, const int32_t* __restrict__ cv, 
 #pragma unroll
       for (int e = 0; e < U; ++e) {
         const int i = i0 + t + e * BKT_T;
-        int j = 1;
-        for (int l = 0; l < L; ++l) {
-          const uint64_t tk = tkey[j];
-          const bool right = tk > K[e] || (tk == K[e] && tval[j] < V[e]);
-          j = 2 * j + (right ? 1 : 0);
+        // splitters before (K, V): none before the largest key, all after
+        // the smallest, else those before the cell and some of its own
+        int bk = 0;
+        if (K[e] < kmin) {
+          bk = nsp;
+        } else if (K[e] <= kmax) {
+          const int c = (int)((kmax - K[e]) >> shift);
+          bk = cell0[c];
+          int hi = cell0[c + 1];
+          while (bk < hi) {
+            const int mid = (bk + hi) >> 1;
+            const uint64_t tk = tkey[mid];
+            if (tk > K[e] || (tk == K[e] && tval[mid] < V[e])) bk = mid + 1; else hi = mid;
+          }
         }
-        const int bk = j - (1 << L);  // splitters before (K, V)
         const bool act = i < m;
         if (act) bc[i] = (uint16_t)bk;
         const unsigned peers = __match_any_sync(0xffffffffu, act ? bk : -1);
