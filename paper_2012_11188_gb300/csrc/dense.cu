@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "exact_sim.cuh"
 #include "scan_internal.cuh"
 
 namespace gscan {
@@ -146,11 +147,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 // from divergent loops); group g uses barriers 1 + 2g (sync) and 2 + 2g (vote).
 __device__ __forceinline__ void epi_barrier(int id) {
   asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(32 * EPI_WARPS) : "memory");
-}
-
-__device__ __forceinline__ double sim_from(int kind, int64_t c, int64_t du, int64_t dv) {
-  if (kind == SCAN_COSINE) return __ddiv_rn((double)c, __dsqrt_rn((double)((du + 1) * (dv + 1))));
-  return __ddiv_rn((double)c, (double)(du + dv + 2 - c));
 }
 
 // (A+I) as a dense row-major np x np bf16 matrix (zeroed by the caller), and
@@ -395,7 +391,7 @@ k_dense_mma(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
               const int64_t dx = a.deg[x];
               // LSH mode: approximated edges are written by the estimate pass
               if (a.lsh_T >= 0 && dx > a.lsh_T && dj > a.lsh_T) continue;
-              const double sv = sim_from(a.kind, cnt, dx, dj);
+              const double sv = sim_of(a.kind, cnt, dx, dj);
               a.sim[pos_x] = sv;
               a.sim[p] = sv;
             }

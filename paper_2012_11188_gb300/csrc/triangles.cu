@@ -15,6 +15,7 @@
 // This replaces the paper's merge (which reads sum(d+_u + d+_v)) by a hash
 // probe of out(u) only (sum over u of d+_u squared), the scheme of the paper's
 // Algorithm 1 applied to the oriented lists.
+#include "exact_sim.cuh"
 #include "scan_internal.cuh"
 
 namespace gscan {
@@ -1115,15 +1116,6 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
     }
   }
   if (bad) atomicOr(status, (unsigned)DEV_BADGRAPH);
-}
-
-// Cosine (Section 3.1) or Jaccard (Section 2.1.1) from the closed count.
-__device__ __forceinline__ double sim_of(int kind, int64_t c, int64_t du, int64_t dv) {
-  if (kind == SCAN_COSINE) {
-    const int64_t prod = (du + 1) * (dv + 1);
-    return __ddiv_rn((double)c, __dsqrt_rn((double)prod));
-  }
-  return __ddiv_rn((double)c, (double)(du + dv + 2 - c));
 }
 
 // Every oriented edge a->b writes sigma to both of its CSR arcs. Threads run
