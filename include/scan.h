@@ -273,7 +273,10 @@ int scan_kernel_launches(uint64_t* count);
  *              dense_min_n 2..65536);
  *   warp_deg   rows of at most this many positions whose out-list has at
  *              most 256 entries are handled by one warp with its own table;
- *              the others by a CTA sharing one table (32..4096);
+ *              the others by a CTA sharing one table (32..4096); rows of
+ *              more than 320 positions among the 65535 vertices of highest
+ *              degree always go to a CTA, which holds their out-list as a
+ *              bitmap;
  *   cta_chunk  CSR positions of a row per CTA work item (256..65536, a
  *              multiple of 32);
  *   long_list  suffixes of an out-list at least this long are streamed one

@@ -30,10 +30,6 @@ constexpr int TRI_THREADS = 512;
 constexpr int TRI_WARPS = TRI_THREADS / 32;
 constexpr int SMEM_OD_MAX = 4096;    // out(v) sizes handled by the shared-memory table
 
-__device__ __forceinline__ bool lower(int32_t du, int32_t u, int32_t dv, int32_t v) {
-  return du < dv || (du == dv && u < v);
-}
-
 // Key of vertex x in the degree order: descending keys = ascending (d_x, x).
 __device__ __forceinline__ uint64_t rank_key(int32_t d, int32_t x) {
   return ~(((uint64_t)(uint32_t)d << 32) | (uint32_t)x);
@@ -59,6 +55,24 @@ constexpr int SW_SLOTS = 2 * SMALL_OD;  // 2^table_log2(SMALL_OD) slots per tabl
 __host__ __device__ __forceinline__ bool warp_vertex(int64_t d, int64_t od, int warp_deg) {
   return d <= warp_deg && od <= SMALL_OD;
 }
+
+// The hubs (below): the vertices of at least min_deg. A hub of more than
+// HUB_DEG positions is the CTA kernel's whatever warp_deg says: its bitmap
+// costs less per probe than a warp's hash table. R-MAT s20, ms per build:
+// without this rule 9.53, HUB_DEG 320 8.82, 256 8.81, 192 8.81, 128 9.03;
+// weighted 14.56, then 13.51, 13.52, 13.52, 13.74; R-MAT s22 with MinHash 30.57,
+// then 30.65, 30.70, 30.81, 30.77; 512 SBM graphs 67.9, then 67.3 for all. (A
+// smaller warp_deg for every vertex loses where there are no hubs to gain: s24
+// 174 ms at 192.)
+constexpr int HUB_DEG = 320;
+struct HubInfo {
+  int32_t min_deg;
+  int32_t count;
+  int64_t items;       // leading items of the degree order whose vertex is a hub
+};
+__device__ __forceinline__ int hub_cta_deg(const HubInfo* info) {
+  return info ? max(info->min_deg, HUB_DEG + 1) : 0x7fffffff;
+}
 constexpr int SW_WARPS = 4;
 
 // Work items of the CTA kernel: a vertex v not handled by a warp contributes
@@ -69,14 +83,15 @@ constexpr int SW_WARPS = 4;
 // (v0, v1): only middle vertices in [v0, v1) get items (a rank's share of a
 // sharded count; the whole graph otherwise).
 __global__ void k_item_counts(const int32_t* __restrict__ odeg, const int32_t* __restrict__ deg,
-                              int64_t n, int warp_deg, int chunk, int64_t v0, int64_t v1,
-                              int32_t* __restrict__ items) {
+                              int64_t n, int warp_deg, const HubInfo* __restrict__ hubs,
+                              int chunk, int64_t v0, int64_t v1, int32_t* __restrict__ items) {
+  const int hub_deg = hub_cta_deg(hubs);
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int64_t od = odeg[v];
     const int32_t d = deg[v];
     int c = 0;
-    if (v >= v0 && v < v1 && !warp_vertex(d, od, warp_deg) && d - od > 0)
+    if (v >= v0 && v < v1 && (!warp_vertex(d, od, warp_deg) || d >= hub_deg) && d - od > 0)
       c = (int)((d - od + chunk - 1) / chunk);
     items[v] = c;
   }
@@ -631,12 +646,6 @@ constexpr int HUB_WARPS = HUB_T / 32;
 constexpr int HUB_WORDS = 2048;         // 32 numbers each
 constexpr int HUB_PAIRS = 4;            // 64-element rounds in flight of a long suffix
 
-struct HubInfo {
-  int32_t min_deg;     // hubs: the vertices of at least this degree
-  int32_t count;
-  int64_t items;       // leading items of the degree order whose vertex is a hub
-};
-
 // vertices per degree, bins of descending degree, degrees >= HUB_MIN_DEG
 __global__ void k_hub_hist(const int32_t* __restrict__ deg, int64_t n, int32_t maxdeg,
                            unsigned long long* __restrict__ hist) {
@@ -1049,7 +1058,8 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
             const int32_t* __restrict__ oadj, const int32_t* __restrict__ opos,
             const uint64_t* __restrict__ okey,
             const int64_t* __restrict__ odp, int64_t n, unsigned long long* __restrict__ work,
-            int batch, int lsh_T, int warp_deg, int long_list, uint32_t* __restrict__ tcnt,
+            int batch, int lsh_T, int warp_deg, const HubInfo* __restrict__ hubs, int long_list,
+            uint32_t* __restrict__ tcnt,
             uint32_t* __restrict__ tc16,
             int32_t* __restrict__ twin_rel, unsigned* status, const double* __restrict__ ow,
             double* __restrict__ tsum) {
@@ -1064,6 +1074,7 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
   uint32_t* vcnt = WT ? nullptr : s_cnt[wid];
   const Weights wt{ow, tsum, WT ? (void*)s_hb[wid] : nullptr};
   const SliceSmem sm{s_u[wid], s_p[wid], s_acc[wid]};
+  const int hub_deg = hub_cta_deg(hubs);
   unsigned bad = 0;
   for (;;) {
     unsigned long long base = 0;
@@ -1077,7 +1088,7 @@ k_tri_small(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
     const bool inb = lane < batch && vl < n;
     const int32_t dl = inb ? deg[vl] : 0;
     const int32_t ol = inb ? odeg[vl] : 0;
-    const bool mine = dl > 0 && warp_vertex(dl, ol, warp_deg) && dl - ol > 0;
+    const bool mine = dl > 0 && warp_vertex(dl, ol, warp_deg) && dl < hub_deg && dl - ol > 0;
     const int64_t offl = mine ? off[vl] : 0, odpl = mine ? odp[vl] : 0;
     unsigned todo = __ballot_sync(FULL, mine);
     while (todo) {
@@ -1453,7 +1464,7 @@ int launch_counting(const int64_t* off, const int32_t* adj, const int32_t* deg, 
   const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(32, n / (2 * small_warps)));
   k_tri_small<IT, WT, R><<<sms * small_per_sm, SW_WARPS * 32, 0, s>>>(
       off, adj, deg, odeg, oadj, opos, okey, odp, small_end, work + 2, batch, lsh_T, cfg.warp_deg,
-      cfg.long_list, tcnt, tc16, twin, status, ow, tsum);
+      hubs.info, cfg.long_list, tcnt, tc16, twin, status, ow, tsum);
   GS_LAUNCH();
   // items with out-lists too long for the shared table, and items deferred
   // by the CTA kernel (normally none: the launch then ends at once)
@@ -1541,25 +1552,13 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     k_fill_i32<<<1024, 256, 0, s>>>(twin, m, -1);
     GS_LAUNCH();
   }
-  if (n > 0) {
-    const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 64);
-    k_item_counts<<<g, 256, 0, s>>>(odeg, deg, n, cfg.warp_deg, cfg.cta_chunk, v0, v1, items);
-    GS_LAUNCH();
-    k_item_hist<<<g, 256, 0, s>>>(items, deg, n, maxdeg, hist);
-    GS_LAUNCH();
-    GS_TRY(exclusive_scan_i64(reinterpret_cast<const int64_t*>(hist), start, nbins, pool, s));
-    k_item_place<<<g, 256, 0, s>>>(items, deg, n, maxdeg, start, hist + nbins, order);
-    GS_LAUNCH();
-    k_item_gather<<<g, 256, 0, s>>>(items, order, start, maxdeg, n, items_sorted);
-    GS_LAUNCH();
-  }
-  GS_TRY(exclusive_scan_i32_to_i64(items_sorted, item_off, n, pool, s));
-  // hub numbers, when some vertex is beyond the warp kernel
+  // hub numbers, when some vertex may be the CTA kernel's
   Hubs hubs;
   uint16_t *num = nullptr, *o16 = nullptr;
   int32_t* hub_list = nullptr;
   HubInfo* hub_info = nullptr;
-  if (n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG && !warp_vertex(maxdeg, max_od, cfg.warp_deg)) {
+  if (n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG &&
+      (maxdeg > HUB_DEG || !warp_vertex(maxdeg, max_od, cfg.warp_deg))) {
     num = pool.tmp<uint16_t>(n);
     o16 = pool.tmp<uint16_t>(m + 2);
     hub_list = pool.tmp<int32_t>(HUB_MAX);
@@ -1580,11 +1579,27 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     GS_LAUNCH();
     k_hub_number<<<sm_count() * 8, 256, 0, s>>>(deg, maxdeg, hub_info, pre, hub_list, num);
     GS_LAUNCH();
-    k_hub_items<<<1, 32, 0, s>>>(hub_info, maxdeg, start, item_off, work);
-    GS_LAUNCH();
     pool.put(hh);
     pool.put(pre);
     hubs = Hubs{num, o16, hub_info};
+  }
+  if (n > 0) {
+    const unsigned g = (unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 64);
+    k_item_counts<<<g, 256, 0, s>>>(odeg, deg, n, cfg.warp_deg, hub_info, cfg.cta_chunk, v0, v1,
+                                    items);
+    GS_LAUNCH();
+    k_item_hist<<<g, 256, 0, s>>>(items, deg, n, maxdeg, hist);
+    GS_LAUNCH();
+    GS_TRY(exclusive_scan_i64(reinterpret_cast<const int64_t*>(hist), start, nbins, pool, s));
+    k_item_place<<<g, 256, 0, s>>>(items, deg, n, maxdeg, start, hist + nbins, order);
+    GS_LAUNCH();
+    k_item_gather<<<g, 256, 0, s>>>(items, order, start, maxdeg, n, items_sorted);
+    GS_LAUNCH();
+  }
+  GS_TRY(exclusive_scan_i32_to_i64(items_sorted, item_off, n, pool, s));
+  if (hubs.num) {
+    k_hub_items<<<1, 32, 0, s>>>(hub_info, maxdeg, start, item_off, work);
+    GS_LAUNCH();
   }
   cudaEvent_t *k0 = nullptr, *k1 = nullptr;  // around the CTA kernels, for their roofline
   if (timer) {
