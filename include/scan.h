@@ -242,10 +242,11 @@ const char* scan_strerror(int status);
 int scan_last_build_timings(double* ms7);
 
 /* Duration (ms, CUDA events on the build's stream) of the last exact build's
- * CTA counting kernel on this thread: the oriented triangle enumeration over
- * the rows whose out-lists sit in a shared-memory table (Section 6.1 and the
- * hash intersection of Algorithm 1), the bulk of the counting step; 0 if the
- * last build did not run it. */
+ * CTA counting kernels on this thread: the oriented triangle enumeration over
+ * the rows whose out-lists sit in a CTA's shared-memory table, a bitmap for
+ * the vertices of highest degree and a hash table for the others (Section 6.1
+ * and the hash intersection of Algorithm 1), the bulk of the counting step; 0
+ * if the last build did not run them. */
 int scan_last_count_kernel_ms(double* ms);
 
 /* Test hook for the index width of the counting kernels. Graphs with at
@@ -360,10 +361,11 @@ int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end
  * (checked on the device before any element is read or written: otherwise
  * SCAN_EINVAL and the arrays are unchanged); max_len: an upper bound of every
  * segment's length. All three arrays device memory (host pointers:
- * SCAN_EINVAL). Synchronises `stream`. Segments longer than 4096 are split
- * into buckets by a sample sort (sorted random samples give the splitters,
- * one scatter places every element in its bucket), then the buckets are
- * sorted in shared memory. */
+ * SCAN_EINVAL). Synchronises `stream`. Long segments (beyond 4096 elements;
+ * up to 8192 or 16384 are sorted whole where there are very many or very few
+ * of them) are split into buckets by a sample sort (sorted random samples
+ * give the splitters, one scatter places every element in its bucket), then
+ * the buckets are sorted in shared memory. */
 int scan_sort_segments_desc(double* keys, int32_t* ids, const int64_t* seg_off, int64_t nseg,
                             int64_t total, int64_t max_len, uintptr_t stream);
 

@@ -8,7 +8,7 @@
 // Flood 2014) whose state starts at key, i.e. mix64(key + (c+1) * golden).
 //  SimHash (Charikar): hyperplane j gives x in N̄(v) the sign +1 iff bit j%64 of
 //    R(ks, x*1024 + j/64) is set, ks = mix64(seed ^ "SIMH"); s_j = sum of the
-//    signs over N̄(v) in FP32 (exact: |s_j| <= d+1 < 2^24); bit j = [s_j >= 0].
+//    signs over N̄(v); bit j = [s_j >= 0], i.e. at least half of them are +1.
 //    Estimate max(0, cos(pi h / k)) for Hamming distance h, from a table
 //    computed on the host in double precision.
 //  MinHash: h(x) = low 32 bits of R(km, x), km = mix64(seed ^ "MINH").
