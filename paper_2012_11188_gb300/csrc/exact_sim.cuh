@@ -5,8 +5,9 @@
 // clocks, and a correctly rounded square root and division are some 18 of
 // them, 290 clocks for 32 edges; the 64-bit integer form below is about 130
 // instructions that issue four a clock (builds: dense graph of 25,825 vertices,
-// whose similarities the matrix product's epilogue forms, 24.4 -> 22.5 ms,
-// R-MAT s24 155.5 -> 152.5, 512 SBM graphs 69.8 -> 68.7). Both steps are Newton's iteration in
+// whose similarities the matrix product's epilogue forms, 24.4 -> 22.5 ms, 512
+// SBM graphs 69.8 -> 68.7; R-MAT s24 within the noise, since its similarity
+// pass waits for gathers and scattered stores). Both steps are Newton's iteration in
 // fixed point from a 23-bit hardware approximation, of third order, to
 // some 50 bits, one correction by the remainder, and then the exact whole remainder, which
 // decides the last bit: the result does not depend on how good the

@@ -1302,27 +1302,51 @@ k_out_weights(const int64_t* __restrict__ off, const int64_t* __restrict__ odp, 
 // norm[x] = sqrt(1 + sum of w(x,y)^2 over N(x)): the closed neighbourhood
 // with w(x,x) = 1 (Section 4.1.1). FP64 instructions are issued for a whole
 // warp at a time, so rows of at most 32 entries are summed by one thread each
-// (32 vertices per instruction); longer rows by the whole warp.
-__global__ void k_wnorm(const int64_t* __restrict__ off, const double* __restrict__ wcsr, int64_t n,
-                        double* __restrict__ norm) {
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; base < n;
-       base += stride) {
-    const int64_t x = base + lane;
+// (32 vertices per instruction), their entries first brought to shared memory
+// by coalesced loads (RowGroup); longer rows by the whole warp, and rows of
+// more than WNORM_LONG by a CTA (one warp on a hub's row was most of the
+// kernel: R-MAT s20 490 us, now 328).
+constexpr int WNORM_LONG = 4096;
+constexpr int WNORM_T = 128;
+
+__global__ void __launch_bounds__(WNORM_T)
+k_wnorm(const int64_t* __restrict__ off, const double* __restrict__ wcsr, int64_t n,
+        double* __restrict__ norm) {
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ double stage[WNORM_T / 32][32 * 32];
+  __shared__ int scratch[WNORM_T / 32][64];
+  __shared__ int32_t s_long[WNORM_T];
+  __shared__ int s_nlong;
+  __shared__ double s_part[WNORM_T / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double* st = stage[wid];
+  const int64_t stride = (int64_t)gridDim.x * WNORM_T;
+  for (int64_t base = (int64_t)blockIdx.x * WNORM_T; base < n; base += stride) {
+    if (threadIdx.x == 0) s_nlong = 0;
+    __syncthreads();
+    const int64_t x0 = base + wid * 32, x = x0 + lane;
     int64_t b = 0, e = 0;
     if (x < n) {
       b = off[x];
       e = off[x + 1];
     }
-    const bool long_row = e - b > 32;
-    if (x < n && !long_row) {
-      double s2 = 0.0;
-      for (int64_t i = b; i < e; ++i) s2 += wcsr[i] * wcsr[i];
-      norm[x] = sqrt(1.0 + s2);
+    if (x < n && b == e) norm[x] = 1.0;
+    if (e - b > WNORM_LONG) s_long[atomicAdd(&s_nlong, 1)] = (int32_t)(x - base);
+    RowGroup g;
+    g.init(e - b <= 32 ? (int)(e - b) : 0, scratch[wid]);
+    const int64_t first = __shfl_sync(FULL, b, g.row) - g.vs;
+    for (int i0 = 0; i0 < g.total; i0 += 32) {
+      const int64_t bk = __shfl_sync(FULL, first, g.chunk(i0));
+      if (i0 + lane < g.total) st[i0 + lane] = wcsr[bk + i0 + lane];
     }
-    unsigned lm = __ballot_sync(FULL, long_row);
+    __syncwarp();
+    if (lane < g.cnt) {
+      double s2 = 0.0;
+      for (int i = g.vs; i < g.ve; ++i) s2 += st[i] * st[i];
+      norm[x0 + g.row] = sqrt(1.0 + s2);
+    }
+    __syncwarp();
+    unsigned lm = __ballot_sync(FULL, e - b > 32 && e - b <= WNORM_LONG);
     while (lm) {
       const int src = __ffs(lm) - 1;
       lm &= lm - 1;
@@ -1330,8 +1354,34 @@ __global__ void k_wnorm(const int64_t* __restrict__ off, const double* __restric
       double s2 = 0.0;
       for (int64_t i = bb + lane; i < ee; i += 32) s2 += wcsr[i] * wcsr[i];
       for (int o = 16; o; o >>= 1) s2 += __shfl_xor_sync(FULL, s2, o);
-      if (lane == 0) norm[base + src] = sqrt(1.0 + s2);
+      if (lane == 0) norm[x0 + src] = sqrt(1.0 + s2);
     }
+    __syncthreads();
+    const int nl = s_nlong;
+    for (int k = 0; k < nl; ++k) {
+      const int64_t y = base + s_long[k];
+      const int64_t bb = off[y], ee = off[y + 1];
+      // four sums in flight per thread
+      double s2[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int64_t i = bb + threadIdx.x; i < ee; i += 4 * WNORM_T)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int64_t j = i + q * WNORM_T;
+          const double w = j < ee ? wcsr[j] : 0.0;
+          s2[q] += w * w;
+        }
+      double t = (s2[0] + s2[1]) + (s2[2] + s2[3]);
+      for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
+      if (lane == 0) s_part[wid] = t;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double a = 0.0;
+        for (int w = 0; w < WNORM_T / 32; ++w) a += s_part[w];
+        norm[y] = sqrt(1.0 + a);
+      }
+      __syncthreads();
+    }
+    __syncthreads();
   }
 }
 
@@ -1654,8 +1704,8 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     GS_LAUNCH();
   } else if (n > 0 && m > 0) {
     if (weighted) {
-      k_wnorm<<<(unsigned)std::min<int64_t>((n + 255) / 256, sm_count() * 16), 256, 0, s>>>(off, wcsr, n,
-                                                                                      norm);
+      k_wnorm<<<(unsigned)std::min<int64_t>((n + WNORM_T - 1) / WNORM_T, sm_count() * 12), WNORM_T, 0,
+                s>>>(off, wcsr, n, norm);
       GS_LAUNCH();
       k_expand_w<<<egrid, EXPAND_T, 0, s>>>(off, adj, odp, oadj, opos, ow, tsum, twin, wcsr, norm,
                                             deg, n, per, lsh_T, sim_csr, status);
