@@ -1185,6 +1185,13 @@ __device__ __forceinline__ void walk_out_arcs(const int64_t* __restrict__ off,
   }
 }
 
+// BY_OFF: the head's degree from its two offsets, one sector, of which the
+// first is gathered anyway: taken where offsets and degrees together outgrow
+// L2 (R-MAT s24 build 152.4 -> 150.7 ms); elsewhere from deg (s20 8.82 ms, 8.84
+// by offsets).
+constexpr int64_t EXPAND_BY_OFF = 8 << 20;  // vertices
+
+template <bool BY_OFF>
 __global__ void __launch_bounds__(EXPAND_T)
 k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
          const int64_t* __restrict__ odp, const int32_t* __restrict__ oadj,
@@ -1207,7 +1214,8 @@ k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ 
       const int64_t ra = off[a];
       const int64_t j = ra + (k - odp[a]);
       const int32_t b = oadj[j];
-      const int32_t da = deg[a], db = deg[b];
+      const int64_t rb = off[b];
+      const int32_t da = deg[a], db = BY_OFF ? (int32_t)(off[b + 1] - rb) : deg[b];
       // LSH mode: approximated edges are written by the estimate pass
       if (lsh_T >= 0 && da > lsh_T && db > lsh_T) continue;
       int64_t t = tcnt[j];
@@ -1216,7 +1224,7 @@ k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ 
       sim_csr[ra + opos[j]] = sv;
       const int32_t tr = twin_rel[j];
       if (tr < 0) bad = 1;
-      else sim_csr[off[b] + tr] = sv;
+      else sim_csr[rb + tr] = sv;
     }
     __syncthreads();
   }
@@ -1710,8 +1718,9 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
       k_expand_w<<<egrid, EXPAND_T, 0, s>>>(off, adj, odp, oadj, opos, ow, tsum, twin, wcsr, norm,
                                             deg, n, per, lsh_T, sim_csr, status);
     } else {
-      k_expand<<<egrid, EXPAND_T, 0, s>>>(kind, off, deg, odp, oadj, opos, tcnt, tc16, twin, n,
-                                          per, lsh_T, sim_csr, status);
+      auto expand = n > EXPAND_BY_OFF ? k_expand<true> : k_expand<false>;
+      expand<<<egrid, EXPAND_T, 0, s>>>(kind, off, deg, odp, oadj, opos, tcnt, tc16, twin, n, per,
+                                        lsh_T, sim_csr, status);
     }
     GS_LAUNCH();
   }
