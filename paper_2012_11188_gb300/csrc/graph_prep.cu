@@ -100,14 +100,17 @@ int scan_impl(const T* in, int64_t* out, int64_t n, Pool& pool, cudaStream_t s) 
 // Degrees and CSR checks, 32 rows per warp (RowGroup). Rows longer than
 // DEG_LONG are listed for k_degrees_long and left out (one warp would walk
 // a hub's row alone, one dependent load at a time). A group with a bad row
-// bound is not walked.
+// bound is not walked. The list has max_long = arcs / DEG_LONG + 1 places,
+// enough for offsets that do not descend; more long rows than that prove the
+// offsets bad (0, arcs, 0, arcs, ... makes every other row a long one), and
+// what does not fit is not listed.
 constexpr int DEG_LONG = 4096;
 
 __global__ void __launch_bounds__(256)
 k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
           int64_t n, int64_t arcs, int32_t* __restrict__ deg, int32_t* maxdeg,
           unsigned* status, int32_t* __restrict__ long_rows,
-          unsigned* __restrict__ n_long) {
+          unsigned* __restrict__ n_long, unsigned max_long) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ int scratch[8][64];
   const int lane = threadIdx.x & 31;
@@ -125,7 +128,10 @@ k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
     if (v < n) {
       deg[v] = row_bad ? 0 : (int32_t)(e - b);
       if (!row_bad) local_max = max(local_max, (int32_t)(e - b));
-      if (is_long) long_rows[atomicAdd(n_long, 1u)] = (int32_t)v;
+      if (is_long) {
+        const unsigned at = atomicAdd(n_long, 1u);
+        if (at < max_long) long_rows[at] = (int32_t)v; else bad = 1;
+      }
     }
     if (__any_sync(FULL, row_bad)) {
       bad = 1;
@@ -165,8 +171,8 @@ k_degrees(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
 __global__ void __launch_bounds__(1024)
 k_degrees_long(const int64_t* __restrict__ off, const int32_t* __restrict__ adj, int64_t n,
                const int32_t* __restrict__ long_rows, const unsigned* __restrict__ n_long,
-               unsigned* status) {
-  const unsigned cnt = *n_long;
+               unsigned max_long, unsigned* status) {
+  const unsigned cnt = min(*n_long, max_long);
   unsigned bad = 0;
   for (unsigned r = blockIdx.x; r < cnt; r += gridDim.x) {
     const int32_t v = long_rows[r];
@@ -353,10 +359,10 @@ int launch_degrees(const int64_t* off, const int32_t* adj, int64_t n, int64_t ar
   if (!long_rows || !n_long) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(n_long, 0, sizeof(unsigned), s));
   k_degrees<<<grid_for(n, 256), 256, 0, s>>>(off, adj, n, arcs, deg, maxdeg_dev, status, long_rows,
-                                             n_long);
+                                             n_long, (unsigned)max_long);
   GS_LAUNCH();
   k_degrees_long<<<(unsigned)std::min<int64_t>(max_long, sm_count() * 2), 1024, 0, s>>>(
-      off, adj, n, long_rows, n_long, status);
+      off, adj, n, long_rows, n_long, (unsigned)max_long, status);
   GS_LAUNCH();
   pool.put(long_rows);
   pool.put(n_long);
@@ -370,7 +376,9 @@ int launch_orient(const int64_t* off, const int32_t* adj, const int32_t* deg, in
   int32_t* od = pool.tmp<int32_t>(n > 0 ? n : 1);
   int32_t* oadj = pool.tmp<int32_t>(arcs > 0 ? arcs : 1);
   int32_t* opos = pool.tmp<int32_t>(arcs > 0 ? arcs : 1);
-  // rows longer than LONG_ROW: at most arcs / LONG_ROW of them
+  // rows longer than LONG_ROW: at most arcs / LONG_ROW of them (the degree
+  // pass has refused offsets that descend, and k_orient_inplace lists nothing
+  // then)
   const int64_t max_long = arcs / LONG_ROW + 1;
   int32_t* long_rows = pool.tmp<int32_t>(max_long);
   unsigned* n_long = pool.tmp<unsigned>(1);
