@@ -957,7 +957,9 @@ int scan_index_export(scan_index* index, double* sim, int32_t* no_id, double* no
   size_t total = 0;
   for (int k = 0; k < 5; ++k) {
     if (!dst[k] || bytes[k] == 0) continue;
-    if (A * 24 <= EXPORT_ONE && kernel_reads(dst[k], 4)) {
+    // (the index may be on another device than the current one: a copy crosses
+    // devices, a kernel does not)
+    if (A * 24 <= EXPORT_ONE && kernel_reads(dst[k], 4) && kernel_reads(src[k], 4)) {
       parts.dst[k] = dst[k];
       parts.src[k] = src[k];
       parts.words[k] = bytes[k] / 4;

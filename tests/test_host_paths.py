@@ -1,0 +1,46 @@
+"""Host code of the library where the outcome depends on the machine: memory of
+another device, refused launches. On a CUDA runtime of host memory."""
+import numpy as np
+import pytest
+
+import fake_cuda
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_cuda.Fake(str(tmp_path_factory.mktemp("fake_cuda")))
+
+
+@pytest.fixture()
+def clean(fake):
+    yield fake
+    fake.lib.fake_set_device(0)
+    fake.lib.fake_refuse_cooperative(0)
+
+
+def edgeless(fake, n=5):
+    off, adj = np.zeros(n + 1, np.int64), np.zeros(0, np.int32)
+    return fake.build(fake.csr(off, adj, 0)), (off, adj)
+
+
+# device of the index, of the destination, and the current one; what copies
+@pytest.mark.parametrize("index,dst,now,kernel", [(0, 0, 0, True), (1, 1, 1, True),
+                                                  (0, 1, 1, False), (0, 1, 0, False),
+                                                  (0, 0, 1, False)])
+def test_export_across_devices(clean, index, dst, now, kernel):
+    """A kernel of the current device copies only where both sides are its
+    own memory; everything else is a copy of the runtime's."""
+    fake = clean
+    fake.lib.fake_set_device(index)
+    h, _ = edgeless(fake)
+    co_off = np.full(1, 77, np.int64)
+    fake.region(co_off, device=dst)
+    fake.lib.fake_set_device(now)
+    fake.lib.fake_clear_log()
+    assert fake.lib.scan_index_export(h, None, None, None, co_off.ctypes.data, None, None) == 0
+    log = fake.log()
+    assert any("k_export" in x for x in log) == kernel
+    if not kernel:
+        assert co_off[0] == 0 and "copy 8" in log
+    fake.lib.fake_set_device(index)
+    fake.lib.scan_index_free(h)
