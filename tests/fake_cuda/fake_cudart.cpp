@@ -3,6 +3,7 @@
 // their ranges as the driver does, kernel launches do nothing but leave their
 // name in a log, and single calls can be made to fail. Two devices, four
 // multiprocessors each.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -144,11 +145,25 @@ cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3, dim3, void**, size_
   note((refuse_cooperative ? "refused " : "launch ") + kernels()[f]);
   return refuse_cooperative ? cudaErrorCooperativeLaunchTooLarge : cudaSuccess;
 }
-cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, unsigned long long,
+static CUresult attributes(unsigned n, CUpointer_attribute* what, void** to, CUdeviceptr p) {
+  std::lock_guard<std::mutex> lk(mu);
+  auto* r = find((const void*)p);
+  for (unsigned i = 0; i < n; ++i) switch (what[i]) {
+    case CU_POINTER_ATTRIBUTE_MEMORY_TYPE: *(unsigned*)to[i] = r ? r->second.type : 0; break;
+    case CU_POINTER_ATTRIBUTE_IS_MANAGED: *(unsigned*)to[i] = 0; break;
+    case CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL: *(int*)to[i] = r ? r->second.device : -2; break;
+    case CU_POINTER_ATTRIBUTE_RANGE_START_ADDR: *(CUdeviceptr*)to[i] = r ? (CUdeviceptr)r->first : 0; break;
+    case CU_POINTER_ATTRIBUTE_RANGE_SIZE: *(size_t*)to[i] = r ? r->second.bytes : 0; break;
+    default: return CUDA_ERROR_INVALID_VALUE;
+  }
+  return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,
                                              cudaDriverEntryPointQueryResult* q) {
-  *f = nullptr;
-  if (q) *q = cudaDriverEntryPointSymbolNotFound;
-  return cudaErrorInvalidValue;
+  const bool known = !std::strcmp(name, "cuPointerGetAttributes");
+  *f = known ? (void*)attributes : nullptr;
+  if (q) *q = known ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return known ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 }  // extern "C"

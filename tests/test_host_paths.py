@@ -1,5 +1,8 @@
 """Host code of the library where the outcome depends on the machine: memory of
-another device, refused launches. On a CUDA runtime of host memory."""
+another device, refused launches, arrays shorter than the call says. On a CUDA runtime of host
+memory."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -43,4 +46,41 @@ def test_export_across_devices(clean, index, dst, now, kernel):
     if not kernel:
         assert co_off[0] == 0 and "copy 8" in log
     fake.lib.fake_set_device(index)
+    fake.lib.scan_index_free(h)
+
+
+EBADGRAPH, ECUDA = -3, -4
+
+
+@pytest.mark.parametrize("short", [None, "offsets", "adj"])
+@pytest.mark.parametrize("off_type", [np.int64, np.int32])
+def test_batch_of_short_arrays(clean, short, off_type):
+    """Kernels pack a batch from the callers' arrays only where those are as
+    long as the call says: a copy refuses the others, a kernel would read past
+    their ends."""
+    fake = clean
+    off, adj = np.array([0, 2, 4, 6], off_type), np.array([1, 2, 0, 2, 0, 1], np.int32)
+    fake.region(off, nbytes=off.nbytes - off.itemsize if short == "offsets" else None)
+    fake.region(adj, nbytes=adj.nbytes - 8 if short == "adj" else None)
+    graphs = (fake_cuda.scan_csr * 2)(*[fake.csr(off, adj, 1)] * 2)
+    out = (ctypes.c_void_p * 2)()
+    fake.lib.fake_clear_log()
+    rc = fake.lib.scan_index_build_batch(graphs, 2, 0, None, 0, out)
+    log = fake.log()
+    # (the kernels do nothing here, so the checks of a whole graph find no edge)
+    assert rc == (ECUDA if short else EBADGRAPH)
+    assert any("k_pack" in x for x in log) == (short is None)
+    assert ("copy refused" in log) == (short is not None)
+
+
+@pytest.mark.parametrize("short", [False, True])
+def test_export_to_a_short_array(clean, short):
+    fake = clean
+    h, _ = edgeless(fake)
+    co_off = np.full(1, 77, np.int64)
+    fake.region(co_off, nbytes=4 if short else 8)
+    fake.lib.fake_clear_log()
+    rc = fake.lib.scan_index_export(h, None, None, None, co_off.ctypes.data, None, None)
+    assert rc == (ECUDA if short else 0)
+    assert any("k_export" in x for x in fake.log()) != short
     fake.lib.scan_index_free(h)
