@@ -555,7 +555,6 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   const size_t head = ((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255;
   char* scratch = pool.get<char>(head + (qb ? qb : 16));
   if (!scratch) return SCAN_ENOMEM;
-  *done = true;
   int32_t* parent = reinterpret_cast<int32_t*>(scratch);
   unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + head);
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
@@ -567,7 +566,15 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   const unsigned g = (unsigned)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
   int hubs = flags & SCAN_Q_HUBS;
   void* args[] = {&a, &mu, &eps, &hubs};
-  GS_CUDA(cudaLaunchCooperativeKernel((const void*)k_query_one, dim3(g), dim3(ONE_T), args, 0, s));
+  // refused where the stream or the process has fewer multiprocessors than
+  // the device: the launches of a batch answer then
+  if (cudaLaunchCooperativeKernel((const void*)k_query_one, dim3(g), dim3(ONE_T), args, 0, s) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    pool.put(scratch);
+    return SCAN_OK;
+  }
+  *done = true;
   GS_LAUNCH();
   if (host_labels)
     GS_CUDA(cudaMemcpyAsync(host_labels, labels, (size_t)n * sizeof(int32_t),

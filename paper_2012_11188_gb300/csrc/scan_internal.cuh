@@ -329,7 +329,7 @@ int run_queries(const IndexData& ix, int q, const int* mu, const double* eps, in
 
 // One query into device labels (copied to host_labels too unless null) as one
 // cooperative launch; synchronises s. *done = false: such a launch is not to
-// be had, nothing was enqueued.
+// be had or was refused, nothing was enqueued.
 int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels_dev,
                   int32_t* host_labels, int flags, Pool& pool, cudaStream_t s, bool* done);
 

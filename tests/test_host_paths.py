@@ -84,3 +84,26 @@ def test_export_to_a_short_array(clean, short):
     assert rc == (ECUDA if short else 0)
     assert any("k_export" in x for x in fake.log()) != short
     fake.lib.scan_index_free(h)
+
+
+@pytest.mark.parametrize("refuse", [False, True])
+@pytest.mark.parametrize("device", [False, True])
+def test_query_where_a_cooperative_launch_is_refused(clean, refuse, device):
+    """A single query is one cooperative launch; a stream or a process with
+    fewer multiprocessors than the device refuses it, and the launches of a
+    batch answer."""
+    fake = clean
+    h, _ = edgeless(fake)
+    labels = np.full(5, 77, np.int32)
+    if device:
+        fake.region(labels)
+    fake.lib.fake_refuse_cooperative(int(refuse))
+    fake.lib.fake_clear_log()
+    assert fake.lib.scan_query(h, 2, 0.5, labels.ctypes.data, 1, 0) == 0
+    log = fake.log()
+    assert any("k_query_one" in x for x in log)
+    for name in ("k_get_cores", "k_core_prefix", "k_mark_cores", "k_union", "k_labels", "k_hubs"):
+        assert any(name in x for x in log) == refuse, name
+    if refuse:  # cleared by the batch's own memset
+        assert (labels == -1).all()
+    fake.lib.scan_index_free(h)
