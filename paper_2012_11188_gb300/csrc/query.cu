@@ -551,16 +551,21 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   unsigned* status = static_cast<unsigned*>(slot.p);
   if (per_sm == 0 || !status) return SCAN_OK;
   *status = 0;
-  const size_t qb = query_queue_bytes(ix, 1);
-  const size_t head = ((size_t)n * sizeof(int32_t) + 255) & ~(size_t)255;
-  char* scratch = pool.get<char>(head + (qb ? qb : 16));
+  // the count of queued pieces, parents, pieces; without pieces where there is
+  // no room for them
+  const size_t head = 16 + (((size_t)n * sizeof(int32_t) + 15) & ~(size_t)15);
+  unsigned cap = queue_capacity(ix, 1);
+  char* scratch = cap ? pool.get<char>(head + (size_t)cap * sizeof(QPiece)) : nullptr;
+  if (!scratch) {
+    cap = 0;
+    scratch = pool.get<char>(head);
+  }
   if (!scratch) return SCAN_ENOMEM;
-  int32_t* parent = reinterpret_cast<int32_t*>(scratch);
-  unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + head);
+  unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch);
+  int32_t* parent = reinterpret_cast<int32_t*>(scratch + 16);
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
           n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status,
-          qb ? reinterpret_cast<QPiece*>(scratch + head + 16) : nullptr, queued,
-          queue_capacity(ix, 1)};
+          cap ? reinterpret_cast<QPiece*>(scratch + head) : nullptr, queued, cap};
   // a warp per core at most, and no more CTAs than are resident at once
   const int64_t want = std::max<int64_t>(1, (n + ONE_T / 32 - 1) / (ONE_T / 32));
   const unsigned g = (unsigned)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
@@ -592,9 +597,10 @@ int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* ep
   double* eps = pool.get<double>(Q);
   int64_t* nc = pool.get<int64_t>((size_t)Q + 1);
   int32_t* parent = pool.get<int32_t>((size_t)Q * (size_t)(n > 0 ? n : 1));
-  const size_t qb = query_queue_bytes(ix, Q);
+  if (!mu || !eps || !nc || !parent) return SCAN_ENOMEM;
+  size_t qb = query_queue_bytes(ix, Q);
   char* queue = qb ? pool.get<char>(qb) : nullptr;
-  if (!mu || !eps || !nc || !parent || (qb && !queue)) return SCAN_ENOMEM;
+  if (!queue) qb = 0;  // no room: a warp walks a long row alone
   GS_CUDA(cudaMemcpyAsync(mu, mu_host, sizeof(int) * Q, cudaMemcpyHostToDevice, s));
   GS_CUDA(cudaMemcpyAsync(eps, eps_host, sizeof(double) * Q, cudaMemcpyHostToDevice, s));
   if (n == 0) return SCAN_OK;

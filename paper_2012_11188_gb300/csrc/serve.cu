@@ -89,10 +89,11 @@ void finish(scan_server* s, Request* r, int status) {
 }
 
 // Scratch of the query worker, kept across batches and grown on demand:
-// parents (cap x n), mu/eps/core counts, the queue of row pieces and the table of label destinations,
-// and two sets of what a batch in flight owns until its copies are done:
-// staging rows for host destinations, a device status word, its pinned host
-// copy and the event that marks its kernels done.
+// parents (cap x n), mu/eps/core counts, the queue of row pieces (null where
+// there is no room for it) and the table of label destinations, and two sets of
+// what a batch in flight owns until its copies are done: staging rows for host
+// destinations, a device status word, its pinned host copy and the event that
+// marks its kernels done.
 struct QueryScratch {
   int cap = 0;
   int64_t n = 0;
@@ -146,8 +147,7 @@ struct QueryScratch {
     bool ev_ok = true;
     for (auto& e : kern_done)
       ev_ok &= cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
-    if (!parent || !ptrs || !mu || !eps || !nc || !queue || !status[0] || !status[1] || !status_host ||
-        !ev_ok) {
+    if (!parent || !ptrs || !mu || !eps || !nc || !status[0] || !status[1] || !status_host || !ev_ok) {
       release(s);
       return SCAN_ENOMEM;
     }

@@ -1,0 +1,99 @@
+"""Calls at the limit of device memory: an allocator that refuses requests
+beyond a number of bytes. What is only there for speed (slabs, hub numbers,
+the queue of row pieces, the labels turned for the sweep) is left out where
+there is no room for it, and the results are the same."""
+import contextlib
+import ctypes
+
+import numpy as np
+import pytest
+
+import graphgen
+import paper_2012_11188_gb300 as gs
+from paper_2012_11188_gb300 import scan
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+class Limited:
+    """Allocator hooks over torch's allocator: bytes held, their peak, a limit."""
+
+    def __init__(self):
+        self.held = self.peak = 0
+        self.limit = None
+        self.sizes = {}
+
+    def alloc(self, nbytes, stream, ctx):
+        import torch
+        if self.limit is not None and self.held + nbytes > self.limit:
+            return None
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+        self.held += nbytes
+        self.peak = max(self.peak, self.held)
+        self.sizes[p] = nbytes
+        return p
+
+    def free(self, p, nbytes, stream, ctx):
+        import torch
+        assert self.sizes.pop(p) == nbytes
+        self.held -= nbytes
+        torch.cuda.caching_allocator_delete(p)
+
+    @contextlib.contextmanager
+    def at_most(self, more):
+        """`more` bytes beyond what is held now."""
+        self.limit, self.peak = self.held + more, self.held
+        yield
+        self.limit = None
+
+
+@pytest.fixture()
+def memory():
+    m = Limited()
+    hooks = scan.ALLOC_FN(m.alloc), scan.FREE_FN(m.free)
+    cast = [ctypes.cast(h, ctypes.c_void_p) for h in hooks]
+    assert gs.load().scan_set_allocator(cast[0], cast[1], None) == 0
+    yield m
+    assert gs.load().scan_set_allocator(None, None, None) == 0
+    assert m.held == 0 and not m.sizes
+
+
+def hub_rows():
+    """Rows of several pieces (1024 entries) and many short ones."""
+    edges = [(i, j) for i in range(6) for j in range(i)]
+    edges += [(i, 6 + x) for i in range(6) for x in range(1500 + 700 * i)]
+    edges += [(6 + x, 6 + x + 1) for x in range(0, 6000, 2)]
+    return graphgen.from_edges(6 + 6001, edges)
+
+
+@pytest.mark.parametrize("count", [1, 5])
+def test_queries_without_room_for_the_queue(memory, count):
+    import torch
+    g = hub_rows()
+    with gs.ScanIndex.build(g) as ix:
+        mus, epss = [3, 2, 900, 4, 2500][:count], [0.0, 0.02, 0.01, 0.3, 0.0][:count]
+        want = np.stack([ix.query(m, e, hubs=True) for m, e in zip(mus, epss)])
+        out = torch.full((count, g.n), 77, dtype=torch.int32, device="cuda")
+        # parents, parameters, core counts and a status word
+        with memory.at_most(4 * count * g.n + 4 * count + 8 * count + 8 * (2 * count + 1) + 4):
+            if count == 1:
+                ix.query(mus[0], epss[0], hubs=True, out=out)
+            else:
+                ix.query_batch(mus, epss, hubs=True, out=out)
+    assert np.array_equal(out.cpu().numpy(), want)
+
+
+def test_server_without_room_for_the_queue(memory):
+    import torch
+    g = hub_rows()
+    with gs.ScanIndex.build(g) as ix:
+        want = ix.query(3, 0.0, hubs=True)
+        out = torch.full((g.n,), 77, dtype=torch.int32, device="cuda")
+        # parents of four queries, destinations, parameters, core counts, two
+        # status words
+        with memory.at_most(4 * 4 * g.n + 4 * 8 + 4 * 4 + 4 * 8 + 8 * 9 + 8):
+            with gs.Server(max_batch=4) as srv:
+                srv.wait(srv.submit_query(ix, 3, 0.0, out, hubs=True), timeout_ms=60000)
+    assert np.array_equal(out.cpu().numpy(), want)
