@@ -277,7 +277,8 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   // own skips the rows that its one clustering leaves out
   int32_t* lt = B >= 8 ? pool.get<int32_t>((size_t)SWEEP_BATCH * n) : nullptr;
   unsigned long long* dsum = lt ? pool.get<unsigned long long>((size_t)B * n) : nullptr;
-  const bool together = dsum != nullptr;
+  if (lt && !dsum) pool.put(lt);
+  bool together = dsum != nullptr;
   if (!dsum) dsum = pool.get<unsigned long long>(n);
   if (!lab || !dsum || !acc || !st) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(dsum, 0, (together ? (size_t)B : 1) * n * sizeof(unsigned long long), s));
@@ -287,7 +288,17 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   GS_LAUNCH();
   for (int b0 = 0; b0 < count; b0 += B) {
     const int nb = count - b0 < B ? count - b0 : B;
-    GS_TRY(run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st));
+    int rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st);
+    if (rc == SCAN_ENOMEM && together) {  // the queries need the room themselves
+      pool.put(lt);
+      pool.put(dsum);
+      together = false;
+      dsum = pool.get<unsigned long long>(n);
+      if (!dsum) return SCAN_ENOMEM;
+      GS_CUDA(cudaMemsetAsync(dsum, 0, n * sizeof(unsigned long long), s));
+      rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st);
+    }
+    GS_TRY(rc);
     if (together) {
       k_turn_labels<<<grid_of(n, 32), 256, 0, s>>>(lab, n, nb, lt);
       GS_LAUNCH();

@@ -597,7 +597,13 @@ int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* ep
   double* eps = pool.get<double>(Q);
   int64_t* nc = pool.get<int64_t>((size_t)Q + 1);
   int32_t* parent = pool.get<int32_t>((size_t)Q * (size_t)(n > 0 ? n : 1));
-  if (!mu || !eps || !nc || !parent) return SCAN_ENOMEM;
+  if (!mu || !eps || !nc || !parent) {
+    pool.put(mu);
+    pool.put(eps);
+    pool.put(nc);
+    pool.put(parent);
+    return SCAN_ENOMEM;
+  }
   size_t qb = query_queue_bytes(ix, Q);
   char* queue = qb ? pool.get<char>(qb) : nullptr;
   if (!queue) qb = 0;  // no room: a warp walks a long row alone

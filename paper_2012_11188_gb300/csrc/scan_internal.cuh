@@ -323,7 +323,8 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
                           cudaStream_t s, CountTimer* timer);
 
 // Queries (Algorithms 3-5). status_dev: a zeroed device word that receives
-// DEV_LIMIT if a bounded union-find loop gave up.
+// DEV_LIMIT if a bounded union-find loop gave up. On SCAN_ENOMEM nothing was
+// enqueued and its scratch is back with the pool.
 int run_queries(const IndexData& ix, int q, const int* mu, const double* eps, int32_t* labels_dev,
                 int flags, Pool& pool, cudaStream_t s, unsigned* status_dev);
 

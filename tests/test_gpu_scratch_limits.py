@@ -97,3 +97,27 @@ def test_server_without_room_for_the_queue(memory):
             with gs.Server(max_batch=4) as srv:
                 srv.wait(srv.submit_query(ix, 3, 0.0, out, hubs=True), timeout_ms=60000)
     assert np.array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("count,room", [(40, "one"), (40, "labels"), (40, "queries"), (40, "all"),
+                                        (8, "one"), (8, "queries")])
+def test_sweep_without_room_for_all_clusterings(memory, count, room):
+    """Room for the passes of one clustering at a time, for the turned labels
+    but not the sums of all clusterings, for both but not the queries' own
+    scratch, and for everything."""
+    g = hub_rows()
+    mus = [2 + 3 * (i % 13) for i in range(count)]
+    epss = [(i % 9) / 20.0 for i in range(count)]
+    batch = min(count, 32)
+    need = 4 * batch * g.n  # label rows
+    need += 4 * batch * g.n + 12 * batch + 8 * (2 * batch + 1)  # the queries
+    need += 8 * g.n  # sums of one clustering
+    need += 8 * (4 * count + 1) + 4
+    turned, sums = 4 * 32 * g.n, 8 * batch * g.n
+    more = {"one": 0, "labels": turned, "queries": turned + sums - 4 * batch * g.n + 8 * g.n,
+            "all": turned + sums + 4 * MB}[room]
+    with gs.ScanIndex.build(g) as ix:
+        want = ix.sweep(mus, epss)
+        with memory.at_most(need + more):
+            got = ix.sweep(mus, epss)
+    assert np.array_equal(got, want)
