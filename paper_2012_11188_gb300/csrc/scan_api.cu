@@ -391,17 +391,28 @@ int check_csr_args(const scan_csr* csr) {
   return SCAN_OK;
 }
 
+// Runs f(pool); where there is no room for all it asks for, once more in a
+// lean pool.
+template <class F>
+int with_scratch(cudaStream_t s, F f) {
+  Pool pool(s);
+  const int rc = f(pool);
+  if (rc != SCAN_ENOMEM) return rc;
+  pool.release_all();
+  pool.lean = true;
+  return f(pool);
+}
+
 // Build one index into ix; on error every block is released by the pool.
-int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStream_t s,
-              IndexData* ix, int counts_mode = SCAN_COUNTS_AUTO, const double* weights = nullptr,
-              const CountCfg* cfg_in = nullptr) {
+int build_one_in(Pool& pool, const scan_csr* csr, int kind, const scan_lsh_params* lsh,
+                 IndexData* ix, int counts_mode, const double* weights, const CountCfg* cfg_in) {
+  const cudaStream_t s = pool.s;
   if (counts_mode < SCAN_COUNTS_AUTO || counts_mode > SCAN_COUNTS_DENSE) return SCAN_EINVAL;
   GS_TRY(check_csr_args(csr));
   if (kind != SCAN_COSINE && kind != SCAN_JACCARD) return SCAN_EINVAL;
   GS_TRY(validate_lsh(lsh, kind));
   if (weights && (kind != SCAN_COSINE || counts_mode == SCAN_COUNTS_DENSE)) return SCAN_EINVAL;
   const int64_t n = csr->n, arcs = csr->num_arcs;
-  Pool pool(s);
   Events ev;
   GS_TRY(ev.mark(s));
   ix->n = n;
@@ -461,6 +472,14 @@ int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStr
   ix->bytes = 0;
   for (auto& b : ix->blocks) ix->bytes += b.b;
   return SCAN_OK;
+}
+
+int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStream_t s,
+              IndexData* ix, int counts_mode = SCAN_COUNTS_AUTO, const double* weights = nullptr,
+              const CountCfg* cfg_in = nullptr) {
+  return with_scratch(s, [&](Pool& pool) {
+    return build_one_in(pool, csr, kind, lsh, ix, counts_mode, weights, cfg_in);
+  });
 }
 
 // ---------------------------------------------------------------- batched build
@@ -593,8 +612,9 @@ struct Arena {
 
 // The G graphs packed into one union CSR and built by one pass of the
 // pipeline; the per-graph indexes are views into one shared arena.
-int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* lsh,
-                cudaStream_t s, const CountCfg& cfg, scan_index** out) {
+int build_union_in(Pool& pool, const scan_csr* graphs, int G, int kind, const scan_lsh_params* lsh,
+                   const CountCfg& cfg, scan_index** out) {
+  const cudaStream_t s = pool.s;
   std::vector<int64_t> vb(G + 1, 0), ab(G + 1, 0);
   for (int g = 0; g < G; ++g) {
     GS_TRY(check_csr_args(&graphs[g]));
@@ -603,7 +623,6 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
   }
   const int64_t N = vb[G], A = ab[G];
   if (N > 0x7ffffffe) return SCAN_EINVAL;  // union ids are int32
-  Pool pool(s);
   Events ev;
   GS_TRY(ev.mark(s));
   IndexData u;
@@ -757,6 +776,13 @@ int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
     out[g] = hs[g];
   }
   return SCAN_OK;
+}
+
+int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* lsh,
+                cudaStream_t s, const CountCfg& cfg, scan_index** out) {
+  return with_scratch(s, [&](Pool& pool) {
+    return build_union_in(pool, graphs, G, kind, lsh, cfg, out);
+  });
 }
 
 // Batched build: the members that the counting configuration sends to the
@@ -1219,16 +1245,11 @@ int scan_tuning_load(const char* path) {
   return SCAN_OK;
 }
 
-int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end,
-                             uint32_t* counts, uintptr_t stream) {
-  if (!csr) return SCAN_EINVAL;
-  GS_TRY(gscan::check_csr_args(csr));
+namespace {
+int closed_counts_range_in(gscan::Pool& pool, const scan_csr* csr, int64_t v_begin, int64_t v_end,
+                           uint32_t* counts) {
+  const cudaStream_t s = pool.s;
   const int64_t n = csr->n, arcs = csr->num_arcs;
-  if (v_begin < 0 || v_end < v_begin || v_end > n) return SCAN_EINVAL;
-  if (arcs > 0 && !counts) return SCAN_EINVAL;
-  if (arcs == 0) return SCAN_OK;
-  cudaStream_t s = (cudaStream_t)stream;
-  gscan::Pool pool(s);
   int64_t* off = pool.get<int64_t>(n + 1);
   int32_t* adj = pool.get<int32_t>(arcs);
   int32_t* deg = pool.get<int32_t>(n > 0 ? n : 1);
@@ -1292,6 +1313,19 @@ int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end
   }
   return SCAN_OK;
 }
+}  // namespace
+
+int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end,
+                             uint32_t* counts, uintptr_t stream) {
+  if (!csr) return SCAN_EINVAL;
+  GS_TRY(gscan::check_csr_args(csr));
+  if (v_begin < 0 || v_end < v_begin || v_end > csr->n) return SCAN_EINVAL;
+  if (csr->num_arcs > 0 && !counts) return SCAN_EINVAL;
+  if (csr->num_arcs == 0) return SCAN_OK;
+  return gscan::with_scratch((cudaStream_t)stream, [&](gscan::Pool& pool) {
+    return closed_counts_range_in(pool, csr, v_begin, v_end, counts);
+  });
+}
 
 int scan_sort_segments_desc(double* keys, int32_t* ids, const int64_t* seg_off, int64_t nseg,
                             int64_t total, int64_t max_len, uintptr_t stream) {
@@ -1303,6 +1337,11 @@ int scan_sort_segments_desc(double* keys, int32_t* ids, const int64_t* seg_off, 
     return SCAN_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
   gscan::Pool pool(s);
+  // the sort is in place and cannot be begun again: a slab only where there is
+  // room beside it for the rest (a second pair, bucket ids, samples; the list
+  // of segments)
+  const size_t rest = (max_len > 4096 ? 16 * (size_t)total : 0) + 8 * (size_t)nseg;
+  if (rest > gscan::Pool::TMP_BYTES) pool.lean = !pool.room(rest + gscan::Pool::SLAB);
   GS_TRY(gscan::segmented_sort_desc(reinterpret_cast<uint64_t*>(keys), ids, seg_off, nseg, total,
                                     max_len, pool, s));
   GS_CUDA(cudaStreamSynchronize(s));

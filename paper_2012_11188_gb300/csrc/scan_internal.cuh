@@ -104,8 +104,10 @@ void dev_free(void* p, size_t bytes, cudaStream_t s);
 // with the fewer waits for results below, an SBM graph of 10k vertices
 // 0.70 -> 0.61 ms), larger ones are blocks of their own. put() gives a block back
 // and leaves a slab piece where it is. What detach() hands over is get()'s.
+// lean: no slabs, and nothing else that is there for speed alone (hub numbers).
 struct Pool {
   cudaStream_t s;
+  bool lean = false;
   struct Blk { void* p; size_t b; };
   std::vector<Blk> blocks;
   static constexpr size_t TMP_BYTES = 256u << 10, SLAB = 4u << 20;
@@ -133,7 +135,7 @@ struct Pool {
   template <class T>
   T* tmp(size_t count) {
     const size_t b = (count * sizeof(T) + 255) / 256 * 256;
-    if (b > TMP_BYTES) return get<T>(count);
+    if (lean || b > TMP_BYTES) return get<T>(count);
     if (slab_used + b > SLAB) {
       void* p = dev_alloc(SLAB, s);
       if (!p) return get<T>(count);
@@ -150,6 +152,12 @@ struct Pool {
     for (void* p : slabs) dev_free(p, SLAB, s);
     slabs.clear();
     slab_used = SLAB;
+  }
+  // whether `bytes` are to be had now
+  bool room(size_t bytes) {
+    void* p = dev_alloc(bytes, s);
+    if (p) dev_free(p, bytes, s);
+    return p != nullptr;
   }
   // hand ownership of every block to the caller (the index)
   std::vector<Blk> detach() {

@@ -1610,12 +1610,13 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
     k_fill_i32<<<1024, 256, 0, s>>>(twin, m, -1);
     GS_LAUNCH();
   }
-  // hub numbers, when some vertex may be the CTA kernel's
+  // hub numbers, when some vertex may be the CTA kernel's (a lean build counts
+  // without them, by hash tables alone)
   Hubs hubs;
   uint16_t *num = nullptr, *o16 = nullptr;
   int32_t* hub_list = nullptr;
   HubInfo* hub_info = nullptr;
-  if (n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG &&
+  if (!pool.lean && n > 0 && m > 0 && maxdeg >= HUB_MIN_DEG &&
       (maxdeg > HUB_DEG || !warp_vertex(maxdeg, max_od, cfg.warp_deg))) {
     num = pool.tmp<uint16_t>(n);
     o16 = pool.tmp<uint16_t>(m + 2);

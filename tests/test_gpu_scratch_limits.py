@@ -121,3 +121,83 @@ def test_sweep_without_room_for_all_clusterings(memory, count, room):
         with memory.at_most(need + more):
             got = ix.sweep(mus, epss)
     assert np.array_equal(got, want)
+
+
+def graphs():
+    return {"sbm": graphgen.sbm(10000, 50, 0.05, 0.0004, seed=1),
+            "rmat": graphgen.rmat(13, 16, seed=2),
+            "sparse": graphgen.sbm(60000, 3000, 0.05, 0.00001, seed=3),
+            "tiny": graphgen.sbm(500, 5, 0.1, 0.01, seed=4)}
+
+
+def figure(g):
+    """Device bytes of a build, without what is only there for speed."""
+    return 51 * g.arcs + 36 * g.n + MB
+
+
+def same(a, b):
+    for key in a:
+        assert np.array_equal(a[key], b[key]), key
+
+
+@pytest.mark.parametrize("name", ["sbm", "rmat", "sparse", "tiny"])
+@pytest.mark.parametrize("kind", [gs.COSINE, gs.JACCARD])
+def test_builds_in_little_room(memory, name, kind):
+    g = graphs()[name]
+    with gs.ScanIndex.build(g, kind, counts=gs.COUNTS_SPARSE) as ix:
+        want = ix.export()
+    with memory.at_most(figure(g)):
+        ix = gs.ScanIndex.build(g, kind, counts=gs.COUNTS_SPARSE)
+    got = ix.export()
+    ix.free()
+    same(got, want)
+
+
+def test_batch_and_counts_in_little_room(memory):
+    gl = [graphgen.sbm(3000 + 500 * i, 20, 0.05, 0.001, seed=i) for i in range(6)]
+    n, arcs = sum(g.n for g in gl), sum(g.arcs for g in gl)
+    want = []
+    for ix in gs.ScanIndex.build_batch(gl):
+        want.append(ix.export())
+        ix.free()
+    # a build of the union, and offsets relative to each graph
+    with memory.at_most(51 * arcs + 36 * n + MB + 16 * (n + len(gl))):
+        ixs = gs.ScanIndex.build_batch(gl)
+    for ix, w in zip(ixs, want):
+        same(ix.export(), w)
+        ix.free()
+    g = graphs()["rmat"]
+    counts = gs.closed_counts_range(g, 0, g.n)
+    # the graph and the counts (8 bytes an arc), the counting's own (28)
+    with memory.at_most(36 * g.arcs + 36 * g.n + MB):
+        assert np.array_equal(gs.closed_counts_range(g, 0, g.n), counts)
+
+
+def test_out_of_memory_is_reported(memory):
+    g = graphs()["sbm"]
+    with memory.at_most(28 * g.arcs):
+        for call in (lambda: gs.ScanIndex.build(g), lambda: gs.ScanIndex.build_batch([g, g]),
+                     lambda: gs.closed_counts_range(g, 0, g.n)):
+            with pytest.raises(gs.ScanError) as e:
+                call()
+            assert e.value.status == -2
+
+
+@pytest.mark.parametrize("nseg,length", [(1, 400000), (40000, 10), (60, 9000)])
+def test_sort_in_little_room(memory, nseg, length):
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    keys = torch.randint(0, 5000, (nseg * length,), device="cuda", generator=gen).double()
+    ids = torch.arange(nseg * length, device="cuda", dtype=torch.int32) % length
+    off = torch.arange(nseg + 1, device="cuda", dtype=torch.int64) * length
+    sorted_in = []
+    for less in (0, 3 * MB):  # with the slab of 4 MB, then less than that needs
+        k, v = keys.clone(), ids.clone()
+        with memory.at_most((memory.peak - less) if less else 1 << 40):
+            gs.sort_segments_desc(k, v, off, max_len=length)
+        sorted_in.append((k.cpu().numpy(), v.cpu().numpy()))
+    for a, b in zip(*sorted_in):
+        assert np.array_equal(a, b)
+    order = np.lexsort((ids.cpu().numpy(), -keys.cpu().numpy(),
+                        np.repeat(np.arange(nseg), length)))
+    assert np.array_equal(sorted_in[0][1], ids.cpu().numpy()[order])
