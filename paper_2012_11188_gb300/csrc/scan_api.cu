@@ -158,13 +158,14 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-size_t build_footprint(int64_t n, int64_t arcs) {
+size_t build_footprint(int64_t n, int64_t arcs, bool lean) {
   // index 28 B/arc + 12 B/vertex; build temporaries: oriented lists, counts,
   // twins (16 B/edge), sort scratch (a second key/val pair, bucket ids,
-  // samples and group counts: 15 B/arc), item and scan arrays (~24 B/vertex),
-  // hub numbers (2 B/arc, 2 B/vertex)
-  return (size_t)arcs * 28 + (size_t)n * 12 + (size_t)(arcs / 2) * 16 + (size_t)arcs * 17 +
-         (size_t)n * 26 + (1u << 20);
+  // samples and group counts: 15 B/arc), item and scan arrays (~24 B/vertex)
+  const size_t least = (size_t)arcs * 28 + (size_t)n * 12 + (size_t)(arcs / 2) * 16 +
+                       (size_t)arcs * 15 + (size_t)n * 24 + (1u << 20);
+  // hub numbers (2 B/arc, 2 B/vertex) and the slab of small scratch
+  return lean ? least : least + (size_t)arcs * 2 + (size_t)n * 2 + Pool::SLAB;
 }
 
 namespace {
@@ -394,10 +395,10 @@ int check_csr_args(const scan_csr* csr) {
 // Runs f(pool); where there is no room for all it asks for, once more in a
 // lean pool.
 template <class F>
-int with_scratch(cudaStream_t s, F f) {
-  Pool pool(s);
+int with_scratch(cudaStream_t s, bool lean, F f) {
+  Pool pool(s, lean);
   const int rc = f(pool);
-  if (rc != SCAN_ENOMEM) return rc;
+  if (rc != SCAN_ENOMEM || pool.lean) return rc;
   pool.release_all();
   pool.lean = true;
   return f(pool);
@@ -476,8 +477,8 @@ int build_one_in(Pool& pool, const scan_csr* csr, int kind, const scan_lsh_param
 
 int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStream_t s,
               IndexData* ix, int counts_mode = SCAN_COUNTS_AUTO, const double* weights = nullptr,
-              const CountCfg* cfg_in = nullptr) {
-  return with_scratch(s, [&](Pool& pool) {
+              const CountCfg* cfg_in = nullptr, bool lean = false) {
+  return with_scratch(s, lean, [&](Pool& pool) {
     return build_one_in(pool, csr, kind, lsh, ix, counts_mode, weights, cfg_in);
   });
 }
@@ -780,7 +781,7 @@ int build_union_in(Pool& pool, const scan_csr* graphs, int G, int kind, const sc
 
 int build_union(const scan_csr* graphs, int G, int kind, const scan_lsh_params* lsh,
                 cudaStream_t s, const CountCfg& cfg, scan_index** out) {
-  return with_scratch(s, [&](Pool& pool) {
+  return with_scratch(s, false, [&](Pool& pool) {
     return build_union_in(pool, graphs, G, kind, lsh, cfg, out);
   });
 }
@@ -846,8 +847,8 @@ int build_batch(const scan_csr* graphs, int G, int kind, const scan_lsh_params* 
 }  // namespace
 
 int build_index(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStream_t s,
-                IndexData* ix) {
-  return build_one(csr, kind, lsh, s, ix);
+                IndexData* ix, bool lean) {
+  return build_one(csr, kind, lsh, s, ix, SCAN_COUNTS_AUTO, nullptr, nullptr, lean);
 }
 
 void free_index_data(IndexData* ix) {
@@ -1322,7 +1323,7 @@ int scan_closed_counts_range(const scan_csr* csr, int64_t v_begin, int64_t v_end
   if (v_begin < 0 || v_end < v_begin || v_end > csr->n) return SCAN_EINVAL;
   if (csr->num_arcs > 0 && !counts) return SCAN_EINVAL;
   if (csr->num_arcs == 0) return SCAN_OK;
-  return gscan::with_scratch((cudaStream_t)stream, [&](gscan::Pool& pool) {
+  return gscan::with_scratch((cudaStream_t)stream, false, [&](gscan::Pool& pool) {
     return closed_counts_range_in(pool, csr, v_begin, v_end, counts);
   });
 }

@@ -113,7 +113,7 @@ struct Pool {
   static constexpr size_t TMP_BYTES = 256u << 10, SLAB = 4u << 20;
   std::vector<void*> slabs;
   size_t slab_used = SLAB;
-  explicit Pool(cudaStream_t st) : s(st) {}
+  explicit Pool(cudaStream_t st, bool lean_ = false) : s(st), lean(lean_) {}
   ~Pool() { release_all(); }
   template <class T>
   T* get(size_t count) {
@@ -361,12 +361,13 @@ int run_queries_prealloc(const IndexData& ix, int Q, const int* mu_dev, const do
                          cudaStream_t s, unsigned* status_dev);
 
 // Whole index build into ix (scan_api.cu); on error every block is released.
+// lean: in as little memory as it goes (Pool).
 int build_index(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStream_t s,
-                IndexData* ix);
+                IndexData* ix, bool lean);
 // Release an index's device memory.
 void free_index_data(IndexData* ix);
 // Device footprint estimate of a build (temporaries included), bytes.
-size_t build_footprint(int64_t n, int64_t arcs);
+size_t build_footprint(int64_t n, int64_t arcs, bool lean);
 // Host or device pointer?
 bool is_device_ptr(const void* p);
 

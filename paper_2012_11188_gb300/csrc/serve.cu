@@ -9,7 +9,8 @@
 //    stream completes the batch). At most two batches are in flight; queries
 //    that arrive meanwhile wait in the queue and join the next batch.
 //  - the build worker admits build requests in arrival order when their
-//    footprint fits the memory budget and the device's free memory, and builds
+//    footprint fits the memory budget and the device's free memory (of a lean
+//    build, which is what is built where only that fits), and builds
 //    them on its own stream, overlapping with the query batches.
 // Latencies are measured on the host from submit to completion (the trace
 // replay measures from each query's scheduled arrival instead).
@@ -43,7 +44,7 @@ struct Request {
   int kind = 0;
   bool has_lsh = false;
   scan_lsh_params lsh{};
-  size_t est = 0;
+  size_t est = 0, est_full = 0;  // of a build, lean and not
   // completion
   int status = SCAN_OK;
   bool done = false;
@@ -316,7 +317,9 @@ void build_worker(scan_server* s) {
       if (!h) rc = SCAN_ENOMEM;
     }
     if (rc == SCAN_OK) {
-      rc = gscan::build_index(&r->csr, r->kind, r->has_lsh ? &r->lsh : nullptr, s->bs, &h->d);
+      const bool lean = (s->p.memory_budget_bytes && r->est_full > s->p.memory_budget_bytes) ||
+                        r->est_full > free_device_bytes();
+      rc = gscan::build_index(&r->csr, r->kind, r->has_lsh ? &r->lsh : nullptr, s->bs, &h->d, lean);
       if (rc != SCAN_OK) { delete h; h = nullptr; }
     }
     {
@@ -403,7 +406,8 @@ int scan_serve_submit_build(scan_server* s, const scan_csr* csr, scan_sim_kind k
   r->csr = *csr;
   r->kind = (int)kind;
   if (lsh) { r->has_lsh = true; r->lsh = *lsh; }
-  r->est = gscan::build_footprint(csr->n, csr->num_arcs);
+  r->est = gscan::build_footprint(csr->n, csr->num_arcs, true);
+  r->est_full = gscan::build_footprint(csr->n, csr->num_arcs, false);
   if (s->p.memory_budget_bytes && r->est > s->p.memory_budget_bytes) {
     delete r;
     return SCAN_EBUSY;  // would never fit

@@ -173,6 +173,21 @@ def test_batch_and_counts_in_little_room(memory):
         assert np.array_equal(gs.closed_counts_range(g, 0, g.n), counts)
 
 
+@pytest.mark.parametrize("name", ["sbm", "rmat", "sparse", "tiny"])
+@pytest.mark.parametrize("more", [0, 2 * MB, 8 * MB])
+def test_server_builds_stay_within_their_budget(memory, name, more):
+    g = graphs()[name]
+    with gs.ScanIndex.build(g) as ix:
+        want = ix.export()
+    budget = figure(g) + more
+    with gs.Server(memory_budget=budget) as srv:
+        memory.peak = memory.held
+        ix = srv.wait(srv.submit_build(g, gs.COSINE), timeout_ms=60000)
+        assert memory.peak - memory.held + ix.device_bytes <= budget
+    same(ix.export(), want)
+    ix.free()
+
+
 def test_out_of_memory_is_reported(memory):
     g = graphs()["sbm"]
     with memory.at_most(28 * g.arcs):
