@@ -311,7 +311,7 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
     if (row) pool.put(row);
     GS_TRY(ev.mark(s));
     GS_TRY(segmented_sort_desc((uint64_t*)ix->no_sim, ix->no_id, ix->off, n, arcs, ix->maxdeg, pool,
-                               s, true));
+                               s, true, scalars));
     GS_TRY(ev.mark(s));
     return SCAN_OK;
   }
@@ -342,8 +342,8 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
     GS_TRY(launch_closed_counts_and_sims(kind, ix->off, ix->adj, ix->deg, n, arcs, od, oadj, opos,
                                          ix->maxdeg, max_od, use_lsh ? lsh->degree_threshold : -1,
                                          wcsr, ix->no_sim, scalars, pool, s, &timer, cfg));
-    // (what the counting finds wrong is read with the build's final status:
-    // the sorts take any bits for keys)
+    // (what the counting finds wrong is read with the sort's segment classes;
+    // the estimates take any graph whose ids are in range)
     pool.put(od);
     pool.put(oadj);
     pool.put(opos);
@@ -356,7 +356,7 @@ int run_pipeline(IndexData* ix, int kind, const scan_lsh_params* lsh, Pool& pool
   GS_TRY(ev.mark(s));
   // ---- neighbour order (Algorithm 2)
   GS_TRY(segmented_sort_desc((uint64_t*)ix->no_sim, ix->no_id, ix->off, n, arcs, ix->maxdeg, pool, s,
-                             true));
+                             true, scalars));
   GS_TRY(ev.mark(s));
   return SCAN_OK;
 }
@@ -378,10 +378,7 @@ void store_timings(Events& ev, const CountTimer& timer) {
 int check_final_status(const unsigned* scalars, cudaStream_t s) {
   unsigned hs = 0;
   GS_TRY(read_back(&hs, scalars, sizeof(hs), s));
-  if (hs & DEV_BADGRAPH) return SCAN_EBADGRAPH;
-  if (hs & DEV_BADWEIGHT) return SCAN_EINVAL;
-  if (hs & DEV_LIMIT) return SCAN_ETIMEOUT;
-  return SCAN_OK;
+  return status_code(hs);
 }
 
 int check_csr_args(const scan_csr* csr) {

@@ -48,6 +48,14 @@ enum : unsigned {
   DEV_BADWEIGHT = 8u,  // a weight negative, not finite, or not symmetric
 };
 
+// what a build answers for a status word
+inline int status_code(unsigned st) {
+  if (st & DEV_BADGRAPH) return SCAN_EBADGRAPH;
+  if (st & DEV_BADWEIGHT) return SCAN_EINVAL;
+  if (st & DEV_LIMIT) return SCAN_ETIMEOUT;
+  return SCAN_OK;
+}
+
 // ------------------------------------------------------------ pinned host words
 // A slot of pinned host memory that the device writes directly (one page for
 // the process, slots handed out and taken back under a lock); p is null when
@@ -306,10 +314,12 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
 // descending, then val ascending. Keys are non-negative doubles viewed as
 // uint64. max_len bounds every segment length. ascending_vals: the vals of
 // every segment ascend (as in an id-sorted CSR row), so that ties may be kept
-// in place.
+// in place. status: a device word read with the segment classes, for which the
+// host waits; where it says that the build has failed, nothing is sorted and
+// its status_code is returned.
 int segmented_sort_desc(uint64_t* key, int32_t* val, const int64_t* seg_off, int64_t nseg,
                         int64_t total, int64_t max_len, Pool& pool, cudaStream_t s,
-                        bool ascending_vals = false);
+                        bool ascending_vals = false, const unsigned* status = nullptr);
 
 // Core order from the neighbour order (Algorithm 2, MakeCoreOrder).
 int build_core_order(IndexData& ix, Pool& pool, cudaStream_t s);

@@ -62,12 +62,14 @@ __device__ __forceinline__ int seg_class(int64_t len) {
 
 // Count segments per class and number of tiles of long segments.
 // counts[]: per class, tiles of the long class, the longest long segment,
-// and a flag for offsets that are not non-decreasing within [0, total]
-constexpr int NCNT = NCLASS + 3;
+// a flag for offsets that are not non-decreasing within [0, total], and the
+// caller's status word
+constexpr int NCNT = NCLASS + 4;
 
-__global__ void k_classify_count(Segs S, int64_t nseg, int64_t total,
+__global__ void k_classify_count(Segs S, int64_t nseg, int64_t total, const unsigned* status,
                                  unsigned long long* counts) {
   __shared__ unsigned long long c[NCLASS + 2];
+  const unsigned said = status && blockIdx.x == 0 && threadIdx.x == 0 ? *status : 0u;
   if (threadIdx.x < NCLASS + 2) c[threadIdx.x] = 0;
   __syncthreads();
   bool bad = false;
@@ -99,6 +101,7 @@ __global__ void k_classify_count(Segs S, int64_t nseg, int64_t total,
   if (threadIdx.x < NCLASS + 1 && c[threadIdx.x]) atomicAdd(&counts[threadIdx.x], c[threadIdx.x]);
   if (threadIdx.x == NCLASS + 1 && c[threadIdx.x]) atomicMax(&counts[threadIdx.x], c[threadIdx.x]);
   if (bad) atomicOr(&counts[NCLASS + 2], 1ull);
+  if (said) counts[NCLASS + 3] = said;
 }
 
 // Fill per-class segment lists (order irrelevant). The lanes of a warp that
@@ -1186,7 +1189,7 @@ unsigned grid_of(int64_t units, int per) {
 // segment ascend.
 int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Segs S, int64_t nseg,
                int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth,
-               bool ascending = false);
+               bool ascending = false, const unsigned* status = nullptr);
 
 // Moves the elements of the nlong long segments (device list llist) into
 // their buckets in the other array pair and sorts the buckets, as segments of
@@ -1279,16 +1282,18 @@ int bucket_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, S
 }
 
 int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Segs S, int64_t nseg,
-               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth, bool ascending) {
+               int64_t total, bool in_alt, Pool& pool, cudaStream_t s, int depth, bool ascending,
+               const unsigned* status) {
   if (nseg <= 0 || total <= 1) return SCAN_OK;
   unsigned long long* counts = pool.tmp<unsigned long long>(2 * NCNT);
   if (!counts) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(counts, 0, 2 * NCNT * sizeof(unsigned long long), s));
   const unsigned g_seg = (unsigned)std::min<int64_t>((nseg + 255) / 256, sm_count() * 16);
-  k_classify_count<<<g_seg, 256, 0, s>>>(S, nseg, total, counts);
+  k_classify_count<<<g_seg, 256, 0, s>>>(S, nseg, total, status, counts);
   GS_LAUNCH();
   unsigned long long hc[NCNT];
   GS_TRY(read_back(hc, counts, sizeof(hc), s));
+  GS_TRY(status_code((unsigned)hc[NCLASS + 3]));
   if (hc[NCLASS + 2]) return SCAN_EINVAL;  // before any element is touched
   int64_t base[NCLASS + 1];
   base[0] = 0;
@@ -1436,10 +1441,10 @@ int sort_level(uint64_t* key, int32_t* val, uint64_t* alt_k, int32_t* alt_v, Seg
 
 int segmented_sort_desc(uint64_t* key, int32_t* val, const int64_t* seg_off, int64_t nseg,
                         int64_t total, int64_t max_len, Pool& pool, cudaStream_t s,
-                        bool ascending_vals) {
+                        bool ascending_vals, const unsigned* status) {
   if (nseg <= 0 || total <= 1 || max_len <= 1) return SCAN_OK;
   return sort_level(key, val, nullptr, nullptr, Segs{seg_off, seg_off + 1}, nseg, total, false, pool,
-                    s, 0, ascending_vals);
+                    s, 0, ascending_vals, status);
 }
 
 }  // namespace gscan
