@@ -10,6 +10,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "graph_walk.cuh"
 #include "scan_internal.cuh"
 
 namespace gscan {
@@ -481,15 +482,6 @@ int build_one(const scan_csr* csr, int kind, const scan_lsh_params* lsh, cudaStr
 }
 
 // ---------------------------------------------------------------- batched build
-__device__ __forceinline__ int64_t last_le(const int64_t* a, int64_t cnt, int64_t x) {
-  int64_t lo = 0, hi = cnt;
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (a[mid] <= x) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 // Where a graph's CSR is on the device while it is packed (one in host memory
 // is first copied to the arena).
 struct PackSrc {
@@ -502,21 +494,11 @@ __device__ __forceinline__ int64_t src_offset(const PackSrc& p, int64_t i) {
   return p.off64 ? static_cast<const int64_t*>(p.off)[i] : static_cast<const int32_t*>(p.off)[i];
 }
 
-// A CTA's chunk of the union's arcs or vertices: the graph of each element is
-// found by walking on from that of the chunk's first (one search per CTA and
-// chunk; a search per element was 1.4 ms of each pass over the 190M arcs of
-// 512 SBM graphs).
+// A CTA takes chunks of PACK_CH of the union's arcs or vertices; every thread
+// searches the graph of the chunk's first element and walks on from there
+// (GraphWalk; a search per element was 1.4 ms of each pass over the 190M arcs
+// of 512 SBM graphs).
 constexpr int PACK_CH = 4096;
-struct GraphWalk {
-  const int64_t* base;  // ascending bases, G + 1 entries
-  int64_t g;
-  __device__ __forceinline__ GraphWalk(const int64_t* a, int G, int64_t first)
-      : base(a), g(last_le(a, G, first)) {}
-  __device__ __forceinline__ int64_t at(int64_t i) {  // i must not descend
-    while (base[g + 1] <= i) ++g;
-    return g;
-  }
-};
 
 // union offsets: off[u] = ab_g + o_g[u - vb_g] for u in graph g; off[N] = A;
 // every graph's first and last offset are checked.
@@ -526,7 +508,7 @@ k_pack_offsets(const PackSrc* __restrict__ src, const int64_t* __restrict__ vb,
                unsigned* status) {
   bool bad = false;
   for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < N; c0 += (int64_t)gridDim.x * PACK_CH) {
-    GraphWalk w(vb, G, c0);
+    GraphWalk<const int64_t*> w(vb, G, c0);
     const int64_t c1 = min(N, c0 + PACK_CH);
     for (int64_t u = c0 + threadIdx.x; u < c1; u += blockDim.x) {
       const int64_t g = w.at(u);
@@ -552,7 +534,7 @@ k_pack_adj(const PackSrc* __restrict__ src, const int64_t* __restrict__ vb,
            const int64_t* __restrict__ ab, int G, int64_t A, int32_t* adj, unsigned* status) {
   bool bad = false;
   for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < A; c0 += (int64_t)gridDim.x * PACK_CH) {
-    GraphWalk w(ab, G, c0);
+    GraphWalk<const int64_t*> w(ab, G, c0);
     const int64_t c1 = min(A, c0 + PACK_CH);
     for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
       const int64_t g = w.at(i);
@@ -570,7 +552,7 @@ __global__ void k_graph_maxdeg(const int32_t* __restrict__ deg, const int64_t* _
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < N;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int32_t d = deg[v];
-    if (d > 0) atomicMax(&md[last_le(vb, G, v)], d);
+    if (d > 0) atomicMax(&md[last_le(vb, 0, G, v)], d);
   }
 }
 
@@ -579,7 +561,7 @@ __global__ void __launch_bounds__(256)
 k_rebase_ids(int32_t* __restrict__ adj, int32_t* __restrict__ no_id,
              const int64_t* __restrict__ vb, const int64_t* __restrict__ ab, int G, int64_t A) {
   for (int64_t c0 = (int64_t)blockIdx.x * PACK_CH; c0 < A; c0 += (int64_t)gridDim.x * PACK_CH) {
-    GraphWalk w(ab, G, c0);
+    GraphWalk<const int64_t*> w(ab, G, c0);
     const int64_t c1 = min(A, c0 + PACK_CH);
     for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
       const int32_t b = (int32_t)vb[w.at(i)];
@@ -596,7 +578,7 @@ __global__ void k_rebase_offsets(const int64_t* __restrict__ src, const int64_t*
                                  int G, int64_t total, int64_t* __restrict__ rel) {
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < total;
        u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t g = last_le(rb, G, u);
+    const int64_t g = last_le(rb, 0, G, u);
     rel[u] = src[base[g] + (u - rb[g])] - ab[g];
   }
 }
