@@ -1185,13 +1185,12 @@ __device__ __forceinline__ void walk_out_arcs(const int64_t* __restrict__ off,
   }
 }
 
-// BY_OFF: the head's degree from its two offsets, one sector, of which the
-// first is gathered anyway: taken where offsets and degrees together outgrow
-// L2 (R-MAT s24 build 152.4 -> 150.7 ms); elsewhere from deg (s20 8.82 ms, 8.84
-// by offsets).
-constexpr int64_t EXPAND_BY_OFF = 8 << 20;  // vertices
-
-template <bool BY_OFF>
+// The head's degree comes from its two offsets, one sector, of which the first
+// is gathered anyway; gathered from deg it is a second one. Pass over R-MAT
+// graphs of n vertices, edge factor 16, by deg and by offsets, ms: n 2^21 1.31
+// and 1.30, 2^22 2.64 and 2.58, 7 2^20 4.84 and 4.58, 12 2^20 9.06 and 8.31, 2^24
+// 12.64 and 11.50; edge factor 6: n 6 2^20 1.66 and 1.62, 2^24 4.82 and 4.47; an SBM
+// graph of 200,000 vertices 0.154 both ways.
 __global__ void __launch_bounds__(EXPAND_T)
 k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ deg,
          const int64_t* __restrict__ odp, const int32_t* __restrict__ oadj,
@@ -1215,7 +1214,7 @@ k_expand(int kind, const int64_t* __restrict__ off, const int32_t* __restrict__ 
       const int64_t j = ra + (k - odp[a]);
       const int32_t b = oadj[j];
       const int64_t rb = off[b];
-      const int32_t da = deg[a], db = BY_OFF ? (int32_t)(off[b + 1] - rb) : deg[b];
+      const int32_t da = deg[a], db = (int32_t)(off[b + 1] - rb);
       // LSH mode: approximated edges are written by the estimate pass
       if (lsh_T >= 0 && da > lsh_T && db > lsh_T) continue;
       int64_t t = tcnt[j];
@@ -1719,9 +1718,8 @@ int launch_closed_counts_and_sims(int kind, const int64_t* off, const int32_t* a
       k_expand_w<<<egrid, EXPAND_T, 0, s>>>(off, adj, odp, oadj, opos, ow, tsum, twin, wcsr, norm,
                                             deg, n, per, lsh_T, sim_csr, status);
     } else {
-      auto expand = n > EXPAND_BY_OFF ? k_expand<true> : k_expand<false>;
-      expand<<<egrid, EXPAND_T, 0, s>>>(kind, off, deg, odp, oadj, opos, tcnt, tc16, twin, n, per,
-                                        lsh_T, sim_csr, status);
+      k_expand<<<egrid, EXPAND_T, 0, s>>>(kind, off, deg, odp, oadj, opos, tcnt, tc16, twin, n, per,
+                                          lsh_T, sim_csr, status);
     }
     GS_LAUNCH();
   }
