@@ -551,9 +551,10 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   unsigned* status = static_cast<unsigned*>(slot.p);
   if (per_sm == 0 || !status) return SCAN_OK;
   *status = 0;
-  // the count of queued pieces, parents, pieces; without pieces where there is
+  // parents, the count of queued pieces, pieces; without pieces where there is
   // no room for them
-  const size_t head = 16 + (((size_t)n * sizeof(int32_t) + 15) & ~(size_t)15);
+  const size_t count_at = ((size_t)n * sizeof(int32_t) + 15) & ~(size_t)15;
+  const size_t head = count_at + 16;
   unsigned cap = queue_capacity(ix, 1);
   char* scratch = cap ? pool.get<char>(head + (size_t)cap * sizeof(QPiece)) : nullptr;
   if (!scratch) {
@@ -561,8 +562,8 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
     scratch = pool.get<char>(head);
   }
   if (!scratch) return SCAN_ENOMEM;
-  unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch);
-  int32_t* parent = reinterpret_cast<int32_t*>(scratch + 16);
+  int32_t* parent = reinterpret_cast<int32_t*>(scratch);
+  unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + count_at);
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
           n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status,
           cap ? reinterpret_cast<QPiece*>(scratch + head) : nullptr, queued, cap};
