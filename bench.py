@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -165,15 +166,18 @@ def measured_bf16_peak():
 
 
 def kernel_source_hash() -> str:
+    """Of the counting kernels' source without its comments and blanks."""
     src = os.path.join(ROOT, "paper_2012_11188_gb300", "csrc", "triangles.cu")
-    return hashlib.sha1(open(src, "rb").read()).hexdigest()[:12]
+    code = re.sub(r"//[^\n]*", "", open(src, encoding="utf-8").read())
+    return hashlib.sha1(" ".join(code.split()).encode()).hexdigest()[:12]
 
 
 def profiled_traffic(touch_bytes: int):
-    """DRAM bytes per launch of the counting step from the committed ncu summary
-    (a smaller R-MAT captured with `ncu --set full`), scaled to this graph by the
-    ratio of algorithmic bytes, or None when the kernel source changed since."""
-    path = os.path.join(ROOT, "profiles", "counting_kernel_rmat.txt")
+    """DRAM bytes of the CTA counting kernels of one build (k_tri_hub and
+    k_triangles) from the committed ncu summary (R-MAT scale 24), scaled to this
+    graph by the ratio of algorithmic bytes, or None when the kernels' code
+    changed since."""
+    path = os.path.join(ROOT, "profiles", "counting_kernels_rmat_s24.txt")
     try:
         kv = {}
         for line in open(path):
@@ -187,9 +191,16 @@ def profiled_traffic(touch_bytes: int):
         return None
 
 
+HUB_MAX, HUB_DEG = 65535, 320  # middle vertices counted by bitmap (csrc/triangles.cu)
+
+
 def algorithmic_bytes(off_t, adj_t):
     """Bytes the paper's oriented merge reads (4 * sum over oriented u->v of
-    d+_u + d+_v = 4 * sum_u d_u d+_u), plus the CSR and output bytes of a build."""
+    d+_u + d+_v = 4 * sum_u d_u d+_u), plus the CSR and output bytes of a build;
+    and the bytes that the counting kernels stream: for every oriented u->v the
+    entries after v of out(u) in rank order, 2 bytes each where v is a hub (whole
+    degree classes of at most HUB_MAX vertices, more than HUB_DEG positions) and 4
+    elsewhere."""
     import torch
     n = off_t.shape[0] - 1
     deg = (off_t[1:] - off_t[:-1])
@@ -197,14 +208,31 @@ def algorithmic_bytes(off_t, adj_t):
     dsrc, ddst = deg[src], deg[adj_t.long()]
     up = (dsrc < ddst) | ((dsrc == ddst) & (src < adj_t.long()))
     dplus = torch.bincount(src[up], minlength=n)
-    del src, dsrc, ddst, up
+    del dsrc, ddst
     touch = 4 * int((deg * dplus).sum().item())
-    hash_probe = 4 * int((dplus * dplus).sum().item())
+    rank = torch.empty(n, dtype=torch.int64, device=off_t.device)
+    order = torch.argsort(deg, stable=True)
+    rank[order] = torch.arange(n, device=off_t.device)
+    key = torch.sort(src[up] * n + rank[adj_t[up].long()])[0]
+    del src, up
+    at = torch.arange(key.shape[0], device=off_t.device)
+    first = torch.cumsum(dplus, 0) - dplus
+    tail = key // n
+    after = dplus[tail] - 1 - (at - first[tail])
+    by_deg = deg[order]
+    cut = HUB_DEG + 1
+    if n > HUB_MAX:  # a class that does not fit as a whole is left out
+        cut = max(cut, int(by_deg[n - HUB_MAX - 1].item()) + 1)
+    hub = by_deg[key % n] >= cut
+    stream = int((after * (4 - 2 * hub.long())).sum().item())
+    hub_elements = int((after * hub.long()).sum().item())
+    elements = int(after.sum().item())
+    del key, at, tail, after, hub
     A = int(adj_t.shape[0])
     csr = 8 * (n + 1) + 4 * A
     out = 60 * A + 4 * n
-    return {"touch": touch, "csr": csr, "out": out, "hash_probe": hash_probe,
-            "max_out_degree": int(dplus.max().item()) if n else 0}
+    return {"touch": touch, "csr": csr, "out": out, "stream": stream, "elements": elements,
+            "hub_elements": hub_elements, "max_out_degree": int(dplus.max().item()) if n else 0}
 
 
 def bench_batched(gs, kind: int, count: int, seed: int, stream):
@@ -860,10 +888,10 @@ def main():
     k_ms = statistics.mean(kernel_ms)
     achieved = alg["touch"] / (cnt_ms / 1000.0) / 1e9
     traffic = profiled_traffic(alg["touch"])
-    # the CTA counting kernel's DRAM traffic (ncu) over its live duration, and
-    # the kernel's own algorithmic bytes (hash probes) over the counting step
+    # the CTA counting kernels' DRAM traffic (ncu) over their live duration, and
+    # the bytes that all counting kernels stream over the counting step
     dram_gbs = traffic / (k_ms / 1000.0) / 1e9 if traffic and k_ms > 0 else None
-    probe_gbs = alg["hash_probe"] / (cnt_ms / 1000.0) / 1e9
+    stream_gbs = alg["stream"] / (cnt_ms / 1000.0) / 1e9
     out = {
         "metric": f"index-build edges/s (R-MAT s{args.scale})",
         "value": value, "unit": "edges/s", "n_gpus": ws, "steps": args.steps,
@@ -883,7 +911,8 @@ def main():
                                 "core_order_ms", "total_ms")},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": "k_triangles (closed counts by oriented triangle enumeration)",
+                     "kernel": "k_tri_hub and k_triangles (closed counts by oriented triangle "
+                               "enumeration)",
                      "algorithmic_bytes_per_launch": alg["touch"],
                      "achieved_note": "B_touch (the bytes of the paper's oriented merge) over "
                                       "the whole counting step: a speed relative to a merge "
@@ -892,11 +921,13 @@ def main():
                      "cta_kernel_ms": k_ms,
                      "dram_gbs": dram_gbs,
                      "dram_frac": dram_gbs / peak if dram_gbs else None,
-                     "dram_note": "ncu DRAM bytes of one CTA counting-kernel launch over its "
-                                  "live CUDA-event duration",
-                     "hash_probe_bytes_per_launch": alg["hash_probe"],
-                     "hash_probe_gbs": probe_gbs,
-                     "hash_probe_frac": probe_gbs / peak,
+                     "dram_note": "ncu DRAM bytes of one launch of each CTA counting kernel over "
+                                  "their live CUDA-event duration",
+                     "stream_bytes_per_launch": alg["stream"],
+                     "stream_elements": alg["elements"],
+                     "stream_elements_by_bitmap": alg["hub_elements"],
+                     "stream_gbs": stream_gbs,
+                     "stream_frac": stream_gbs / peak,
                      "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)"},
         "build_roofline": build_roofline(alg, statistics.mean(step_ms), peak),
         "query": qres,

@@ -636,9 +636,10 @@ k_triangles(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
 //    so twice as many middle vertices walk the same in-neighbours' lists and
 //    counters at a time, which are read from L2 instead of HBM.
 // The position of w in out(v) follows from its word's prefix count.
-// R-MAT s24: CTA kernels 88.5 -> 62.6 ms (46 here, bound by instruction issue,
-// 17 in the hash-table kernel for the middle vertices below the hubs), DRAM
-// traffic 465 -> 260 GB; s20: 2.3 -> 1.4 ms.
+// R-MAT s24, 242M edges: CTA kernels 88.5 -> 62.6 ms (46 here, bound by
+// instruction issue, 17 in the hash-table kernel for the middle vertices below
+// the hubs); s20: 2.3 -> 1.4 ms. DRAM traffic of the two at 260M edges 465 -> 306
+// GB in 70 ms (239 GB here).
 constexpr int HUB_MAX = 65535;          // numbers 0..65534; 0xffff: not a hub
 constexpr int HUB_MIN_DEG = 64;         // no hubs below this degree
 constexpr int HUB_T = 256;
