@@ -270,82 +270,115 @@ __device__ __forceinline__ void phase_core_labels(const QArgs& a, int64_t total,
 }
 
 constexpr int32_t CLAIMED = -3;
-constexpr int OWN_SCAN = 8;  // entries of its own prefix a border's lane looks at alone
+constexpr int OWN_STEP = 4;    // entries of its own prefix a border's lane looks at per step
+constexpr int OWN_LEAST = 8;   // entries looked at before the warp may take over
+constexpr int OWN_MOST = 64;   // and at which it takes over in any case
+constexpr int OWN_LANES = 4;   // borders left over of which the warp takes over before
 
-// Every non-core x in entries [b, e) of NO[u] is a border. The lane that
+// 32 neighbours of core c, x in the lane's (-1: none, or a core). The lane that
 // claims x first looks for the first core in x's own eps-prefix of NO (most
 // similar, smallest id on ties; sigma is symmetric, so that prefix holds at
-// least u): OWN_SCAN entries by itself, all loads in flight, the rest of a
-// longer prefix by the whole warp, 128 entries at a time.
-__device__ __forceinline__ void border_range(const QArgs& a, const Item& c, int64_t b, int64_t e) {
+// least the core that found it). The lanes go through their prefixes side by
+// side, OWN_STEP entries in flight each; once few are left, or the prefixes are
+// long, the whole warp takes one border after another, 128 entries at a time.
+// (One at a time from the ninth entry on was slower than a lane alone where
+// many borders look a little further: (20, 0.1) on R-MAT s22 1.09 -> 1.74 ms.)
+__device__ __forceinline__ void border_chunk(const QArgs& a, const Item& c, int32_t x) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   int32_t* parent = c.parent;
-  const int32_t* ids = a.no_id + a.off[c.u];
-  for (int64_t j0 = b; j0 < e; j0 += 32) {
-    const int64_t j = j0 + lane;
-    const int32_t x = j < e ? ids[j] : -1;
-    bool mine = x >= 0 && ld_volatile(parent + x) < 0 &&
-                atomicCAS(c.lab + x, -1, CLAIMED) == -1;
-    int64_t xb = 0;
-    int32_t xd = 0;
+  bool mine = x >= 0 && atomicCAS(c.lab + x, -1, CLAIMED) == -1;
+  unsigned todo = __ballot_sync(FULL, mine);
+  if (!todo) return;
+  int64_t xb = 0;
+  int32_t xd = 0;
+  if (mine) {
+    xb = a.off[x];
+    xd = a.deg[x];
+  }
+  int t0 = 0;  // entries looked at
+  do {
     if (mine) {
-      xb = a.off[x];
-      xd = a.deg[x];
-      double sv[OWN_SCAN];
-      int32_t y[OWN_SCAN], py[OWN_SCAN];
+      double sv[OWN_STEP];
+      int32_t y[OWN_STEP], py[OWN_STEP];
 #pragma unroll
-      for (int t = 0; t < OWN_SCAN; ++t) {
-        sv[t] = t < xd ? a.no_sim[xb + t] : -1.0;
-        y[t] = t < xd ? a.no_id[xb + t] : x;
+      for (int t = 0; t < OWN_STEP; ++t) {
+        const bool in = t0 + t < xd;
+        sv[t] = in ? a.no_sim[xb + t0 + t] : -1.0;
+        y[t] = in ? a.no_id[xb + t0 + t] : x;
       }
 #pragma unroll
-      for (int t = 0; t < OWN_SCAN; ++t) py[t] = ld_volatile(parent + y[t]);
-      bool over = false;
+      for (int t = 0; t < OWN_STEP; ++t) py[t] = ld_volatile(parent + y[t]);
+      int32_t first = -1;
+      bool over = false;  // the end of the prefix
 #pragma unroll
-      for (int t = 0; t < OWN_SCAN; ++t) {
-        if (over || !mine) continue;
-        if (!(sv[t] >= c.eps)) {  // end of the prefix
-          over = true;
-        } else if (py[t] >= 0) {
-          c.lab[x] = uf_find(parent, y[t]);
-          mine = false;
-        }
+      for (int t = 0; t < OWN_STEP; ++t) {
+        over |= first < 0 && !(sv[t] >= c.eps);
+        if (first < 0 && !over && py[t] >= 0) first = y[t];
       }
-      if (mine && (over || xd <= OWN_SCAN)) {  // no core (cannot be with symmetric similarities)
-        c.lab[x] = -1;
+      // (over without a core cannot be with symmetric similarities)
+      if (first >= 0 || over) {
+        c.lab[x] = first >= 0 ? uf_find(parent, first) : -1;
         mine = false;
       }
     }
-    unsigned todo = __ballot_sync(FULL, mine);
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const int64_t rb = __shfl_sync(FULL, xb, src);
-      const int32_t rd = __shfl_sync(FULL, xd, src);
-      const int32_t xs = __shfl_sync(FULL, x, src);
-      int32_t first = -1;
-      bool end = false;
-      for (int32_t t0 = OWN_SCAN; t0 < rd && first < 0 && !end; t0 += 128) {
-        double sv[4];
-        int32_t y[4], py[4];
+    t0 += OWN_STEP;
+    todo = __ballot_sync(FULL, mine);
+    if (!todo) return;
+  } while (t0 < OWN_LEAST || (t0 < OWN_MOST && __popc(todo) > OWN_LANES));
+  do {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const int64_t rb = __shfl_sync(FULL, xb, src);
+    const int32_t rd = __shfl_sync(FULL, xd, src);
+    const int32_t xs = __shfl_sync(FULL, x, src);
+    int32_t first = -1;
+    bool end = false;
+    for (int32_t t1 = t0; t1 < rd && first < 0 && !end; t1 += 128) {
+      double sv[4];
+      int32_t y[4], py[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int32_t t = t0 + 32 * k + lane;
-          sv[k] = t < rd ? a.no_sim[rb + t] : -1.0;
-          y[k] = t < rd ? a.no_id[rb + t] : xs;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) py[k] = ld_volatile(parent + y[k]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const bool in = sv[k] >= c.eps;
-          const unsigned m = __ballot_sync(FULL, in && py[k] >= 0);
-          if (first < 0 && m) first = __shfl_sync(FULL, y[k], __ffs(m) - 1);
-          end |= !__all_sync(FULL, in);
-        }
+      for (int k = 0; k < 4; ++k) {
+        const int32_t t = t1 + 32 * k + lane;
+        sv[k] = t < rd ? a.no_sim[rb + t] : -1.0;
+        y[k] = t < rd ? a.no_id[rb + t] : xs;
       }
-      if (lane == 0) c.lab[xs] = first >= 0 ? uf_find(parent, first) : -1;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) py[k] = ld_volatile(parent + y[k]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const bool in = sv[k] >= c.eps;
+        const unsigned m = __ballot_sync(FULL, in && py[k] >= 0);
+        if (first < 0 && m) first = __shfl_sync(FULL, y[k], __ffs(m) - 1);
+        end |= !__all_sync(FULL, in);
+      }
+    }
+    if (lane == 0) c.lab[xs] = first >= 0 ? uf_find(parent, first) : -1;
+  } while (todo);
+}
+
+// Every non-core in entries [b, e) of NO[u] is a border. Most entries are cores:
+// 128 at a time are tested, and what is left goes on by chunks of 32.
+__device__ __forceinline__ void border_range(const QArgs& a, const Item& c, uint32_t b, uint32_t e) {
+  constexpr int W = 4;
+  const int lane = threadIdx.x & 31;
+  const int32_t* ids = a.no_id + a.off[c.u];
+  for (uint32_t j0 = b; j0 < e; j0 += 32 * W) {
+    int32_t x[W];
+    unsigned some = 0;  // bit k: a non-core in chunk k
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+      const uint32_t j = j0 + 32 * k + lane;
+      x[k] = j < e ? ids[j] : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < W; ++k)
+      if (x[k] >= 0 && ld_volatile(c.parent + x[k]) < 0) some |= 1u << k;
+    unsigned any = __reduce_or_sync(0xffffffffu, some);
+    while (any) {
+      const int k = __ffs(any) - 1;
+      any &= any - 1;
+      border_chunk(a, c, some >> k & 1u ? ids[j0 + 32 * k + lane] : -1);
     }
   }
 }
@@ -361,7 +394,7 @@ __device__ __forceinline__ void phase_borders(const QArgs& a, int64_t total, int
     const Item x = item_at<ONE>(a, it, mu, eps);
     int64_t pu = prefix_ge(a.no_sim + a.off[x.u], a.deg[x.u], x.eps);
     if (a.queue && queued) pu = min(pu, (int64_t)PIECE);
-    border_range(a, x, 0, pu);
+    border_range(a, x, 0, (uint32_t)pu);
   }
   if (a.queue && queued)
     for (int64_t i = w0; i < asked; i += nw) {
@@ -410,7 +443,11 @@ __global__ void k_union(QArgs a) {
 __global__ void k_union_queue(QArgs a) {
   phase_union_queue(a, grid_thread() >> 5, grid_threads() >> 5);
 }
-__global__ void k_labels(QArgs a) {  // borders do not read core labels, only parents
+// Borders do not read core labels, only parents. Six CTAs a multiprocessor: the
+// walks wait for dependent loads, and the registers spilled for it are those of
+// the few borders (72 registers and three CTAs before: a ring of 1M vertices, five
+// queries, 3.19 ms, now 2.76).
+__global__ void __launch_bounds__(256, 6) k_labels(QArgs a) {
   const int64_t total = a.ncp[a.Q];
   phase_core_labels<false>(a, total, 0, 0.0, grid_thread(), grid_threads());
   phase_borders<false>(a, total, 0, 0.0, grid_thread() >> 5, grid_threads() >> 5);
@@ -434,7 +471,7 @@ __device__ __forceinline__ void fill_minus1(int32_t* p, int64_t n, int64_t t0, i
 // (mu, eps) as arguments, the status in a word that the host reads directly.
 // Every CTA searches the core count for itself (it is one cached path).
 constexpr int ONE_T = 256;
-__global__ void __launch_bounds__(ONE_T)
+__global__ void __launch_bounds__(ONE_T, 4)
 k_query_one(QArgs a, int mu, double eps, int hubs) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   __shared__ int64_t s_nc;
