@@ -453,6 +453,7 @@ __global__ void __launch_bounds__(256, 6) k_labels(QArgs a) {
   phase_borders<false>(a, total, 0, 0.0, grid_thread() >> 5, grid_threads() >> 5);
 }
 __global__ void k_hubs(QArgs a) {
+  if (a.ncp[blockIdx.y + 1] == a.ncp[blockIdx.y]) return;  // no clusters, no hubs
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   phase_hubs(a, labels_of(a, blockIdx.y), w0, ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
@@ -469,10 +470,15 @@ __device__ __forceinline__ void fill_minus1(int32_t* p, int64_t n, int64_t t0, i
 
 // One query as one cooperative launch: the same phases between grid barriers,
 // (mu, eps) as arguments, the status in a word that the host reads directly.
-// Every CTA searches the core count for itself (it is one cached path).
+// Every CTA searches the core count for itself (it is one cached path). A query
+// of more than `most` cores is left to the batch's launches, and hubs of a large
+// graph to k_hubs: one kernel for all phases has the registers of the largest, so
+// half as many warps walk the rows (ring of 1M vertices, each a core: 1.95 ms
+// here, 1.07 as a batch of one).
 constexpr int ONE_T = 256;
+constexpr unsigned ONE_HEAVY = 1u << 31;  // in the status word: nothing was labelled
 __global__ void __launch_bounds__(ONE_T, 4)
-k_query_one(QArgs a, int mu, double eps, int hubs) {
+k_query_one(QArgs a, int mu, double eps, int hubs, int64_t most) {
   cooperative_groups::grid_group grid = cooperative_groups::this_grid();
   __shared__ int64_t s_nc;
   const int64_t t0 = grid_thread(), nt = grid_threads();
@@ -484,8 +490,13 @@ k_query_one(QArgs a, int mu, double eps, int hubs) {
     if (threadIdx.x == 0) s_nc = c;
   }
   __syncthreads();
-  const int64_t nc = s_nc;
-  if (nc == 0 && !hubs) return;  // the same in every CTA
+  const int64_t nc = s_nc;  // the same in every CTA
+  if (t0 == 0) {
+    a.ncp[0] = 0;
+    a.ncp[1] = nc > most ? 0 : nc;
+    if (nc > most) *a.status = ONE_HEAVY;
+  }
+  if (nc == 0 || nc > most) return;
   grid.sync();
   phase_mark<true>(a, nc, mu, eps, t0, nt);
   grid.sync();
@@ -521,6 +532,22 @@ int query_one_per_sm() {
   return c - 1;
 }
 
+// Where a single query leaves the cooperative launch: where it is expected to
+// take ONE_LOSS us longer than the launches of a batch, which cost 45 us more,
+// and 20 us for the attempt. Measured, always one launch, always a batch, and by
+// this rule, us: ring of 1M vertices 1900, 1067, 1090, of 300k 555, 367, 385, of
+// 100k 230, 213, 228; 100 cliques of 600 547, 456, 490; SBM of 100k vertices (2, 0)
+// 500, 690, 500.
+constexpr double ONE_LOSS = 150.0;
+constexpr int64_t ONE_HUBS = 8;         // vertices per resident warp: hubs in a launch of their own
+                                        // beyond (R-MAT s22 (3, 0.3) 1686 -> 1092 us)
+constexpr int64_t ONE_COPY = 1 << 16;   // labels
+
+dim3 hubs_grid(int64_t n, int Q) {
+  return dim3((unsigned)std::max<int64_t>(
+                  1, std::min<int64_t>((n + 7) / 8, sm_count() * 16 / std::min(Q, 16) + 1)), Q);
+}
+
 unsigned queue_capacity(const IndexData& ix, int Q) {
   // pieces past the first of a row: none when no row is longer than one
   if (ix.maxdeg <= PIECE) return 0;
@@ -545,7 +572,6 @@ int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* 
           reinterpret_cast<unsigned long long*>(queue), cap};
   if (cap) GS_CUDA(cudaMemsetAsync(queue, 0, 16, s));
   const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, sm_count() * 8 / std::min(Q, 8) + 1));
-  const unsigned gw = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, sm_count() * 16 / std::min(Q, 16) + 1));
   if (lab_ptrs) {
     k_init_labels<<<dim3(gx, Q), 256, 0, s>>>(a);
     GS_LAUNCH();
@@ -568,7 +594,7 @@ int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* 
   k_labels<<<sm_count() * 16, 256, 0, s>>>(a);
   GS_LAUNCH();
   if (flags & SCAN_Q_HUBS) {
-    k_hubs<<<dim3(gw, Q), 256, 0, s>>>(a);
+    k_hubs<<<hubs_grid(n, Q), 256, 0, s>>>(a);
     GS_LAUNCH();
   }
   return SCAN_OK;
@@ -588,10 +614,10 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   unsigned* status = static_cast<unsigned*>(slot.p);
   if (per_sm == 0 || !status) return SCAN_OK;
   *status = 0;
-  // parents, the count of queued pieces, pieces; without pieces where there is
-  // no room for them
-  const size_t count_at = ((size_t)n * sizeof(int32_t) + 15) & ~(size_t)15;
-  const size_t head = count_at + 16;
+  // parents, the counts of queued pieces and of cores, pieces; without pieces
+  // where there is no room for them
+  const size_t count_at = ((size_t)n * sizeof(int32_t) + 7) & ~(size_t)7;
+  const size_t head = count_at + 3 * sizeof(int64_t);
   unsigned cap = queue_capacity(ix, 1);
   char* scratch = cap ? pool.get<char>(head + (size_t)cap * sizeof(QPiece)) : nullptr;
   if (!scratch) {
@@ -601,14 +627,22 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   if (!scratch) return SCAN_ENOMEM;
   int32_t* parent = reinterpret_cast<int32_t*>(scratch);
   unsigned long long* queued = reinterpret_cast<unsigned long long*>(scratch + count_at);
+  int64_t* nc = reinterpret_cast<int64_t*>(scratch + count_at) + 1;
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
-          n, ix.maxdeg, nullptr, nullptr, nullptr, 1, parent, labels, nullptr, status,
+          n, ix.maxdeg, nullptr, nullptr, nc, 1, parent, labels, nullptr, status,
           cap ? reinterpret_cast<QPiece*>(scratch + head) : nullptr, queued, cap};
   // a warp per core at most, and no more CTAs than are resident at once
   const int64_t want = std::max<int64_t>(1, (n + ONE_T / 32 - 1) / (ONE_T / 32));
-  const unsigned g = (unsigned)std::min<int64_t>(want, (int64_t)sm_count() * per_sm);
-  int hubs = flags & SCAN_Q_HUBS;
-  void* args[] = {&a, &mu, &eps, &hubs};
+  const int64_t resident = (int64_t)sm_count() * per_sm;
+  const unsigned g = (unsigned)std::min<int64_t>(want, resident);
+  const int64_t warps = resident * (ONE_T / 32);
+  // the most cores: an item costs a warp here about 2.5 us and 1.5 us per 32
+  // entries of its row more than in the batch's launches
+  const double steps = (double)ix.arcs / (double)n / 32.0;
+  int64_t most = (int64_t)(ONE_LOSS * (double)warps / (2.5 + 1.5 * steps));
+  const bool hubs = flags & SCAN_Q_HUBS, hubs_after = hubs && n > ONE_HUBS * warps;
+  int hubs_in = hubs && !hubs_after;
+  void* args[] = {&a, &mu, &eps, &hubs_in, &most};
   // refused where the stream or the process has fewer multiprocessors than
   // the device: the launches of a batch answer then
   if (cudaLaunchCooperativeKernel((const void*)k_query_one, dim3(g), dim3(ONE_T), args, 0, s) !=
@@ -617,13 +651,30 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
     pool.put(scratch);
     return SCAN_OK;
   }
-  *done = true;
   GS_LAUNCH();
-  if (host_labels)
-    GS_CUDA(cudaMemcpyAsync(host_labels, labels, (size_t)n * sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, s));
+  if (hubs_after) {
+    k_hubs<<<hubs_grid(n, 1), 256, 0, s>>>(a);
+    GS_LAUNCH();
+  }
+  // labels for the host follow at once where they are few
+  const bool copy_now = host_labels && n <= ONE_COPY;
+  auto copy = [&] {
+    return cudaMemcpyAsync(host_labels, labels, (size_t)n * sizeof(int32_t),
+                           cudaMemcpyDeviceToHost, s);
+  };
+  if (copy_now) GS_CUDA(copy());
   GS_CUDA(cudaStreamSynchronize(s));
-  if (*(volatile unsigned*)status & DEV_LIMIT) return SCAN_ETIMEOUT;
+  const unsigned st = *(volatile unsigned*)status;
+  if (st & ONE_HEAVY) {
+    pool.put(scratch);
+    return SCAN_OK;
+  }
+  *done = true;
+  if (host_labels && !copy_now) {
+    GS_CUDA(copy());
+    GS_CUDA(cudaStreamSynchronize(s));
+  }
+  if (st & DEV_LIMIT) return SCAN_ETIMEOUT;
   return SCAN_OK;
 }
 
