@@ -18,15 +18,24 @@ namespace {
 
 // Per clustering: acc[0] = I, acc[1] = sum of d^2 over clustered vertices,
 // acc[2] = S_c, acc[3] != 0 if a label was not a vertex id. dsum[c] (zero on
-// entry and on exit) accumulates D_c at the cluster's label c.
+// entry and on exit) accumulates D_c at the cluster's label c. Clustering
+// blockIdx.y of several: rows of n labels and sums, four words of acc each;
+// nothing is done where cores (null: none given) are `most` or more, and what
+// lies inside a row of more than `longest` is left to k_mod_long.
 __global__ void k_mod_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                            const int32_t* __restrict__ labels, int64_t n,
                            unsigned long long* __restrict__ dsum,
-                           unsigned long long* __restrict__ acc) {
+                           unsigned long long* __restrict__ acc, const int64_t* cores,
+                           int64_t most, int64_t longest) {
+  if (cores && *cores >= most) return;
+  labels += (int64_t)blockIdx.y * n;
+  dsum += (int64_t)blockIdx.y * n;
+  acc += 4 * blockIdx.y;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  unsigned long long inside = 0, dsq = 0;
+  unsigned long long inside = 0, dsq = 0, run = 0;  // run: of vertices with run_label
+  int32_t run_label = -1;
   bool bad = false;
   for (int64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32) {
     // 32 vertices per step: one label load per lane, then the clustered rows
@@ -41,21 +50,60 @@ __global__ void k_mod_rows(const int64_t* __restrict__ off, const int32_t* __res
       const int32_t lv = __shfl_sync(0xffffffffu, ll, src);
       const int64_t b = off[v], e = off[v + 1];
       unsigned cnt = 0;
-      for (int64_t i = b + lane; i < e; i += 32) cnt += labels[adj[i]] == lv ? 1u : 0u;
+      if (e - b <= longest)
+        for (int64_t i = b + lane; i < e; i += 32) cnt += labels[adj[i]] == lv ? 1u : 0u;
       cnt = __reduce_add_sync(0xffffffffu, cnt);
       if (lane == 0) {
         const unsigned long long d = (unsigned long long)(e - b);
         inside += cnt;
         dsq += d * d;
-        if (d) atomicAdd(&dsum[lv], d);
+        if (lv != run_label) {
+          if (run) atomicAdd(&dsum[run_label], run);
+          run_label = lv;
+          run = 0;
+        }
+        run += d;
       }
     }
   }
   if (lane == 0) {
+    if (run) atomicAdd(&dsum[run_label], run);
     if (inside) atomicAdd(&acc[0], inside);
     if (dsq) atomicAdd(&acc[1], dsq);
   }
   if (bad) atomicOr(&acc[3], 1ull);
+}
+
+// The arcs inside the rows of more than MOD_LONG entries (CO[MOD_LONG + 2] lists
+// them) of clustering blockIdx.y: a CTA per row, all CTAs on a row of more than
+// MOD_HUGE. (One warp on a star's row of 4M entries: 1.5 ms for each clustering.)
+constexpr int MOD_LONG = 2048, MOD_HUGE = 65536;
+
+__global__ void __launch_bounds__(256)
+k_mod_long(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+           const int32_t* __restrict__ labels, int64_t n, const int64_t* __restrict__ co_off,
+           const int32_t* __restrict__ co_id, int32_t maxdeg,
+           unsigned long long* __restrict__ acc, const int64_t* cores, int64_t most) {
+  if (*cores >= most) return;
+  labels += (int64_t)blockIdx.y * n;
+  unsigned long long inside = 0;
+  auto walk = [&](int64_t from, int64_t to, int64_t step, int32_t lv) {
+    for (int64_t i = from; i < to; i += step) inside += labels[adj[i]] == lv ? 1u : 0u;
+  };
+  for (int64_t r = co_off[MOD_LONG] + blockIdx.x; r < co_off[MOD_LONG + 1]; r += gridDim.x) {
+    const int32_t v = co_id[r], lv = labels[v];
+    const int64_t b = off[v], e = off[v + 1];
+    if (lv >= 0 && e - b <= MOD_HUGE) walk(b + threadIdx.x, e, blockDim.x, lv);
+  }
+  if (maxdeg > MOD_HUGE)
+    for (int64_t r = co_off[MOD_HUGE]; r < co_off[MOD_HUGE + 1]; ++r) {
+      const int32_t v = co_id[r], lv = labels[v];
+      if (lv >= 0)
+        walk(off[v] + (int64_t)blockIdx.x * blockDim.x + threadIdx.x, off[v + 1],
+             (int64_t)gridDim.x * blockDim.x, lv);
+    }
+  for (int o = 16; o; o >>= 1) inside += __shfl_xor_sync(0xffffffffu, inside, o);
+  if ((threadIdx.x & 31) == 0 && inside) atomicAdd(&acc[4 * blockIdx.y], inside);
 }
 
 // S_c = sum over the cluster labels c of D_c^2; dsum is cleared for the next
@@ -87,8 +135,10 @@ constexpr int SWEEP_BATCH = 32;
 
 // lab[q][v] (nq rows) -> lt[v][32], -1 for the queries past nq
 __global__ void __launch_bounds__(256)
-k_turn_labels(const int32_t* __restrict__ lab, int64_t n, int nq, int32_t* __restrict__ lt) {
+k_turn_labels(const int32_t* __restrict__ lab, int64_t n, int nq, int32_t* __restrict__ lt,
+              const int64_t* cores, int64_t least) {
   __shared__ int32_t tile[32][33];
+  if (cores && *cores < least) return;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int64_t v0 = (int64_t)blockIdx.x * 32; v0 < n; v0 += (int64_t)gridDim.x * 32) {
     for (int q = ty; q < 32; q += 8)
@@ -110,8 +160,10 @@ constexpr int MOD_PIECE = 512;
 __global__ void __launch_bounds__(256)
 k_mod_rows_all(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                const int32_t* __restrict__ lt, int64_t n, int64_t arcs, int nq,
-               unsigned long long* __restrict__ dsum, unsigned long long* __restrict__ acc) {
+               unsigned long long* __restrict__ dsum, unsigned long long* __restrict__ acc,
+               const int64_t* cores, int64_t least) {
   constexpr unsigned FULL = 0xffffffffu;
+  if (cores && *cores < least) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -184,6 +236,15 @@ __global__ void k_mod_clusters_all(int64_t n, unsigned long long* __restrict__ d
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(&acc[4 * blockIdx.y + 2], s);
 }
 
+// Cores of a batch, in units of n * n / arcs, from which its labels are turned (16
+// pairs, turned and one by one, ms: grid of 4M vertices without clusters 1.17 and
+// 0.61; R-MAT s22 at .5 units 1.49 and .49, R-MAT s20 at 2.8 0.77 and 0.73, edge factor
+// 2 at 3.4 4.6 and 6.9; tree of 3M vertices at 4 7.4 and 13.7).
+constexpr double MOD_TOGETHER = 2.0;
+// vertices from which the choice is made: turning the labels of fewer costs less
+// than the launches that choose (SBM of 10k vertices, 16 pairs, 125 us and 140)
+constexpr int64_t MOD_CHOOSE = 1 << 17;
+
 // sum of d^2 over all vertices
 __global__ void k_deg_sq(const int32_t* __restrict__ deg, int64_t n,
                          unsigned long long* __restrict__ out) {
@@ -218,7 +279,8 @@ double modularity_of(const unsigned long long* acc, unsigned long long deg_sq_al
 int launch_modularity(const IndexData& ix, const int32_t* labels_dev, unsigned long long* dsum,
                       unsigned long long* acc, cudaStream_t s) {
   if (ix.n == 0) return SCAN_OK;
-  k_mod_rows<<<grid_of(ix.n, 256), 256, 0, s>>>(ix.off, ix.adj, labels_dev, ix.n, dsum, acc);
+  k_mod_rows<<<grid_of(ix.n, 256), 256, 0, s>>>(ix.off, ix.adj, labels_dev, ix.n, dsum, acc, nullptr,
+                                                0, INT64_MAX);
   GS_LAUNCH();
   k_mod_clusters<<<grid_of(ix.n, 256 * 8), 256, 0, s>>>(ix.n, dsum, acc);
   GS_LAUNCH();
@@ -269,7 +331,8 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   const int B = count < SWEEP_BATCH ? count : SWEEP_BATCH;
   int32_t* lab = pool.get<int32_t>((size_t)B * n);
   unsigned long long* acc = pool.get<unsigned long long>(4 * (size_t)count + 1);
-  unsigned* st = pool.get<unsigned>(1);
+  unsigned* st = pool.get<unsigned>(4);  // status, -, the cores of a batch (2 words)
+  int64_t* cores = n >= MOD_CHOOSE ? reinterpret_cast<int64_t*>(st + 2) : nullptr;
   // all clusterings of a batch at once: 12 more bytes per vertex and query;
   // one at a time where there is no room for them, and for a few pairs: a
   // gather of turned labels is 128 bytes per arc whatever their number, one
@@ -283,12 +346,17 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   if (!lab || !dsum || !acc || !st) return SCAN_ENOMEM;
   GS_CUDA(cudaMemsetAsync(dsum, 0, (together ? (size_t)B : 1) * n * sizeof(unsigned long long), s));
   GS_CUDA(cudaMemsetAsync(acc, 0, (4 * (size_t)count + 1) * sizeof(unsigned long long), s));
-  GS_CUDA(cudaMemsetAsync(st, 0, sizeof(unsigned), s));
+  GS_CUDA(cudaMemsetAsync(st, 0, 4 * sizeof(unsigned), s));
+  // Turned labels pay where many arcs have a clustered end: they cost 256 bytes a
+  // vertex and 132 per arc of rows with a label, whatever the number of
+  // clusterings; single labels 36 bytes per arc of a clustered row. The cores of
+  // the batch, at the average degree, stand for the clustered rows.
+  const int64_t least = (int64_t)(MOD_TOGETHER * (double)n * (double)n / (double)ix.arcs) + 1;
   k_deg_sq<<<grid_of(n, 256 * 8), 256, 0, s>>>(ix.deg, n, acc + 4 * (size_t)count);
   GS_LAUNCH();
   for (int b0 = 0; b0 < count; b0 += B) {
     const int nb = count - b0 < B ? count - b0 : B;
-    int rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st);
+    int rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st, cores);
     if (rc == SCAN_ENOMEM && together) {  // the queries need the room themselves
       pool.put(lt);
       pool.put(dsum);
@@ -300,11 +368,22 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
     }
     GS_TRY(rc);
     if (together) {
-      k_turn_labels<<<grid_of(n, 32), 256, 0, s>>>(lab, n, nb, lt);
+      k_turn_labels<<<grid_of(n, 32), 256, 0, s>>>(lab, n, nb, lt, cores, least);
       GS_LAUNCH();
       k_mod_rows_all<<<grid_of(ix.arcs, MOD_PIECE * 8), 256, 0, s>>>(
-          ix.off, ix.adj, lt, n, ix.arcs, nb, dsum, acc + 4 * (size_t)b0);
+          ix.off, ix.adj, lt, n, ix.arcs, nb, dsum, acc + 4 * (size_t)b0, cores, least);
       GS_LAUNCH();
+      if (cores) {
+        k_mod_rows<<<dim3(grid_of(n, 256), nb), 256, 0, s>>>(
+            ix.off, ix.adj, lab, n, dsum, acc + 4 * (size_t)b0, cores, least, MOD_LONG);
+        GS_LAUNCH();
+      }
+      if (cores && ix.maxdeg > MOD_LONG) {
+        k_mod_long<<<dim3(std::max(8, sm_count() * 8 / nb), nb), 256, 0, s>>>(
+            ix.off, ix.adj, lab, n, ix.co_off, ix.co_id, ix.maxdeg, acc + 4 * (size_t)b0, cores,
+            least);
+        GS_LAUNCH();
+      }
       k_mod_clusters_all<<<dim3(grid_of(n, 256 * 32), nb), 256, 0, s>>>(n, dsum,
                                                                        acc + 4 * (size_t)b0);
       GS_LAUNCH();

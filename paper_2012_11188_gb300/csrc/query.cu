@@ -679,7 +679,8 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
 }
 
 int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* eps_host,
-                int32_t* labels_dev, int flags, Pool& pool, cudaStream_t s, unsigned* status_dev) {
+                int32_t* labels_dev, int flags, Pool& pool, cudaStream_t s, unsigned* status_dev,
+                int64_t* cores_dev) {
   if (Q <= 0) return SCAN_OK;
   const int64_t n = ix.n;
   int* mu = pool.get<int>(Q);
@@ -701,6 +702,8 @@ int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* ep
   if (n == 0) return SCAN_OK;
   GS_TRY(launch_query_batch(ix, Q, mu, eps, nc, parent, labels_dev, nullptr, flags, s, status_dev,
                             queue, qb));
+  if (cores_dev)
+    GS_CUDA(cudaMemcpyAsync(cores_dev, nc + Q, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
   pool.put(mu);
   pool.put(eps);
   pool.put(nc);

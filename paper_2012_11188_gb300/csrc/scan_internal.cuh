@@ -343,8 +343,10 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
 // Queries (Algorithms 3-5). status_dev: a zeroed device word that receives
 // DEV_LIMIT if a bounded union-find loop gave up. On SCAN_ENOMEM nothing was
 // enqueued and its scratch is back with the pool.
+// cores_dev: null, or a device word that receives the cores of all queries.
 int run_queries(const IndexData& ix, int q, const int* mu, const double* eps, int32_t* labels_dev,
-                int flags, Pool& pool, cudaStream_t s, unsigned* status_dev);
+                int flags, Pool& pool, cudaStream_t s, unsigned* status_dev,
+                int64_t* cores_dev = nullptr);
 
 // One query into device labels (copied to host_labels too unless null) as one
 // cooperative launch; synchronises s. *done = false: such a launch is not to
