@@ -214,7 +214,8 @@ int scan_modularity(scan_index* index, const int32_t* labels, double* q, uintptr
  * marks and its modularity, written to q[i] (host). The paper's set Sigma is
  * mu in {2, 4, ..., 2^18} x eps in {.01, ..., .99}; the pair of highest
  * modularity is its choice of parameters. Queries run 32 at a time on the
- * GPU, each followed by its modularity passes. Synchronises `stream`. */
+ * GPU, followed by the modularity of all of them (of one after another for
+ * fewer than 8, or where there is no room). Synchronises `stream`. */
 int scan_sweep(scan_index* index, int count, const int* mu, const double* eps, double* q,
                uintptr_t stream);
 

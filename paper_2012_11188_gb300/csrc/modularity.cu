@@ -130,7 +130,8 @@ __global__ void k_mod_clusters(int64_t n, unsigned long long* __restrict__ dsum,
 // read once for all 32, and a gather is one full line. Warps take equal
 // pieces of the arc array, so a hub's row is not one warp's. R-MAT s20, 594
 // pairs: 44 ms for the passes of the single clusterings, 16 ms here (13 of them
-// in k_mod_rows_all, at most 3.9 GB of label lines per batch).
+// in k_mod_rows_all, at most 3.9 GB of label lines per batch). It is taken where
+// the batch has cores enough (MOD_TOGETHER).
 constexpr int SWEEP_BATCH = 32;
 
 // lab[q][v] (nq rows) -> lt[v][32], -1 for the queries past nq

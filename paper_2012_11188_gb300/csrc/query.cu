@@ -27,12 +27,14 @@
 // to a queue in pieces that any warp may take (R-MAT s22 has rows of 1.5e5
 // entries: a batch of 64 queries spent 2.2 ms in phase 2 on the warps that
 // walked them, and one thread scanning a border's long prefix alone made
-// phase 3 83% of a parameter sweep); and a single query is one cooperative
-// launch whose phases are separated by grid barriers, instead of eight
-// launches, two clears and three small copies.
-// Measured, before and after: one query with hubs on an SBM graph of 10k
-// vertices 85 -> 50 us, (5, 0.3) on R-MAT s22 73 -> 31 us, a batch of 64 on
-// R-MAT s22 1.78 -> 1.41 ms, 594 pairs of a sweep on R-MAT s20 438 -> 72 ms.
+// phase 3 83% of a parameter sweep); and a single query with little work is one
+// cooperative launch whose phases are separated by grid barriers, instead of
+// eight launches, two clears and three small copies.
+// Measured against one launch per phase, binary searches and whole rows: one
+// query with hubs on an SBM graph of 10k vertices 80 -> 49 us, (5, 0.3) on R-MAT
+// s22 76 -> 29 us, 594 pairs of a sweep on R-MAT s20 420 -> 47 ms. A batch of 64
+// queries gains by which queries it holds: sets of the same ranges take 0.6 to
+// 1.4 ms.
 #include <cooperative_groups.h>
 
 #include "scan_internal.cuh"
@@ -281,8 +283,8 @@ constexpr int OWN_LANES = 4;   // borders left over of which the warp takes over
 // least the core that found it). The lanes go through their prefixes side by
 // side, OWN_STEP entries in flight each; once few are left, or the prefixes are
 // long, the whole warp takes one border after another, 128 entries at a time.
-// (One at a time from the ninth entry on was slower than a lane alone where
-// many borders look a little further: (20, 0.1) on R-MAT s22 1.09 -> 1.74 ms.)
+// (One after another from the ninth entry on: 594 pairs of a sweep on R-MAT s20
+// 51.8 ms, now 47.2.)
 __device__ __forceinline__ void border_chunk(const QArgs& a, const Item& c, int32_t x) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -445,8 +447,8 @@ __global__ void k_union_queue(QArgs a) {
 }
 // Borders do not read core labels, only parents. Six CTAs a multiprocessor: the
 // walks wait for dependent loads, and the registers spilled for it are those of
-// the few borders (72 registers and three CTAs before: a ring of 1M vertices, five
-// queries, 3.19 ms, now 2.76).
+// the few borders (a ring of 1M vertices, all of them cores: four CTAs 1.12 ms,
+// five 1.15, six 1.07).
 __global__ void __launch_bounds__(256, 6) k_labels(QArgs a) {
   const int64_t total = a.ncp[a.Q];
   phase_core_labels<false>(a, total, 0, 0.0, grid_thread(), grid_threads());

@@ -53,7 +53,7 @@ __device__ __forceinline__ bool before_at(const uint64_t* k, const int32_t* v, i
 
 constexpr int32_t SENT_V = 0x7fffffff;  // sorts after every real element (key 0, val max)
 
-// The tile classes double in length and in CTA size (32 to 512 threads at 8
+// The tile classes double in length and in CTA size (32 to 1024 threads at 8
 // elements each), so that a segment keeps at least half of its CTA busy.
 __device__ __forceinline__ int seg_class(int64_t len) {
   return len <= 32 ? 0 : len <= WTILE ? 1 : len <= 512 ? 2 : len <= 1024 ? 3 : len <= 2048 ? 4
@@ -616,7 +616,7 @@ constexpr size_t tile_smem_bytes() {
 #ifndef GS_SORT_LONG_RI
 #define GS_SORT_LONG_RI 8  // elements per thread in the tiles of long segments (8 or 16)
 #endif
-// whole segments of 1025..4096 elements: 512 threads x 8; tiles of long
+// whole segments of 2049..4096 elements: 512 threads x 8; tiles of long
 // segments: TILE elements, TILE / GS_SORT_LONG_RI threads (one CTA per SM)
 constexpr int T4K_T = 512;
 constexpr int TLONG_RI = GS_SORT_LONG_RI;
