@@ -18,19 +18,22 @@ namespace {
 
 // Per clustering: acc[0] = I, acc[1] = sum of d^2 over clustered vertices,
 // acc[2] = S_c, acc[3] != 0 if a label was not a vertex id. dsum[c] (zero on
-// entry and on exit) accumulates D_c at the cluster's label c. Clustering
-// blockIdx.y of several: rows of n labels and sums, four words of acc each;
-// nothing is done where cores (null: none given) are `most` or more, and what
-// lies inside a row of more than `longest` is left to k_mod_long.
+// entry and on exit) accumulates D_c at the cluster's label c. MANY: clustering
+// blockIdx.y of several, rows of n labels and sums, four words of acc each;
+// nothing is done where cores are `most` or more, what lies inside a row of more
+// than `longest` is left to k_mod_long, and runs of one label are one addition.
+template <bool MANY>
 __global__ void k_mod_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                            const int32_t* __restrict__ labels, int64_t n,
                            unsigned long long* __restrict__ dsum,
                            unsigned long long* __restrict__ acc, const int64_t* cores,
                            int64_t most, int64_t longest) {
-  if (cores && *cores >= most) return;
-  labels += (int64_t)blockIdx.y * n;
-  dsum += (int64_t)blockIdx.y * n;
-  acc += 4 * blockIdx.y;
+  if (MANY) {
+    if (*cores >= most) return;
+    labels += (int64_t)blockIdx.y * n;
+    dsum += (int64_t)blockIdx.y * n;
+    acc += 4 * blockIdx.y;
+  }
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -50,24 +53,28 @@ __global__ void k_mod_rows(const int64_t* __restrict__ off, const int32_t* __res
       const int32_t lv = __shfl_sync(0xffffffffu, ll, src);
       const int64_t b = off[v], e = off[v + 1];
       unsigned cnt = 0;
-      if (e - b <= longest)
-        for (int64_t i = b + lane; i < e; i += 32) cnt += labels[adj[i]] == lv ? 1u : 0u;
+      const int64_t to = MANY && e - b > longest ? b : e;
+      for (int64_t i = b + lane; i < to; i += 32) cnt += labels[adj[i]] == lv ? 1u : 0u;
       cnt = __reduce_add_sync(0xffffffffu, cnt);
       if (lane == 0) {
         const unsigned long long d = (unsigned long long)(e - b);
         inside += cnt;
         dsq += d * d;
-        if (lv != run_label) {
-          if (run) atomicAdd(&dsum[run_label], run);
-          run_label = lv;
-          run = 0;
+        if (!MANY) {
+          if (d) atomicAdd(&dsum[lv], d);
+        } else {
+          if (lv != run_label) {
+            if (run) atomicAdd(&dsum[run_label], run);
+            run_label = lv;
+            run = 0;
+          }
+          run += d;
         }
-        run += d;
       }
     }
   }
   if (lane == 0) {
-    if (run) atomicAdd(&dsum[run_label], run);
+    if (MANY && run) atomicAdd(&dsum[run_label], run);
     if (inside) atomicAdd(&acc[0], inside);
     if (dsq) atomicAdd(&acc[1], dsq);
   }
@@ -280,8 +287,8 @@ double modularity_of(const unsigned long long* acc, unsigned long long deg_sq_al
 int launch_modularity(const IndexData& ix, const int32_t* labels_dev, unsigned long long* dsum,
                       unsigned long long* acc, cudaStream_t s) {
   if (ix.n == 0) return SCAN_OK;
-  k_mod_rows<<<grid_of(ix.n, 256), 256, 0, s>>>(ix.off, ix.adj, labels_dev, ix.n, dsum, acc, nullptr,
-                                                0, INT64_MAX);
+  k_mod_rows<false><<<grid_of(ix.n, 256), 256, 0, s>>>(ix.off, ix.adj, labels_dev, ix.n, dsum, acc,
+                                                       nullptr, 0, 0);
   GS_LAUNCH();
   k_mod_clusters<<<grid_of(ix.n, 256 * 8), 256, 0, s>>>(ix.n, dsum, acc);
   GS_LAUNCH();
@@ -375,7 +382,7 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
           ix.off, ix.adj, lt, n, ix.arcs, nb, dsum, acc + 4 * (size_t)b0, cores, least);
       GS_LAUNCH();
       if (cores) {
-        k_mod_rows<<<dim3(grid_of(n, 256), nb), 256, 0, s>>>(
+        k_mod_rows<true><<<dim3(grid_of(n, 256), nb), 256, 0, s>>>(
             ix.off, ix.adj, lab, n, dsum, acc + 4 * (size_t)b0, cores, least, MOD_LONG);
         GS_LAUNCH();
       }
