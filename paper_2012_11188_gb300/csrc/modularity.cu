@@ -20,16 +20,16 @@ namespace {
 // acc[2] = S_c, acc[3] != 0 if a label was not a vertex id. dsum[c] (zero on
 // entry and on exit) accumulates D_c at the cluster's label c. MANY: clustering
 // blockIdx.y of several, rows of n labels and sums, four words of acc each;
-// nothing is done where cores are `most` or more, what lies inside a row of more
+// nothing is done where reached is `most` or more, what lies inside a row of more
 // than `longest` is left to k_mod_long, and runs of one label are one addition.
 template <bool MANY>
 __global__ void k_mod_rows(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                            const int32_t* __restrict__ labels, int64_t n,
                            unsigned long long* __restrict__ dsum,
-                           unsigned long long* __restrict__ acc, const int64_t* cores,
-                           int64_t most, int64_t longest) {
+                           unsigned long long* __restrict__ acc, const unsigned long long* reached,
+                           unsigned long long most, int64_t longest) {
   if (MANY) {
-    if (*cores >= most) return;
+    if (*reached >= most) return;
     labels += (int64_t)blockIdx.y * n;
     dsum += (int64_t)blockIdx.y * n;
     acc += 4 * blockIdx.y;
@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(256)
 k_mod_long(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
            const int32_t* __restrict__ labels, int64_t n, const int64_t* __restrict__ co_off,
            const int32_t* __restrict__ co_id, int32_t maxdeg,
-           unsigned long long* __restrict__ acc, const int64_t* cores, int64_t most) {
-  if (*cores >= most) return;
+           unsigned long long* __restrict__ acc, const unsigned long long* reached, unsigned long long most) {
+  if (*reached >= most) return;
   labels += (int64_t)blockIdx.y * n;
   unsigned long long inside = 0;
   auto walk = [&](int64_t from, int64_t to, int64_t step, int32_t lv) {
@@ -138,15 +138,16 @@ __global__ void k_mod_clusters(int64_t n, unsigned long long* __restrict__ dsum,
 // pieces of the arc array, so a hub's row is not one warp's. R-MAT s20, 594
 // pairs: 44 ms for the passes of the single clusterings, 16 ms here (13 of them
 // in k_mod_rows_all, at most 3.9 GB of label lines per batch). It is taken where
-// the batch has cores enough (MOD_TOGETHER).
+// the clusters hold arcs enough (MOD_TOGETHER).
 constexpr int SWEEP_BATCH = 32;
 
 // lab[q][v] (nq rows) -> lt[v][32], -1 for the queries past nq
 __global__ void __launch_bounds__(256)
 k_turn_labels(const int32_t* __restrict__ lab, int64_t n, int nq, int32_t* __restrict__ lt,
-              const int64_t* cores, int64_t least) {
+              const unsigned long long* reached,
+              unsigned long long least) {
   __shared__ int32_t tile[32][33];
-  if (cores && *cores < least) return;
+  if (reached && *reached < least) return;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int64_t v0 = (int64_t)blockIdx.x * 32; v0 < n; v0 += (int64_t)gridDim.x * 32) {
     for (int q = ty; q < 32; q += 8)
@@ -169,9 +170,10 @@ __global__ void __launch_bounds__(256)
 k_mod_rows_all(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                const int32_t* __restrict__ lt, int64_t n, int64_t arcs, int nq,
                unsigned long long* __restrict__ dsum, unsigned long long* __restrict__ acc,
-               const int64_t* cores, int64_t least) {
+               const unsigned long long* reached,
+              unsigned long long least) {
   constexpr unsigned FULL = 0xffffffffu;
-  if (cores && *cores < least) return;
+  if (reached && *reached < least) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -244,10 +246,11 @@ __global__ void k_mod_clusters_all(int64_t n, unsigned long long* __restrict__ d
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(&acc[4 * blockIdx.y + 2], s);
 }
 
-// Cores of a batch, in units of n * n / arcs, from which its labels are turned (16
-// pairs, turned and one by one, ms: grid of 4M vertices without clusters 1.17 and
-// 0.61; R-MAT s22 at .5 units 1.49 and .49, R-MAT s20 at 2.8 0.77 and 0.73, edge factor
-// 2 at 3.4 4.6 and 6.9; tree of 3M vertices at 4 7.4 and 13.7).
+// Entries of the cores' prefixes over a batch's clusterings, per vertex, from which
+// its labels are turned (16 pairs, turned and one by one, ms: grid of 4M vertices
+// without clusters 1.17 and 0.61; R-MAT s22, few clusters, 1.49 and .49; 500k borders
+// of 2000 cores 0.67 and 1.12; tree of 3M vertices, half of it clustered, 7.4 and
+// 13.7).
 constexpr double MOD_TOGETHER = 2.0;
 // vertices from which the choice is made: turning the labels of fewer costs less
 // than the launches that choose (SBM of 10k vertices, 16 pairs, 125 us and 140)
@@ -339,8 +342,9 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   const int B = count < SWEEP_BATCH ? count : SWEEP_BATCH;
   int32_t* lab = pool.get<int32_t>((size_t)B * n);
   unsigned long long* acc = pool.get<unsigned long long>(4 * (size_t)count + 1);
-  unsigned* st = pool.get<unsigned>(4);  // status, -, the cores of a batch (2 words)
-  int64_t* cores = n >= MOD_CHOOSE ? reinterpret_cast<int64_t*>(st + 2) : nullptr;
+  unsigned* st = pool.get<unsigned>(4);  // status, -, entries of a batch's prefixes (2 words)
+  unsigned long long* reached =
+      st && n >= MOD_CHOOSE ? reinterpret_cast<unsigned long long*>(st + 2) : nullptr;
   // all clusterings of a batch at once: 12 more bytes per vertex and query;
   // one at a time where there is no room for them, and for a few pairs: a
   // gather of turned labels is 128 bytes per arc whatever their number, one
@@ -355,16 +359,16 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
   GS_CUDA(cudaMemsetAsync(dsum, 0, (together ? (size_t)B : 1) * n * sizeof(unsigned long long), s));
   GS_CUDA(cudaMemsetAsync(acc, 0, (4 * (size_t)count + 1) * sizeof(unsigned long long), s));
   GS_CUDA(cudaMemsetAsync(st, 0, 4 * sizeof(unsigned), s));
-  // Turned labels pay where many arcs have a clustered end: they cost 256 bytes a
-  // vertex and 132 per arc of rows with a label, whatever the number of
-  // clusterings; single labels 36 bytes per arc of a clustered row. The cores of
-  // the batch, at the average degree, stand for the clustered rows.
-  const int64_t least = (int64_t)(MOD_TOGETHER * (double)n * (double)n / (double)ix.arcs) + 1;
+  // Turned labels cost 256 bytes a vertex and 132 per arc of rows with a label,
+  // whatever the number of clusterings; single labels 36 bytes per arc of a
+  // clustered row.
+  const unsigned long long least = (unsigned long long)(MOD_TOGETHER * (double)n);
   k_deg_sq<<<grid_of(n, 256 * 8), 256, 0, s>>>(ix.deg, n, acc + 4 * (size_t)count);
   GS_LAUNCH();
   for (int b0 = 0; b0 < count; b0 += B) {
     const int nb = count - b0 < B ? count - b0 : B;
-    int rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st, cores);
+    if (reached) GS_CUDA(cudaMemsetAsync(reached, 0, sizeof(*reached), s));
+    int rc = run_queries(ix, nb, mu + b0, eps + b0, lab, 0, pool, s, st, reached);
     if (rc == SCAN_ENOMEM && together) {  // the queries need the room themselves
       pool.put(lt);
       pool.put(dsum);
@@ -376,19 +380,19 @@ int sweep_impl(const IndexData& ix, int count, const int* mu, const double* eps,
     }
     GS_TRY(rc);
     if (together) {
-      k_turn_labels<<<grid_of(n, 32), 256, 0, s>>>(lab, n, nb, lt, cores, least);
+      k_turn_labels<<<grid_of(n, 32), 256, 0, s>>>(lab, n, nb, lt, reached, least);
       GS_LAUNCH();
       k_mod_rows_all<<<grid_of(ix.arcs, MOD_PIECE * 8), 256, 0, s>>>(
-          ix.off, ix.adj, lt, n, ix.arcs, nb, dsum, acc + 4 * (size_t)b0, cores, least);
+          ix.off, ix.adj, lt, n, ix.arcs, nb, dsum, acc + 4 * (size_t)b0, reached, least);
       GS_LAUNCH();
-      if (cores) {
+      if (reached) {
         k_mod_rows<true><<<dim3(grid_of(n, 256), nb), 256, 0, s>>>(
-            ix.off, ix.adj, lab, n, dsum, acc + 4 * (size_t)b0, cores, least, MOD_LONG);
+            ix.off, ix.adj, lab, n, dsum, acc + 4 * (size_t)b0, reached, least, MOD_LONG);
         GS_LAUNCH();
       }
-      if (cores && ix.maxdeg > MOD_LONG) {
+      if (reached && ix.maxdeg > MOD_LONG) {
         k_mod_long<<<dim3(std::max(8, sm_count() * 8 / nb), nb), 256, 0, s>>>(
-            ix.off, ix.adj, lab, n, ix.co_off, ix.co_id, ix.maxdeg, acc + 4 * (size_t)b0, cores,
+            ix.off, ix.adj, lab, n, ix.co_off, ix.co_id, ix.maxdeg, acc + 4 * (size_t)b0, reached,
             least);
         GS_LAUNCH();
       }

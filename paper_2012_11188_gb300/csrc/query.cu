@@ -32,7 +32,7 @@
 // eight launches, two clears and three small copies.
 // Measured against one launch per phase, binary searches and whole rows: one
 // query with hubs on an SBM graph of 10k vertices 80 -> 49 us, (5, 0.3) on R-MAT
-// s22 76 -> 29 us, 594 pairs of a sweep on R-MAT s20 420 -> 47 ms. A batch of 64
+// s22 76 -> 29 us, 594 pairs of a sweep on R-MAT s20 420 -> 48 ms. A batch of 64
 // queries gains by which queries it holds: sets of the same ranges take 0.6 to
 // 1.4 ms.
 #include <cooperative_groups.h>
@@ -125,6 +125,7 @@ struct QArgs {
   QPiece* queue;       // null: every warp walks its whole prefixes
   unsigned long long* queued;  // pieces asked for; more than queue_cap: the queue was full
   unsigned queue_cap;
+  unsigned long long* reached;  // null, or receives the entries of all cores' prefixes
 };
 
 __device__ __forceinline__ int32_t* labels_of(const QArgs& a, int q) {
@@ -236,9 +237,11 @@ __device__ __forceinline__ void phase_union(const QArgs& a, int64_t total, int m
                                             int64_t w0, int64_t nw) {
   const int lane = threadIdx.x & 31;
   bool fail = false;
+  unsigned reached = 0;  // (rows of more than 2^16 entries count as that many)
   for (int64_t it = w0; it < total; it += nw) {
     const Item x = item_at<ONE>(a, it, mu, eps);
     int64_t pu = prefix_ge(a.no_sim + a.off[x.u], a.deg[x.u], x.eps);
+    if (!ONE) reached += (unsigned)min(pu, (int64_t)1 << 16);
     if (pu > PIECE && a.queue) {
       const unsigned np = (unsigned)((pu - 1) / PIECE);  // pieces past the first
       unsigned long long at = 0;
@@ -254,6 +257,7 @@ __device__ __forceinline__ void phase_union(const QArgs& a, int64_t total, int m
     }
     fail |= !union_range(a, x.parent, x.u, 0, pu);
   }
+  if (!ONE && a.reached && reached && lane == 0) atomicAdd(a.reached, (unsigned long long)reached);
   if (__any_sync(0xffffffffu, fail) && lane == 0) atomicOr(a.status, (unsigned)DEV_LIMIT);
 }
 
@@ -446,7 +450,7 @@ __device__ __forceinline__ int64_t grid_threads() { return (int64_t)gridDim.x * 
 __global__ void k_mark_cores(QArgs a) {
   phase_mark<false>(a, a.ncp[a.Q], 0, 0.0, grid_thread(), grid_threads());
 }
-__global__ void k_union(QArgs a) {
+__global__ void __launch_bounds__(256, 8) k_union(QArgs a) {
   phase_union<false>(a, a.ncp[a.Q], 0, 0.0, grid_thread() >> 5, grid_threads() >> 5);
 }
 __global__ void k_union_queue(QArgs a) {
@@ -569,7 +573,8 @@ unsigned queue_capacity(const IndexData& ix, int Q) {
 // Launch sequence of a batch of Q queries; every pointer is device memory.
 int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* eps, int64_t* nc,
                        int32_t* parent, int32_t* labels, int32_t* const* lab_ptrs, int flags,
-                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes) {
+                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes,
+                       unsigned long long* reached) {
   const int64_t n = ix.n;
   GS_CUDA(cudaMemsetAsync(parent, 0xff, sizeof(int32_t) * (size_t)Q * n, s));
   // queue: a 16-byte head with the count, then the pieces
@@ -578,7 +583,7 @@ int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* 
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
           n, ix.maxdeg, mu, eps, nc, Q, parent, labels, lab_ptrs, status_dev,
           cap ? reinterpret_cast<QPiece*>((char*)queue + 16) : nullptr,
-          reinterpret_cast<unsigned long long*>(queue), cap};
+          reinterpret_cast<unsigned long long*>(queue), cap, reached};
   if (cap) GS_CUDA(cudaMemsetAsync(queue, 0, 16, s));
   const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, sm_count() * 8 / std::min(Q, 8) + 1));
   if (lab_ptrs) {
@@ -639,7 +644,7 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
   int64_t* nc = reinterpret_cast<int64_t*>(scratch + count_at) + 1;
   QArgs a{ix.off, ix.deg, ix.adj, ix.no_id, ix.no_sim, ix.co_off, ix.co_id, ix.co_thr,
           n, ix.maxdeg, nullptr, nullptr, nc, 1, parent, labels, nullptr, status,
-          cap ? reinterpret_cast<QPiece*>(scratch + head) : nullptr, queued, cap};
+          cap ? reinterpret_cast<QPiece*>(scratch + head) : nullptr, queued, cap, nullptr};
   // a warp per core at most, and no more CTAs than are resident at once
   const int64_t want = std::max<int64_t>(1, (n + ONE_T / 32 - 1) / (ONE_T / 32));
   const int64_t resident = (int64_t)sm_count() * per_sm;
@@ -689,7 +694,7 @@ int run_query_one(const IndexData& ix, int mu, double eps, int32_t* labels, int3
 
 int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* eps_host,
                 int32_t* labels_dev, int flags, Pool& pool, cudaStream_t s, unsigned* status_dev,
-                int64_t* cores_dev) {
+                unsigned long long* reached_dev) {
   if (Q <= 0) return SCAN_OK;
   const int64_t n = ix.n;
   int* mu = pool.get<int>(Q);
@@ -710,9 +715,7 @@ int run_queries(const IndexData& ix, int Q, const int* mu_host, const double* ep
   GS_CUDA(cudaMemcpyAsync(eps, eps_host, sizeof(double) * Q, cudaMemcpyHostToDevice, s));
   if (n == 0) return SCAN_OK;
   GS_TRY(launch_query_batch(ix, Q, mu, eps, nc, parent, labels_dev, nullptr, flags, s, status_dev,
-                            queue, qb));
-  if (cores_dev)
-    GS_CUDA(cudaMemcpyAsync(cores_dev, nc + Q, sizeof(int64_t), cudaMemcpyDeviceToDevice, s));
+                            queue, qb, reached_dev));
   pool.put(mu);
   pool.put(eps);
   pool.put(nc);

@@ -343,10 +343,11 @@ int dense_counts_and_sims(int kind, const int64_t* off, const int32_t* adj, cons
 // Queries (Algorithms 3-5). status_dev: a zeroed device word that receives
 // DEV_LIMIT if a bounded union-find loop gave up. On SCAN_ENOMEM nothing was
 // enqueued and its scratch is back with the pool.
-// cores_dev: null, or a device word that receives the cores of all queries.
+// reached_dev: null, or a device word to which the entries of all cores'
+// eps-prefixes are added, about the arcs inside the clusters.
 int run_queries(const IndexData& ix, int q, const int* mu, const double* eps, int32_t* labels_dev,
                 int flags, Pool& pool, cudaStream_t s, unsigned* status_dev,
-                int64_t* cores_dev = nullptr);
+                unsigned long long* reached_dev = nullptr);
 
 // One query into device labels (copied to host_labels too unless null) as one
 // cooperative launch; synchronises s. *done = false: such a launch is not to
@@ -364,7 +365,8 @@ constexpr size_t QUERY_QUEUE_MAX_BYTES = 16 + (size_t)QUERY_QUEUE_MAX * 16;
 size_t query_queue_bytes(const IndexData& ix, int Q);
 int launch_query_batch(const IndexData& ix, int Q, const int* mu, const double* eps, int64_t* nc,
                        int32_t* parent, int32_t* labels, int32_t* const* lab_ptrs, int flags,
-                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes);
+                       cudaStream_t s, unsigned* status_dev, void* queue, size_t queue_bytes,
+                       unsigned long long* reached = nullptr);
 
 // run_queries with caller-supplied device scratch: mu_dev/eps_dev hold Q
 // entries, nc_dev Q+1, parent Q*n; nothing is allocated.

@@ -1,6 +1,6 @@
 """Sweeps of eight pairs and more on either side of their routes: from 131,072
-vertices on, labels turned where the batch has many cores and single passes where
-it has few, rows at the lengths from which a CTA (2048) and all CTAs (65,536) take them. Every sum is a
+vertices on, labels turned where the cores reach many neighbours and single passes
+where they reach few, rows at the lengths from which a CTA (2048) and all CTAs (65,536) take them. Every sum is a
 whole number, so the modularity is the same double as that of each clustering
 by itself (scan_modularity)."""
 import numpy as np
